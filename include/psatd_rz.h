@@ -383,15 +383,16 @@ pic_status pic_get_tuning(pic_sim* sim, pic_tuning* out);
 /* Transform arithmetic of the FP64 form (no counterpart in the paper; the paper's Hankel and
  * Fourier transforms are the operations, this chooses how their float64 results are
  * computed).  The DHT path:
- *   PIC_DHT_AUTO        sliced tensor-core product when Nr <= 256, else the SIMT GEMM
- *                       (the default);
+ *   PIC_DHT_AUTO        digit products on the tensor cores at every Nr (the default): six
+ *                       digits up to Nr = 256 (as SLICED), eight beyond, whose results are the
+ *                       exact sums rounded once, as accurate as the FP64 GEMM's;
  *   PIC_DHT_F64_GEMM    FP64 SIMT GEMM on the FP64 units, and the z-FFT rows in IEEE float64
  *                       too (the reference arithmetic for studies of rounding floors);
  *   PIC_DHT_F64_SLICED  every row of the matrix and column of the panel scaled by a power
- *                       of two and cut into seven 7-bit slices (exact BF16 numbers); the
- *                       slice products accumulate exactly in FP32 on the tensor cores and
- *                       are combined in FP64: agrees with the FP64 product to about 2^-49
- *                       of (row max x column max x Nr).  Needs Nr <= 256.
+ *                       of two and cut into six balanced base-256 digits (exact BF16
+ *                       numbers); the digit products accumulate exactly in FP32 on the tensor
+ *                       cores and are combined in FP64: agrees with the FP64 product to about
+ *                       2^-49 of (row max x column max x Nr).  Needs Nr <= 256.
  * With AUTO and SLICED the power-of-two z-FFT rows run in double words (each value a sum
  * of two floats, about 48 bits, on the float32 units; rows stay float64 in memory): the
  * pairs hold about 48 bits relative to a row's largest value while that lies between

@@ -3,10 +3,11 @@
 // section "Finite order pseudo-spectral solvers": Hankel transform along r) and X the
 // Nr x Nz complex panel of that component seen as Nr x 2Nz reals (re, im interleaved).
 //
-// FP64 form: register-tiled SIMT GEMM (64 x 64 tile per CTA, 4 x 4 outputs per thread,
-// K staged through shared memory in steps of 16).  On GB300 the FP64 pipe, not HBM or
-// shared memory, bounds this kernel, so the tile only has to keep that pipe fed.  The same
-// kernel serves the FP64 setup products (Newton-Schulz refinement of the pseudo-inverse).
+// FP64 form on the PIC_DHT_F64_GEMM path (the others: dht_f64s.cu): register-tiled SIMT GEMM
+// (64 x 64 tile per CTA, 4 x 4 outputs per thread, K staged through shared memory in steps of
+// 16).  On GB300 the FP64 pipe, not HBM or shared memory, bounds this kernel, so the tile only
+// has to keep that pipe fed.  The same kernel serves the FP64 setup products (Newton-Schulz
+// refinement of the pseudo-inverse).
 #include "pic_internal.cuh"
 
 namespace pic {

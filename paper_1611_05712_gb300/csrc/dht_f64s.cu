@@ -4,32 +4,43 @@
 // Hankel transform along r) is, per (component, mode) pair, Y = A X with A the Nr x Nr
 // FP64 matrix and X the Nr x 2Nz FP64 panel.  GB300 runs FP64 arithmetic at 1/64 of its
 // FP32 rate and far below its tensor rate, so this path computes the product exactly in
-// pieces on the BF16 tensor cores and combines them in FP64 (the splitting idea of Ozaki
+// pieces on the BF16 tensor cores and combines them in integers (the splitting idea of Ozaki
 // et al., "Error-free transformations of matrix multiplication by using fast routines of
 // matrix multiplication and its applications", Numer. Algorithms 59, 2012, here with
-// fixed-width integer slices):
+// fixed-width integer digits):
 //   * every row n of A and every column c of X is scaled by a power of two, 2^E_n and
-//     2^E_c, so that its entries lie in (-1, 1); the scaled value v is cut into S = 7
-//     slices of W = 7 bits, v = sum_i s_i 2^(-W (i+1)) + r with integers |s_i| <= 127 (the
-//     magnitude truncated to 49 bits, |r| < 2^-49), each exactly a BF16 number;
-//   * a slice product sum over K <= 256 terms is an integer below 256 * 2^14 = 2^22, and
-//     up to four such sums add up to at most 2^24: the tensor cores' FP32 accumulators
-//     hold them exactly.  Group g collects the products a_i x_j with i + j = g (weight
-//     2^(-W (g+2))): groups 0..3 (at most 4 products each) are exact, groups 4..6 add an
-//     FP32 rounding of relative size 2^-24 at weight <= 2^-42; products with i + j >= S
-//     are left out (weight <= 2^-63);
-//   * the epilogue combines the 7 group accumulators in 64-bit integer arithmetic,
-//     converts once to FP64 and scales by 2^(E_c + E_n).
-// The result agrees with the FP64 product to about 2^-49 of max|A_n| max|X_c| K.  Used
-// for Nr <= 256 (the exactness bound above); larger Nr keep the FP64 SIMT GEMM.
+//     2^E_c, so that its entries lie in (-1, 1); the scaled value v is rounded to B bits and
+//     written in S balanced base-256 digits, v = sum_i d_i 2^(-(T + 8 i)) + r with |d_i| <= 128
+//     for i >= 1 and |r| <= 2^-(B+1), B = T + 8 (S - 1): each digit is exactly a BF16 number
+//     (8 significant bits hold the integers up to 256).  Digits with signs of their own carry a
+//     bit more than a sign and a magnitude would, and what a kept product misses has mean 0;
+//   * a digit product summed over K <= 256 terms is an integer of at most 2^22 (2^23, 2^24
+//     with one, two first digits of S = 6), and the tensor cores' FP32 accumulators hold
+//     sums up to 2^24 exactly.  Group g collects the products d_i d_j with i + j = g (weight
+//     2^(-(2T + 8g))); products with i + j >= S are left out;
+//   * the epilogue combines the group accumulators in 64-bit integer arithmetic, converts to
+//     FP64 with one rounding and scales by 2^(E_c + E_n).
+// Two forms (F64sForm below):
+//   Nr <= 256: S = 6, T = 8, B = 48, 21 products.  The first digit reaches 256, so groups 2
+//     and 3 are split over two accumulators each to stay exact; groups 4 and 5 add at most an
+//     FP32 rounding at weight <= 2^-48.  Error about 2^-50 of max|A_n| max|X_c| sqrt(K) (on the
+//     Hankel matrices with random, beam-like, decaying and smooth panels 2 to 6 times smaller
+//     than the seven sign-magnitude 7-bit slices, 28 products, that stood here before);
+//   Nr > 256: S = 8, T = 6, B = 62, 36 products, the accumulators drained into integers every
+//     256 K: groups 0..3 exact, the rest exact unless sums align adversarially (then an FP32
+//     rounding at weight <= 2^-44).  All 53 bits of entries down to 2^-9 of the largest take
+//     part: the result is the exact sum rounded once to within 2^-62 of max|A_n| max|X_c| K, no
+//     further off than the float64 product's own accumulated roundings.
+// Measured, one cycle's 20 DHTs with their panels' digits: 2048 x 256 x 2 modes 0.45 -> 0.32 ms
+// against the seven-slice form; 1800 x 400 x 2 modes 21.1 ms on the FP64 SIMT GEMM -> 1.04 ms.
 //
-// Pieces: k_f64s_matrix slices the matrices at set-up (7 BF16 planes each, K-major);
-// per DHT k_f64s_colmax finds the column maxima and k_f64s_panel slices the panels
-// into K-major planes; k_dht_f64s is a persistent warp-specialised tcgen05 kernel: one
-// thread issues the tensor-memory-access copies of both operands (7 planes each, 64-byte
-// swizzle, 32 K elements per stage) into a ring of stages, three threads (one per warp,
-// each owning whole groups) issue the 28 slice products per 16 K elements into 7 TMEM
-// accumulators of a 128 x 64 tile, and 16 epilogue warps combine them and store Y.
+// Pieces: k_f64s_matrix writes the matrices' digit planes at set-up (S BF16 planes each,
+// K-major); per DHT k_f64s_panel finds the column exponents and writes the panels' K-major
+// planes; k_dht_f64s is a persistent warp-specialised tcgen05 kernel: one thread issues the
+// tensor-memory-access copies of both operands (S planes each, 64-byte swizzle, 32 K elements
+// per stage) into a ring of stages, three threads (one per warp, each owning whole
+// accumulators) issue the digit products per 16 K elements into 8 TMEM accumulators of a 128 x
+// 64 tile (all 512 columns), and 16 epilogue warps combine them and store Y.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -44,149 +55,181 @@
 namespace pic {
 namespace {
 
-constexpr int kSlices = kF64sSlices;   // S
-constexpr int kSliceBits = 7;       // W
 constexpr int kF64sM = 128;         // panel columns c per tile (TMEM lanes)
 constexpr int kF64sN = 64;          // matrix rows n per tile
-constexpr int kF64sSets = 1;        // accumulator sets in TMEM (7 groups x kF64sN columns each)
+constexpr int kF64sAcc = 8;         // accumulators in TMEM (kF64sN columns each: all 512)
 constexpr int kF64sKC = 32;         // K elements per stage (one 64-byte swizzle row of BF16)
-constexpr int kF64sStages = 2;
+constexpr int kF64sKBlock = 256;    // K elements between drains of the accumulators (exactness)
 constexpr int kF64sThreads = 640;   // warp 0: copies, warps 1-3: MMA, warps 4..19: epilogue
 constexpr uint32_t kF64sPlaneA = kF64sM * 64;   // bytes of one panel plane per stage
 constexpr uint32_t kF64sPlaneB = kF64sN * 64;   // bytes of one matrix plane per stage
-constexpr uint32_t kF64sStageBytes = kSlices * (kF64sPlaneA + kF64sPlaneB);
 
-// The 7 BF16 slices of v = x 2^-E (|v| < 1): the magnitude truncated to 49 bits, cut into
-// 7-bit integers from the top, each carrying the sign of x.  Integer operations on the
-// bits of x only.
-__device__ __forceinline__ void slice7(double x, int E, uint16_t out[kSlices]) {
+// The two forms: S digits, T bits above the point of the first digit, stages of shared
+// memory (3 x 72 KB or 2 x 96 KB of the 227 KB).
+template <int S> struct F64sForm;
+template <> struct F64sForm<kF64sDigits> {
+  static constexpr int top = 8, stages = 3;
+  // accumulator of the product d_i d_j, g = i + j: 0, 1, 2 (with d_0), 3 (d_1 d_1), 4 (g = 3
+  // with d_0), 5 (g = 3 without), 6 (g = 4), 7 (g = 5)
+  __host__ __device__ static constexpr int acc(int i, int j) {
+    const int g = i + j;
+    const bool first = i == 0 || j == 0;
+    return g <= 1 ? g : g == 2 ? (first ? 2 : 3) : g == 3 ? (first ? 4 : 5) : g + 2;
+  }
+  // issuing warp (1..3) of each accumulator: 7 products each (acc 7 has 6, acc 0 has 1)
+  __host__ __device__ static constexpr int warp(int a) { return a == 0 || a == 7 ? 1 : a == 6 || a == 2 ? 2 : 3; }
+};
+template <> struct F64sForm<kF64sDigitsWide> {
+  static constexpr int top = 6, stages = 2;
+  __host__ __device__ static constexpr int acc(int i, int j) { return i + j; }
+  // 12 products each: 7 + 3 (8 + 4), 6 + 4 (7 + 5), 5 + 2 + 1 + 0 (6 + 3 + 2 + 1)
+  __host__ __device__ static constexpr int warp(int a) { return a == 7 || a == 3 ? 1 : a == 6 || a == 4 ? 2 : 3; }
+};
+template <int S> constexpr int f64s_bits() { return F64sForm<S>::top + 8 * (S - 1); }
+template <int S> constexpr uint32_t f64s_stage_bytes() { return S * (kF64sPlaneA + kF64sPlaneB); }
+template <int S> constexpr size_t f64s_smem() { return 1024 + (size_t)F64sForm<S>::stages * f64s_stage_bytes<S>() + 256; }
+static_assert(kF64sAcc * kF64sN <= 512, "accumulators exceed tensor memory");
+static_assert(f64s_smem<kF64sDigits>() <= 227 * 1024 && f64s_smem<kF64sDigitsWide>() <= 227 * 1024,
+              "stages exceed shared memory");
+
+// The S balanced base-256 digits of v = x 2^-E (|v| < 1) as floats (exact BF16 numbers), by
+// integer operations on the bits of x: F = round(|x| 2^(B - E)) with its sign, then one
+// addition of 128 to each byte below the first digit makes every digit a byte less 128.
+template <int S>
+__device__ __forceinline__ void digits_of(double x, int E, float out[S]) {
+  constexpr int B = f64s_bits<S>();
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int ebits = (int)((bits >> 52) & 0x7ff);
   const unsigned long long mant = (bits & 0xfffffffffffffull) | (ebits ? (1ull << 52) : 0ull);
-  const int e_eff = ebits ? ebits : 1;
-  // |x| = mant 2^(e_eff - 1075); F = |x| 2^(49 - E) = mant >> (1026 + E - e_eff)
-  const int sh = 1026 + E - e_eff;
-  const unsigned long long F = (sh >= 64 || sh < 0) ? 0ull : (mant >> sh);
-  const uint16_t sign = (uint16_t)((bits >> 48) & 0x8000u);
-#pragma unroll
-  for (int i = 0; i < kSlices; ++i) {
-    const uint32_t q = (uint32_t)(F >> (kSliceBits * (kSlices - 1 - i))) & ((1u << kSliceBits) - 1u);
-    out[i] = (uint16_t)(__float_as_uint((float)q) >> 16) | (q ? sign : (uint16_t)0);
+  const int sh = 1075 - B + E - (ebits ? ebits : 1);   // F = mant 2^-sh, sh >= 53 - B for |v| < 1
+  unsigned long long F;
+  if (B > 53 && sh <= 0) {
+    F = mant << min(-sh, 63);
+  } else {
+    const int r = min(max(sh, 1), 63);
+    F = (mant + (1ull << (r - 1))) >> r;
   }
+  const unsigned long long neg = (unsigned long long)((long long)bits >> 63);   // 0 or all ones
+  constexpr unsigned long long bias = (0x8080808080808080ull >> (8 * (8 - (S - 1))));
+  const unsigned long long t = ((F ^ neg) - neg) + bias;
+  const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
+  // 2^23 + byte as a float, less 2^23 + 128
+#pragma unroll
+  for (int i = 1; i < S; ++i) {
+    const int byte = S - 1 - i;
+    const uint32_t f = __byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7650u + (byte & 3));
+    out[i] = __uint_as_float(f) - 8388736.f;
+  }
+  const int d0 = (int)((long long)t >> (8 * (S - 1)));   // |d0| <= 2^top
+  out[0] = __uint_as_float(0x4B000000u + (uint32_t)(d0 + 512)) - 8389120.f;
 }
 
-// Exponent E with max|entries| < 2^E (0 for an all-zero vector).
-__device__ __forceinline__ int exp_above(double m) {
-  int e = 0;
-  if (m > 0.0) frexp(m, &e);
-  return e;
+// Exponent E with max|entries| < 2^E (0 for an all-zero vector), from the bits of the
+// maximum (non-negative doubles order like their bits, so maxima are integer compares).  An
+// infinity or a NaN gives 1025, more than any finite maximum: such a column's outputs are NaN.
+constexpr int kExpNonFinite = 1025;
+__device__ __forceinline__ int exp_above(unsigned long long mbits) {
+  if (mbits == 0ull) return 0;
+  const int e = (int)(mbits >> 52);
+  return e ? e - 1022 : -1010 - __clzll((long long)mbits);   // subnormal: top bit p, 2^(p - 1074) <= m
 }
 
-// Set-up: rows of every matrix (mats of Nr x Nr, row-major [n][j]) into 7 BF16 planes
-// [mat * 7 + plane][n][pitch] and the row exponents rowexp[mat][n].  One warp per row.
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+
+// Set-up: rows of every matrix (mats of Nr x Nr, row-major [n][j]) into S BF16 planes
+// [mat * S + plane][n][pitch] and the row exponents rowexp[mat][n].  One warp per row.
+template <int S>
 __global__ void k_f64s_matrix(const double* __restrict__ A, int nmat, int Nr, int pitch, uint16_t* __restrict__ planes,
                               int32_t* __restrict__ rowexp) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= nmat * Nr) return;
   const int mat = warp / Nr, n = warp - mat * Nr;
   const double* row = A + ((size_t)mat * Nr + n) * Nr;
-  double m = 0.0;
-  for (int j = lane; j < Nr; j += 32) m = fmax(m, fabs(row[j]));
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  unsigned long long m = 0ull;
+  for (int j = lane; j < Nr; j += 32) m = max(m, abs_bits(row[j]));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int E = exp_above(m);
   if (lane == 0) rowexp[mat * Nr + n] = E;
   const size_t plane_elems = (size_t)Nr * pitch;
   for (int j = lane; j < pitch; j += 32) {
-    uint16_t sl[kSlices];
-    if (j < Nr) {
-      slice7(row[j], E, sl);
-    } else {
+    float d[S];
+    digits_of<S>(j < Nr ? row[j] : 0.0, E, d);
 #pragma unroll
-      for (int i = 0; i < kSlices; ++i) sl[i] = 0;
-    }
-#pragma unroll
-    for (int i = 0; i < kSlices; ++i) planes[((size_t)mat * kSlices + i) * plane_elems + (size_t)n * pitch + j] = sl[i];
+    for (int i = 0; i < S; ++i)
+      planes[((size_t)mat * S + i) * plane_elems + (size_t)n * pitch + j] = (uint16_t)(__float_as_uint(d[i]) >> 16);
   }
 }
 
-// Per DHT: colmax[b][c] = max_j |X_b[j][c]| as the bits of a non-negative double (which
-// order like the values), so that CTAs over slices of j combine with integer atomicMax;
-// colmax starts at 0.  Grid: (columns / 256, rows / 32, items).
-constexpr int kColRows = 32;
-__global__ void k_f64s_colmax(DhtBatch bt, int Nr, int Nc, unsigned long long* __restrict__ colmax) {
-  const int b = blockIdx.z;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= Nc) return;
-  const double* X = static_cast<const double*>(bt.X[b]);
-  const int j0 = blockIdx.y * kColRows, j1 = min(Nr, j0 + kColRows);
-  // |x| as the bits with the sign cleared (non-negative doubles order like their bits):
-  // integer compares, where fmax would run on the float64 unit
-  unsigned long long m = 0ull;
-#pragma unroll 8
-  for (int j = j0; j < j1; ++j) {
-    const unsigned long long a = (unsigned long long)__double_as_longlong(X[(size_t)j * Nc + c]) & 0x7fffffffffffffffull;
-    m = a > m ? a : m;
-  }
-  if (m) atomicMax(colmax + (size_t)b * Nc + c, m);
-}
-
-// Per DHT: the panels into 7 K-major BF16 planes [b * 7 + plane][c][jpad].  Tiles of
-// 64 columns x 32 rows j through shared memory: reads along c, writes along j.
-constexpr int kPanelC = 64, kPanelJ = 32;
-__global__ void __launch_bounds__(256) k_f64s_panel(DhtBatch bt, int Nr, int Nc, int jpad,
-                                                    const unsigned long long* __restrict__ colmax,
+// Per DHT: the panels' column exponents and their S K-major BF16 planes [b * S + plane][c][jpad].
+// One CTA per 32 columns of an item: the first walk over the rows takes the column maxima, the
+// second (from L2: the CTA's Nr x 256 bytes were just read) cuts the digits, in tiles of 64 rows
+// through shared memory, read along c and written along j in 16-byte stores.  Bound by its
+// memory traffic, 8 bytes in and 2 S out per value.  One kernel instead of a column-maximum
+// kernel with atomics, its memset and a slicing kernel that read the panel from HBM again.
+constexpr int kPanelC = 32, kPanelJ = 64, kPanelPitch = kPanelJ / 2 + 1;   // 32-bit words per row
+template <int S>
+__global__ void __launch_bounds__(256) k_f64s_panel(DhtBatch bt, int b0, int Nr, int Nc, int jpad,
                                                     int32_t* __restrict__ colexp, uint16_t* __restrict__ planes) {
-  __shared__ __align__(16) uint16_t tile[kSlices][kPanelC][kPanelJ + 2];   // rows of 68 bytes
-  const int b = blockIdx.z;
-  const int c0 = blockIdx.x * kPanelC, j0 = blockIdx.y * kPanelJ;
-  const double* X = static_cast<const double*>(bt.X[b]);
-  const int tc = threadIdx.x & (kPanelC - 1), tj = threadIdx.x >> 6;   // 64 x 4
+  __shared__ uint32_t tile[S][kPanelC][kPanelPitch];   // two j per word; odd pitch: no bank conflicts
+  __shared__ unsigned long long cmax[8][kPanelC];
+  const int c0 = blockIdx.x * kPanelC;
+  const double* X = static_cast<const double*>(bt.X[b0 + blockIdx.y]);
+  const int tc = threadIdx.x & (kPanelC - 1), tj = threadIdx.x >> 5;   // 32 x 8
   const int c = c0 + tc;
-  const int E = c < Nc ? exp_above(__longlong_as_double((long long)colmax[(size_t)b * Nc + c])) : 0;
-  if (blockIdx.y == 0 && tj == 0 && c < Nc) colexp[(size_t)b * Nc + c] = E;   // for the epilogue
-  double xv[kPanelJ / 4];   // all loads first, then the slicing
-#pragma unroll
-  for (int u = 0; u < kPanelJ / 4; ++u) {
-    const int j = j0 + tj + 4 * u;
-    xv[u] = (c < Nc && j < Nr) ? X[(size_t)j * Nc + c] : 0.0;
+  const bool in = c < Nc;
+  unsigned long long m = 0ull;
+  if (in) {
+#pragma unroll 16
+    for (int j = tj; j < Nr; j += 8) m = max(m, abs_bits(X[(size_t)j * Nc + c]));
   }
-#pragma unroll
-  for (int u = 0; u < kPanelJ / 4; ++u) {
-    uint16_t sl[kSlices];
-    slice7(xv[u], E, sl);
-#pragma unroll
-    for (int i = 0; i < kSlices; ++i) tile[i][tc][tj + 4 * u] = sl[i];
-  }
+  cmax[tj][tc] = m;
   __syncthreads();
-  // out: for each plane and column, kPanelJ consecutive j (64 bytes) as four 16-byte
-  // stores of 8 j each (jpad and j0 are multiples of 8, so a group is inside the row or past
-  // it whole; the tile's rows start on 4-byte boundaries: pitch 68 bytes)
+#pragma unroll
+  for (int q = 0; q < 8; ++q) m = max(m, cmax[q][tc]);
+  const int E = exp_above(m);
+  if (tj == 0 && in) colexp[(size_t)blockIdx.y * Nc + c] = E;   // for the epilogue
   const size_t plane_elems = (size_t)Nc * jpad;
-  constexpr int kQ = kPanelJ / 8;
-  for (int idx = threadIdx.x; idx < kSlices * kPanelC * kQ; idx += blockDim.x) {
-    const int i = idx / (kPanelC * kQ);
-    const int rem = idx - i * kPanelC * kQ;
-    const int cc = rem / kQ, jq = rem - cc * kQ;
-    const int cg = c0 + cc, jg = j0 + 8 * jq;
-    if (cg < Nc && jg < jpad) {
-      const uint32_t* t32 = reinterpret_cast<const uint32_t*>(&tile[i][cc][8 * jq]);
-      const uint4 v = make_uint4(t32[0], t32[1], t32[2], t32[3]);
-      *reinterpret_cast<uint4*>(planes + ((size_t)b * kSlices + i) * plane_elems + (size_t)cg * jpad + jg) = v;
+  uint16_t* out = planes + (size_t)blockIdx.y * S * plane_elems;
+  for (int j0 = 0; j0 < Nr; j0 += kPanelJ) {
+    double xv[kPanelJ / 8];   // all loads first, then the digits; row pairs (2 jp, 2 jp + 1)
+#pragma unroll
+    for (int u = 0; u < kPanelJ / 8; ++u) {
+      const int j = j0 + 2 * (tj + 8 * (u >> 1)) + (u & 1);
+      xv[u] = (in && j < Nr) ? X[(size_t)j * Nc + c] : 0.0;
+    }
+    __syncthreads();   // the previous tile has been written out
+#pragma unroll
+    for (int u = 0; u < kPanelJ / 16; ++u) {
+      float a[S], b[S];
+      digits_of<S>(xv[2 * u], E, a);
+      digits_of<S>(xv[2 * u + 1], E, b);
+#pragma unroll
+      for (int i = 0; i < S; ++i)   // the high halves: two BF16
+        tile[i][tc][tj + 8 * u] = __byte_perm(__float_as_uint(a[i]), __float_as_uint(b[i]), 0x7632);
+    }
+    __syncthreads();
+    // 8 consecutive j (16 bytes) per store; jpad and j0 are multiples of 8, so a group lies
+    // inside the row or past it whole
+    constexpr int kQ = kPanelJ / 8;
+    for (int idx = threadIdx.x; idx < S * kPanelC * kQ; idx += 256) {
+      const int jq = idx % kQ, cc = idx / kQ % kPanelC, i = idx / (kQ * kPanelC);
+      const int cg = c0 + cc, jg = j0 + 8 * jq;
+      if (cg < Nc && jg < jpad) {
+        const uint32_t* w = &tile[i][cc][4 * jq];
+        *reinterpret_cast<uint4*>(out + i * plane_elems + (size_t)cg * jpad + jg) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
   }
 }
 
 // SM100 shared-memory matrix descriptor: K-major, 64-byte swizzle (TMA's SWIZZLE_64B), 8-row
-// groups 512 B apart.
-__device__ __forceinline__ uint64_t make_desc_sw64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);   // start address
-  d |= (uint64_t)1u << 16;                   // leading byte offset (unused: K fits one row)
-  d |= (uint64_t)(512u >> 4) << 32;          // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1u << 46;                   // descriptor version (SM100)
-  d |= (uint64_t)4u << 61;                   // layout: SWIZZLE_64B
-  return d;
-}
+// groups 512 B apart.  The high word is constant; the low word holds the start address in
+// 16-byte units, so that moving along the stage is one 32-bit addition.
+constexpr uint32_t kDescHi = (512u >> 4) | (1u << 14) | (4u << 29);   // stride, SM100 version, SWIZZLE_64B
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo) { return ((uint64_t)kDescHi << 32) | lo; }
 
 // 3-D tiled tensor copy global -> shared (inner coordinate x, then y, z), completing its
 // bytes on `bar`.  x is a multiple of 32 BF16 elements: 64-byte aligned.
@@ -199,12 +242,13 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, int x, 
 }
 
 struct F64sMaps {
-  Sim::TensorMapBytes panel;   // [b * 7 + plane][c][j], box 32 j x 128 c
-  Sim::TensorMapBytes mats;    // [mat * 7 + plane][n][j], box 32 j x 32 n
+  Sim::TensorMapBytes panel;   // [b * S + plane][c][j], box 32 j x 128 c
+  Sim::TensorMapBytes mats;    // [mat * S + plane][n][j], box 32 j x 64 n
 };
 
 struct F64sParams {
   int Nr, Nc, n_tiles, m_tiles, tiles_total;
+  int b0;            // first batch item of this launch
   int16_t mat[24];   // compact matrix index of each batch item
 };
 
@@ -219,23 +263,72 @@ __device__ __forceinline__ F64sTile f64s_tile(int t, const F64sParams& P) {
   return F64sTile{rest / P.m_tiles, nt * kF64sN, (rest % P.m_tiles) * kF64sM};
 }
 
+// The issuing thread of warp W: the products of its accumulators over the digit pairs of one 16-K
+// step.  fresh: the step opens a K block, so each accumulator's first product overwrites it.
+template <int S, int W>
+__device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t la, uint32_t lb, uint32_t idesc, bool fresh) {
+  using F = F64sForm<S>;
+#pragma unroll
+  for (int a = 0; a < kF64sAcc; ++a) {
+    if (F::warp(a) != W) continue;
+    bool first = true;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {   // matrix digit i, panel digit j
+#pragma unroll
+      for (int j = 0; i + j < S; ++j) {
+        if (F::acc(i, j) != a) continue;
+        mma_f16(tmem + a * kF64sN, desc_of(la + j * (kF64sPlaneA >> 4)), desc_of(lb + i * (kF64sPlaneB >> 4)), idesc,
+                first && fresh ? 0u : 1u);
+        first = false;
+      }
+    }
+  }
+}
+
+// 4 columns of one accumulator.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+
+__device__ __forceinline__ int acc_int(uint32_t r) { return __float2int_rn(__uint_as_float(r)); }
+
+// y = t 2^k (t a float64 near an integer), the scaling as an addition to the exponent field
+// while the result stays normal.
+__device__ __forceinline__ double scale_pow2(double t, int k) {
+  const long long bits = __double_as_longlong(t);
+  const int ex = (int)((bits >> 52) & 0x7ff) + k;
+  if (t != 0.0 && ex > 0 && ex < 2047) return __longlong_as_double(bits + (long long)k * (1LL << 52));
+  return t * ldexp(1.0, k);   // zero, or a result outside the normal range
+}
+
+// A tile's accumulators are drained in two steps: the group sums of a thread's 16 outputs are
+// combined into 64-bit integers and TMEM is released at once, so that the next tile's products
+// run while these warps convert to float64 (one instruction per output on the scarce float64
+// unit; three for S = 8) and store.  With the conversions before the release the products stood
+// still for 14 k of a tile's 35 k cycles.
+template <int S>
 __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sParams P,
                                                                const __grid_constant__ F64sMaps maps,
                                                                const int32_t* __restrict__ colexp,
                                                                const int32_t* __restrict__ rowexp, int32_t* err) {
+  constexpr int kStages = F64sForm<S>::stages;
+  constexpr uint32_t kStageBytes = f64s_stage_bytes<S>();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(base + kF64sStages * kF64sStageBytes);
-  uint64_t* empty = full + kF64sStages;
-  uint64_t* tfull = empty + kF64sStages;
-  uint64_t* tempty = tfull + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + kStages * kStageBytes);
+  uint64_t* empty = full + kStages;
+  uint64_t* tfull = empty + kStages;
+  uint64_t* tempty = tfull + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nK = (P.Nr + kF64sKC - 1) / kF64sKC;
-  constexpr uint32_t kTmemCols = 512;                 // sets x 7 groups x kF64sN columns <= 512
-  constexpr uint32_t kSetCols = kSlices * kF64sN;
+  const int nK = (P.Nr + kF64sKC - 1) / kF64sKC;       // K chunks of a tile
+  constexpr int kPerBlock = kF64sKBlock / kF64sKC;     // K chunks between drains
+  constexpr uint32_t kTmemCols = 512;
 
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -244,14 +337,12 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < kF64sStages; ++i) {
+    for (int i = 0; i < kStages; ++i) {
       mbar_init(&full[i], 1);    // the copy issuer's arrive.expect_tx
       mbar_init(&empty[i], 3);   // one MMA commit per issuing warp
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&tfull[i], 3);   // the issuing warps' commits after a tile's last chunk
-      mbar_init(&tempty[i], 16);  // one arrival per epilogue warp
-    }
+    mbar_init(tfull, 3);    // the issuing warps' commits after a K block's last chunk
+    mbar_init(tempty, 16);  // one arrival per epilogue warp
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -259,7 +350,7 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  // kind::f16: D f32, A and B bf16, both K-major; N = 32, M = 128
+  // kind::f16: D f32, A and B bf16, both K-major; N = 64, M = 128
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kF64sN >> 3) << 17) |
                          ((uint32_t)(kF64sM >> 4) << 24);
 
@@ -275,21 +366,21 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
       int last_armed = -1;
       for (int t = blockIdx.x; t < P.tiles_total && !*abort_flag; t += gridDim.x) {
         const F64sTile w = f64s_tile(t, P);
-        const int zm = P.mat[w.b] * kSlices, zp = w.b * kSlices;
+        const int zm = P.mat[P.b0 + w.b] * S, zp = w.b * S;
         bool ok = true;
         for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int st = (int)(g % (uint32_t)kF64sStages);
-          const uint32_t use = g / (uint32_t)kF64sStages;
+          const int st = (int)(g % (uint32_t)kStages);
+          const uint32_t use = g / (uint32_t)kStages;
           if (use > 0 && !mbar_wait(&empty[st], (use - 1) & 1)) { fail(); ok = false; break; }
           if (*abort_flag) { ok = false; break; }
-          unsigned char* sA = base + st * kF64sStageBytes;
-          unsigned char* sB = sA + kSlices * kF64sPlaneA;
-          mbar_arrive_expect_tx(&full[st], kF64sStageBytes);
+          unsigned char* sA = base + st * kStageBytes;
+          unsigned char* sB = sA + S * kF64sPlaneA;
+          mbar_arrive_expect_tx(&full[st], kStageBytes);
 #pragma unroll
-          for (int p = 0; p < kSlices; ++p)
+          for (int p = 0; p < S; ++p)
             tma_load_3d(sA + p * kF64sPlaneA, &maps.panel, kc * kF64sKC, w.c0, zp + p, &full[st]);
 #pragma unroll
-          for (int p = 0; p < kSlices; ++p)
+          for (int p = 0; p < S; ++p)
             tma_load_3d(sB + p * kF64sPlaneB, &maps.mats, kc * kF64sKC, w.n0, zm + p, &full[st]);
           last_armed = st;
         }
@@ -298,54 +389,46 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
       // before shared memory is released: the last armed stage's copies must have landed
       if (last_armed >= 0 && *abort_flag) {
         const uint32_t gl = g == 0 ? 0 : g - 1;
-        mbar_wait(&full[last_armed], (gl / (uint32_t)kF64sStages) & 1);
+        mbar_wait(&full[last_armed], (gl / (uint32_t)kStages) & 1);
       }
     }
     __syncwarp();
   } else if (warp >= 1 && warp <= 3) {
     // ---------------------------------------------------------------- MMA issuers
-    // Three warps issue the products, each into its own accumulator groups (so every
-    // group's first, overwriting product comes from one thread): warp 1 groups 0, 1, 6 (10
-    // products per 16 K), warp 2 groups 2, 5 (9), warp 3 groups 3, 4 (9).  One thread
-    // issuing all 28 left the tensor pipe three quarters idle.
+    // Three warps issue the products, each into its own accumulators (so every accumulator's
+    // first, overwriting product comes from one thread).  One thread issuing all of them left
+    // the tensor pipe three quarters idle.
     if (lane == 0) {
-      const uint32_t gmask = warp == 1 ? 0x43u : (warp == 2 ? 0x24u : 0x18u);   // groups of this warp
-      uint32_t g = 0, i = 0;
+      uint32_t g = 0, i = 0;   // chunks, K blocks
       uint64_t* last_bar = nullptr;
       uint32_t last_parity = 0;
-      for (int t = blockIdx.x; t < P.tiles_total && !*abort_flag; t += gridDim.x, ++i) {
-        const uint32_t set = i % kF64sSets, set_use = i / kF64sSets;
-        if (set_use > 0 && !mbar_wait(&tempty[set], (set_use - 1) & 1)) { fail(); break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d0 = tmem + set * kSetCols;
-        bool ok = true;
-        for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int st = (int)(g % (uint32_t)kF64sStages);
-          if (!mbar_wait(&full[st], (g / (uint32_t)kF64sStages) & 1)) { fail(); ok = false; break; }
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < P.tiles_total && !*abort_flag; t += gridDim.x) {
+        for (int k0 = 0; ok && k0 < nK; k0 += kPerBlock, ++i) {
+          if (i > 0 && !mbar_wait(tempty, (i - 1) & 1)) { fail(); ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = smem_u32(base + st * kF64sStageBytes), sb = sa + kSlices * kF64sPlaneA;
+          const int k1 = min(k0 + kPerBlock, nK);
+          for (int kc = k0; kc < k1; ++kc, ++g) {
+            const int st = (int)(g % (uint32_t)kStages);
+            if (!mbar_wait(&full[st], (g / (uint32_t)kStages) & 1)) { fail(); ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t la = desc_lo(smem_u32(base + st * kStageBytes)), lb = la + ((S * kF64sPlaneA) >> 4);
 #pragma unroll
-          for (int ks = 0; ks < 2; ++ks) {
-            const uint32_t koff = ks * 32;
-#pragma unroll
-            for (int grp = 0; grp < kSlices; ++grp) {
-              if (!((gmask >> grp) & 1u)) continue;
-#pragma unroll
-              for (int ia = 0; ia <= grp; ++ia) {   // matrix slice ia, panel slice grp - ia
-                const uint32_t accf = (kc > 0 || ks > 0 || ia > 0) ? 1u : 0u;
-                mma_f16(d0 + grp * kF64sN, make_desc_sw64(sa + (grp - ia) * kF64sPlaneA + koff),
-                        make_desc_sw64(sb + ia * kF64sPlaneB + koff), idesc, accf);
-              }
+            for (int ks = 0; ks < 2; ++ks) {   // 16 K: 32 bytes along the swizzled row
+              const bool fresh = kc == k0 && ks == 0;
+              if (warp == 1) issue_products<S, 1>(tmem, la + 2 * ks, lb + 2 * ks, idesc, fresh);
+              else if (warp == 2) issue_products<S, 2>(tmem, la + 2 * ks, lb + 2 * ks, idesc, fresh);
+              else issue_products<S, 3>(tmem, la + 2 * ks, lb + 2 * ks, idesc, fresh);
             }
+            mma_commit(&empty[st]);
+            last_bar = &empty[st];
+            last_parity = (g / (uint32_t)kStages) & 1;
           }
-          mma_commit(&empty[st]);
-          last_bar = &empty[st];
-          last_parity = (g / (uint32_t)kF64sStages) & 1;
+          if (!ok) break;
+          mma_commit(tfull);
+          last_bar = tfull;
+          last_parity = i & 1;
         }
-        if (!ok) break;
-        mma_commit(&tfull[set]);
-        last_bar = &tfull[set];
-        last_parity = (i / kF64sSets) & 1;
       }
       if (*abort_flag && last_bar) mbar_wait(last_bar, last_parity);
     }
@@ -354,70 +437,79 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
     // ---------------------------------------------------------------- epilogue (warps 4-19)
     // four warps per TMEM lane quarter (warp % 4 == q: lanes 32q .. 32q + 31), each taking
     // a quarter of the tile's columns
-    const int q = warp & 3, jh = ((warp - 4) >> 2) * (kF64sN / 4);
+    constexpr int kCols = kF64sN / 4;
+    const int q = warp & 3, jh = ((warp - 4) >> 2) * kCols;
+    const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)jh;
     uint32_t i = 0;
-    for (int t = blockIdx.x; t < P.tiles_total && !*abort_flag; t += gridDim.x, ++i) {
-      const uint32_t set = i % kF64sSets;
-      if (!mbar_wait(&tfull[set], (i / kF64sSets) & 1)) { fail(); break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < P.tiles_total && !*abort_flag; t += gridDim.x) {
       const F64sTile w = f64s_tile(t, P);
-      double* __restrict__ Y = static_cast<double*>(bt.Y[w.b]);
-      const int c = w.c0 + q * 32 + lane;
-      const int Ec = c < P.Nc ? colexp[(size_t)w.b * P.Nc + c] : 0;
-      const int32_t* rexp = rowexp + (size_t)P.mat[w.b] * P.Nr;
-      for (int j0 = jh; j0 < jh + kF64sN / 4; j0 += 8) {
-        // the group sums of 8 columns: groups 0..3 exact integers below 2^24 in float,
-        // groups 4..6 below 2^25 within one rounding
-        uint32_t r[kSlices][8];
+      // S = 6: sum = hi 2^-54 (group 5 rounded to that unit); S = 8: sum = hi 2^-36 + lo 2^-68
+      long long hi[kCols], lo[S == kF64sDigits ? 1 : kCols];
 #pragma unroll
-        for (int grp = 0; grp < kSlices; ++grp) {
-          const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + set * kSetCols + grp * kF64sN + (uint32_t)j0;
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-              : "=r"(r[grp][0]), "=r"(r[grp][1]), "=r"(r[grp][2]), "=r"(r[grp][3]), "=r"(r[grp][4]),
-                "=r"(r[grp][5]), "=r"(r[grp][6]), "=r"(r[grp][7])
-              : "r"(taddr)
-              : "memory");
-        }
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (c < P.Nc) {
+      for (int e = 0; e < kCols; ++e) {
+        hi[e] = 0;
+        if (S != kF64sDigits) lo[e] = 0;
+      }
+      for (int k0 = 0; k0 < nK; k0 += kPerBlock, ++i) {
+        if (!mbar_wait(tfull, i & 1)) { fail(); ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int n = w.n0 + j0 + e;
-            if (n >= P.Nr) continue;
-            // sum_g acc_g 2^(-7(g+2)) = T 2^-49 with
-            //   T = (((a0 2^7 + a1) 2^7 + a2) 2^7 + a3) 2^14 + a4 2^7 + a5 + round(a6 2^-7),
-            // all in integer arithmetic: a0..a3 are exact integers below 2^24, a4..a6
-            // integer-valued floats below 2^25 (their sums were rounded at weight <= 2^-42);
-            // |T| < 2^58.  Then one int -> double conversion, the only float64 instruction
-            // (GB300's float64 unit is the scarce one), and the scaling by 2^k as an addition
-            // to the exponent field while the result stays normal.
-            const long long a0 = __float2int_rn(__uint_as_float(r[0][e]));
-            const long long a1 = __float2int_rn(__uint_as_float(r[1][e]));
-            const long long a2 = __float2int_rn(__uint_as_float(r[2][e]));
-            const long long a3 = __float2int_rn(__uint_as_float(r[3][e]));
-            const long long a4 = __float2int_rn(__uint_as_float(r[4][e]));
-            const long long a5 = __float2int_rn(__uint_as_float(r[5][e]));
-            const long long a6 = __float2int_rn(__uint_as_float(r[6][e]) * (1.f / 128.f));
-            const long long T = (((a0 * 128 + a1) * 128 + a2) * 128 + a3) * 16384 + a4 * 128 + a5 + a6;
-            const int k = Ec + rexp[n] - kSliceBits * kSlices;   // 2^(E_c + E_n - 49)
-            const double t = (double)T;
-            long long bits = __double_as_longlong(t);
-            const int ex = (int)((bits >> 52) & 0x7ff) + k;
-            double y;
-            if (T != 0 && ex > 0 && ex < 2047) {
-              bits += (long long)k * (1LL << 52);
-              y = __longlong_as_double(bits);
+        for (int j = 0; j < kCols; j += 4) {
+          uint32_t r[kF64sAcc][4];
+#pragma unroll
+          for (int a = 0; a < kF64sAcc; ++a) tmem_ld4(taddr + a * kF64sN + j, r[a]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if constexpr (S == kF64sDigits) {
+              // one K block: the groups' weights are 2^-(16 + 8 g); |sum| <= 2^8
+              const long long a0 = acc_int(r[0][e]), a1 = acc_int(r[1][e]);
+              const long long a2 = acc_int(r[2][e]) + acc_int(r[3][e]), a3 = acc_int(r[4][e]) + acc_int(r[5][e]);
+              const int a4 = acc_int(r[6][e]), a5 = __float2int_rn(__uint_as_float(r[7][e]) * 0.25f);
+              hi[j + e] = a0 * (1LL << 38) + a1 * (1LL << 30) + a2 * (1LL << 22) + a3 * (1LL << 14) +
+                          ((long long)a4 * 64 + a5);
             } else {
-              y = t * ldexp(1.0, k);   // zero, or a result outside the normal range
+              // weights 2^-(12 + 8 g); |a_g| <= 2^25 a block and at most 4 blocks: both sums < 2^53
+              hi[j + e] += (long long)acc_int(r[0][e]) * (1 << 24) + (long long)acc_int(r[1][e]) * (1 << 16) +
+                           (long long)acc_int(r[2][e]) * (1 << 8) + acc_int(r[3][e]);
+              lo[j + e] += (long long)acc_int(r[4][e]) * (1 << 24) + (long long)acc_int(r[5][e]) * (1 << 16) +
+                           (long long)acc_int(r[6][e]) * (1 << 8) + acc_int(r[7][e]);
             }
-            Y[(size_t)n * P.Nc + c] = y;
+            // combined before the next columns are loaded (else their raw sums pile up in registers)
+            asm volatile("" : "+l"(hi[j + e]));
+            if (S != kF64sDigits) asm volatile("" : "+l"(lo[S == kF64sDigits ? 0 : j + e]));
           }
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[set]);
+      if (!ok) break;
+      double* __restrict__ Y = static_cast<double*>(bt.Y[P.b0 + w.b]);
+      const int c = w.c0 + q * 32 + lane, n0 = w.n0 + jh;
+      if (c < P.Nc) {
+        const int Ec = colexp[(size_t)w.b * P.Nc + c];
+        const int32_t* rexp = rowexp + (size_t)P.mat[P.b0 + w.b] * P.Nr;
+#pragma unroll
+        for (int e = 0; e < kCols; ++e) {
+          const int n = n0 + e;
+          if (n < P.Nr) {
+            double v;
+            int k = Ec + rexp[n];
+            if constexpr (S == kF64sDigits) {
+              v = (double)hi[e];
+              k -= 54;
+            } else {
+              v = fma((double)lo[e], 0x1p-32, (double)hi[e]);   // exact conversions, one rounding
+              k -= 36;
+            }
+            Y[(size_t)n * P.Nc + c] =
+                Ec == kExpNonFinite ? __longlong_as_double(0x7ff8000000000000ll) : scale_pow2(v, k);
+          }
+          asm volatile("" ::: "memory");   // one output at a time: no pile of addresses and exponents
+        }
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -427,10 +519,6 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-constexpr size_t kF64sSmem = 1024 + (size_t)kF64sStages * kF64sStageBytes + 256;
-static_assert(kF64sSets * kSlices * kF64sN <= 512, "accumulators exceed tensor memory");
-static_assert(kF64sSmem <= 227 * 1024, "stages exceed shared memory");
-
 int f64s_pitch(int Nr) { return split_pitch_b16(Nr); }   // BF16 row pitch, 16-byte rows
 
 int blocks_for(size_t n, int t) { return (int)((n + t - 1) / t); }
@@ -439,7 +527,19 @@ int blocks_for(size_t n, int t) { return (int)((n + t - 1) / t); }
 
 bool f64s_supported(const pic_config& c) { return c.precision == PIC_FP64 && c.Nr <= kF64sMaxNr; }
 
-bool f64s_active(const Sim* s) { return f64s_supported(s->cfg) && s->dht_path != PIC_DHT_F64_GEMM; }
+int f64s_digits(const pic_config& c) { return c.Nr <= kF64sMaxNr ? kF64sDigits : kF64sDigitsWide; }
+
+// Items whose panel planes the workspace holds at a time.  The wide form's planes are twice the
+// panels' bytes: a launch takes as many items as fit 1 GB (all 12 of a 2-mode run up to
+// 2048 x 1024), so that they stay a small part of the workspace at any size.
+int f64s_items(const pic_config& c) {
+  const size_t item = (size_t)f64s_digits(c) * 2 * c.Nz * f64s_pitch(c.Nr) * 2;
+  const int all = 6 * c.Nm;
+  if (c.Nr <= kF64sMaxNr) return all;
+  return std::max(1, std::min<int>(all, (int)(((size_t)1 << 30) / item)));
+}
+
+bool f64s_active(const Sim* s) { return s->cfg.precision == PIC_FP64 && s->dht_path != PIC_DHT_F64_GEMM; }
 
 pic_status f64s_configure_device() {
   static std::mutex mu;
@@ -448,24 +548,27 @@ pic_status f64s_configure_device() {
   PIC_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lock(mu);
   if (dev >= 0 && dev < 64 && done[dev]) return PIC_OK;
-  PIC_CUDA(cudaFuncSetAttribute(k_dht_f64s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF64sSmem));
+  PIC_CUDA(cudaFuncSetAttribute(k_dht_f64s<kF64sDigits>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)f64s_smem<kF64sDigits>()));
+  PIC_CUDA(cudaFuncSetAttribute(k_dht_f64s<kF64sDigitsWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)f64s_smem<kF64sDigitsWide>()));
   if (dev >= 0 && dev < 64) done[dev] = true;
   return PIC_OK;
 }
 
-// Set-up (after the FP64 matrices are final): slices of the forward matrices (compact
+// Set-up (after the FP64 matrices are final): digits of the forward matrices (compact
 // index 0 .. 3Nm-1) and of the inverse matrices (3Nm .. 6Nm-1).
 pic_status launch_f64s_setup(Sim* s) {
-  if (!f64s_supported(s->cfg)) return PIC_OK;
-  const int Nr = s->cfg.Nr, nm3 = 3 * s->cfg.Nm, pitch = f64s_pitch(Nr);
+  const int Nr = s->cfg.Nr, nm3 = 3 * s->cfg.Nm, pitch = f64s_pitch(Nr), S = f64s_digits(s->cfg);
   uint16_t* planes = s->at<uint16_t>(s->lay.f64s_mat);
   int32_t* rowexp = s->at<int32_t>(s->lay.f64s_rowexp);
-  const size_t mat_elems = (size_t)kSlices * Nr * pitch;
+  const size_t mat_elems = (size_t)S * Nr * pitch;
   const int blocks = blocks_for((size_t)nm3 * Nr * 32, 256);
-  k_f64s_matrix<<<blocks, 256, 0, s->stream>>>(s->at<double>(s->lay.mfwd), nm3, Nr, pitch, planes, rowexp);
+  auto* k = S == kF64sDigits ? k_f64s_matrix<kF64sDigits> : k_f64s_matrix<kF64sDigitsWide>;
+  k<<<blocks, 256, 0, s->stream>>>(s->at<double>(s->lay.mfwd), nm3, Nr, pitch, planes, rowexp);
   PIC_LAUNCHED(s);
-  k_f64s_matrix<<<blocks, 256, 0, s->stream>>>(s->at<double>(s->lay.binv), nm3, Nr, pitch,
-                                               planes + (size_t)nm3 * mat_elems, rowexp + (size_t)nm3 * Nr);
+  k<<<blocks, 256, 0, s->stream>>>(s->at<double>(s->lay.binv), nm3, Nr, pitch, planes + (size_t)nm3 * mat_elems,
+                                   rowexp + (size_t)nm3 * Nr);
   PIC_LAUNCHED(s);
   return PIC_OK;
 }
@@ -474,7 +577,7 @@ pic_status launch_f64s_setup(Sim* s) {
 // item or matrix x plane), 64-byte swizzle; coordinates past Nr (j, n) or Nc read zero.
 pic_status f64s_make_maps(Sim* s) {
   std::memset(s->f64s_maps, 0, sizeof(s->f64s_maps));
-  if (!f64s_supported(s->cfg)) return PIC_OK;
+  if (s->cfg.precision != PIC_FP64) return PIC_OK;
   using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -483,51 +586,60 @@ pic_status f64s_make_maps(Sim* s) {
     set_error("cuTensorMapEncodeTiled is not available from the driver");
     return PIC_ERR_CUDA;
   }
-  const int Nr = s->cfg.Nr, Nc = 2 * s->cfg.Nz, pitch = f64s_pitch(Nr);
-  const cuuint32_t estr[3] = {1, 1, 1};
-  {
-    const cuuint64_t dims[3] = {(cuuint64_t)Nr, (cuuint64_t)Nc, (cuuint64_t)(6 * s->cfg.Nm * kSlices)};
-    const cuuint64_t strides[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)Nc * pitch * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)kF64sKC, (cuuint32_t)kF64sM, 1};
-    const CUresult r = encode(reinterpret_cast<CUtensorMap*>(s->f64s_maps[0].b), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
-                              s->at<char>(s->lay.f64s_panel), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  const int Nr = s->cfg.Nr, Nc = 2 * s->cfg.Nz, pitch = f64s_pitch(Nr), S = f64s_digits(s->cfg);
+  auto make = [&](int id, size_t off, int rows, int planes, int box_rows, const char* what) -> pic_status {
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const cuuint64_t dims[3] = {(cuuint64_t)Nr, (cuuint64_t)rows, (cuuint64_t)planes};
+    const cuuint64_t strides[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)rows * pitch * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)kF64sKC, (cuuint32_t)box_rows, 1};
+    const CUresult r = encode(reinterpret_cast<CUtensorMap*>(s->f64s_maps[id].b), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                              s->at<char>(off), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-      set_error("cuTensorMapEncodeTiled failed (%d) for the sliced panels", (int)r);
-      return PIC_ERR_CUDA;
-    }
-  }
-  {
-    const cuuint64_t dims[3] = {(cuuint64_t)Nr, (cuuint64_t)Nr, (cuuint64_t)(6 * s->cfg.Nm * kSlices)};
-    const cuuint64_t strides[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)Nr * pitch * 2};
-    const cuuint32_t box[3] = {(cuuint32_t)kF64sKC, (cuuint32_t)kF64sN, 1};
-    const CUresult r = encode(reinterpret_cast<CUtensorMap*>(s->f64s_maps[1].b), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
-                              s->at<char>(s->lay.f64s_mat), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-      set_error("cuTensorMapEncodeTiled failed (%d) for the sliced matrices", (int)r);
-      return PIC_ERR_CUDA;
-    }
-  }
+    if (r == CUDA_SUCCESS) return PIC_OK;
+    set_error("cuTensorMapEncodeTiled failed (%d) for the sliced %s", (int)r, what);
+    return PIC_ERR_CUDA;
+  };
+  const pic_status st = make(0, s->lay.f64s_panel, Nc, f64s_items(s->cfg) * S, kF64sM, "panels");
+  return st != PIC_OK ? st : make(1, s->lay.f64s_mat, Nr, 6 * s->cfg.Nm * S, kF64sN, "matrices");
+}
+
+namespace {
+
+template <int S>
+pic_status launch_items(Sim* s, const DhtBatch& b, F64sParams P, int items) {
+  const int Nr = P.Nr, Nc = P.Nc;
+  int32_t* colexp = s->at<int32_t>(s->lay.f64s_colexp);
+  k_f64s_panel<S><<<dim3(blocks_for(Nc, kPanelC), items), 256, 0, s->stream>>>(
+      b, P.b0, Nr, Nc, f64s_pitch(Nr), colexp, s->at<uint16_t>(s->lay.f64s_panel));
+  PIC_LAUNCHED(s);
+  F64sMaps maps;
+  maps.panel = s->f64s_maps[0];
+  maps.mats = s->f64s_maps[1];
+  P.tiles_total = P.n_tiles * P.m_tiles * items;
+  const int grid = std::min(P.tiles_total, dht_tc_sm_count());
+  k_dht_f64s<S><<<grid, kF64sThreads, f64s_smem<S>(), s->stream>>>(b, P, maps, colexp,
+                                                                   s->at<int32_t>(s->lay.f64s_rowexp),
+                                                                   s->at<int32_t>(s->lay.err));
+  PIC_LAUNCHED(s);
   return PIC_OK;
 }
 
-// Y = A X of a batch in the FP64 form on the tensor cores: column exponents, panel slices,
+}  // namespace
+
+// Y = A X of a batch in the FP64 form on the tensor cores: column exponents and panel digits,
 // then the persistent product kernel.
 pic_status launch_dht_f64s(Sim* s, const DhtBatch& b) {
-  const int Nr = s->cfg.Nr, Nc = 2 * s->cfg.Nz, Nm = s->cfg.Nm, pitch = f64s_pitch(Nr);
+  const int Nm = s->cfg.Nm;
   if (b.n < 1 || b.n > 6 * Nm) {
     set_error("sliced FP64 DHT: batch of %d items (1 .. %d)", b.n, 6 * Nm);
     return PIC_ERR_ARG;
   }
   F64sParams P{};
-  P.Nr = Nr;
-  P.Nc = Nc;
-  P.n_tiles = (Nr + kF64sN - 1) / kF64sN;
-  P.m_tiles = (Nc + kF64sM - 1) / kF64sM;
-  P.tiles_total = P.n_tiles * P.m_tiles * b.n;
+  P.Nr = s->cfg.Nr;
+  P.Nc = 2 * s->cfg.Nz;
+  P.n_tiles = (P.Nr + kF64sN - 1) / kF64sN;
+  P.m_tiles = (P.Nc + kF64sM - 1) / kF64sM;
   for (int i = 0; i < b.n; ++i) {
     const int id = b.mat[i], per = kMaxModes * 3;
     const int dir = id / per, mi = id % per;
@@ -537,21 +649,13 @@ pic_status launch_dht_f64s(Sim* s, const DhtBatch& b) {
     }
     P.mat[i] = (int16_t)(dir * 3 * Nm + mi);
   }
-  int32_t* colexp = s->at<int32_t>(s->lay.f64s_colexp);
-  unsigned long long* colmax = reinterpret_cast<unsigned long long*>(colexp + (size_t)6 * Nm * Nc);
-  PIC_CUDA(cudaMemsetAsync(colmax, 0, (size_t)b.n * Nc * sizeof(unsigned long long), s->stream));
-  k_f64s_colmax<<<dim3(blocks_for(Nc, 256), blocks_for(Nr, kColRows), b.n), 256, 0, s->stream>>>(b, Nr, Nc, colmax);
-  PIC_LAUNCHED(s);
-  k_f64s_panel<<<dim3(blocks_for(Nc, kPanelC), blocks_for(Nr, kPanelJ), b.n), 256, 0, s->stream>>>(
-      b, Nr, Nc, pitch, colmax, colexp, s->at<uint16_t>(s->lay.f64s_panel));
-  PIC_LAUNCHED(s);
-  F64sMaps maps;
-  maps.panel = s->f64s_maps[0];
-  maps.mats = s->f64s_maps[1];
-  const int grid = std::min(P.tiles_total, dht_tc_sm_count());
-  k_dht_f64s<<<grid, kF64sThreads, kF64sSmem, s->stream>>>(b, P, maps, colexp, s->at<int32_t>(s->lay.f64s_rowexp),
-                                                           s->at<int32_t>(s->lay.err));
-  PIC_LAUNCHED(s);
+  const int most = f64s_items(s->cfg);
+  for (; P.b0 < b.n; P.b0 += most) {
+    const int items = std::min(most, b.n - P.b0);
+    const pic_status st = f64s_digits(s->cfg) == kF64sDigits ? launch_items<kF64sDigits>(s, b, P, items)
+                                                             : launch_items<kF64sDigitsWide>(s, b, P, items);
+    if (st != PIC_OK) return st;
+  }
   return PIC_OK;
 }
 

@@ -121,12 +121,13 @@ Layout make_layout(const pic_config& c) {
       L.bspec_f = take((size_t)M * 8);
     }
   }
-  if (f64s_supported(c)) {
+  if (!mixed) {
     const size_t pitch = (size_t)split_pitch_b16(c.Nr), Nc = 2 * (size_t)c.Nz, nmat = 6 * (size_t)c.Nm;
-    L.f64s_mat = take(nmat * kF64sSlices * c.Nr * pitch * 2);
+    const size_t S = (size_t)f64s_digits(c), items = (size_t)f64s_items(c);
+    L.f64s_mat = take(nmat * S * c.Nr * pitch * 2);
     L.f64s_rowexp = take(nmat * c.Nr * 4);
-    L.f64s_panel = take(nmat * kF64sSlices * Nc * pitch * 2);
-    L.f64s_colexp = take(nmat * Nc * 4 + nmat * Nc * 8);   // exponents, then the column maxima
+    L.f64s_panel = take(items * S * Nc * pitch * 2);
+    L.f64s_colexp = take(items * Nc * 4);
   }
   if (mixed) {
     for (int b = 0; b < 2; ++b)

@@ -54,8 +54,8 @@ struct Layout {
   // Nz that is not 7-smooth (Bluestein, 0 otherwise): twiddles of the power-of-two length M,
   // the chirp w_n (Nz), the chirp filter's spectrum (M), float copies
   size_t twm, twm_f, chirp, chirp_f, bspec, bspec_f;
-  // FP64 form with Nr <= 256: the sliced tensor-core DHT (BF16 slice planes of the matrices
-  // and of the current panels, their row and column exponents)
+  // FP64 form: the sliced tensor-core DHT (BF16 digit planes of the matrices and of the
+  // current panels, their row and column exponents)
   size_t f64s_mat, f64s_rowexp, f64s_panel, f64s_colexp;
   size_t total;
 };
@@ -216,10 +216,13 @@ pic_status dht_tc_make_maps(Sim* s);     // once per handle: tensor maps of the 
 pic_status launch_wait_selftest(Sim* s, uint32_t max_polls);   // bounded wait that times out
 void* tensor_map_encoder();              // the driver's cuTensorMapEncodeTiled, or null
 int dht_tc_sm_count();                   // SMs of the current device
-// FP64 form, Nr <= kF64sMaxNr: the DHT from exact BF16 slice products on tcgen05 (dht_f64s.cu)
-constexpr int kF64sSlices = 7;
+// FP64 form: the DHT from exact BF16 digit products on tcgen05 (dht_f64s.cu), in kF64sDigits
+// digits up to Nr = kF64sMaxNr and kF64sDigitsWide beyond
+constexpr int kF64sDigits = 6, kF64sDigitsWide = 8;
 constexpr int kF64sMaxNr = 256;
-bool f64s_supported(const pic_config& c);
+bool f64s_supported(const pic_config& c);   // PIC_DHT_F64_SLICED may be asked for (Nr <= kF64sMaxNr)
+int f64s_digits(const pic_config& c);
+int f64s_items(const pic_config& c);        // batch items whose panel planes the workspace holds
 bool f64s_active(const Sim* s);
 pic_status f64s_configure_device();
 pic_status f64s_make_maps(Sim* s);
