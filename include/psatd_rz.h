@@ -393,16 +393,15 @@ pic_status pic_get_tuning(pic_sim* sim, pic_tuning* out);
  *                       numbers); the digit products accumulate exactly in FP32 on the tensor
  *                       cores and are combined in FP64: agrees with the FP64 product to about
  *                       2^-49 of (row max x column max x Nr).  Needs Nr <= 256.
- * With AUTO and SLICED the power-of-two z-FFT rows run in double words (each value a sum
- * of two floats, about 48 bits, on the float32 units; rows stay float64 in memory): the
- * pairs hold about 48 bits relative to a row's largest value while that lies between
- * about 2^-100 and 2^127 (the low parts' absolute resolution is 2^-149); values below
- * 2^-126 enter as zero and values from 2^128 on overflow; SI grids of plasma runs lie
- * well inside.  With them the inverse rows also leave a double-word copy of PIC_BUF_E and
- * PIC_BUF_B in the workspace, kept current by every call that writes those buffers, and
- * pic_gather_push reads that copy and forms the mode sum in double words too (error a few
- * 2^-48 of the sum of the weighted terms' magnitudes); with F64_GEMM, or an Nz that is not
- * a power of two, the gather reads the float64 grids.
+ * With AUTO and SLICED the 7-smooth z-FFT rows run in 64-bit block fixed point (64-bit
+ * integers with one exponent per row; rows stay float64 in memory and keep float64's range;
+ * no further off than IEEE float64 rows, both measured against extended precision).  With
+ * them the inverse rows of power-of-two Nz also leave a copy of PIC_BUF_E and PIC_BUF_B in
+ * double words (sums of two floats, about 48 bits) in the workspace, kept current by every
+ * call that writes those buffers, and pic_gather_push reads that copy and forms the mode sum
+ * in double words too (error a few 2^-48 of the sum of the weighted terms' magnitudes; fields
+ * below 2^-126 count as zero and from 2^128 on overflow there); with F64_GEMM, or an Nz that
+ * is not a power of two, the gather reads the float64 grids.
  * Errors: PIC_ERR_ARG (unknown path, or SLICED with Nr > 256 or a mixed form). */
 typedef enum { PIC_DHT_AUTO = 0, PIC_DHT_F64_GEMM = 1, PIC_DHT_F64_SLICED = 2 } pic_dht_path;
 pic_status pic_set_dht_path(pic_sim* sim, int32_t path);

@@ -2,11 +2,12 @@
 // quasi-cylindrical scheme (section "Finite order pseudo-spectral solvers").
 //   forward: Fhat(k) = sum_i F(z_i) e^{-2 pi i k i / Nz}
 //   inverse: F(z_i) = (1/Nz) sum_k Fhat(k) e^{+2 pi i k i / Nz}
-// Power-of-two lengths use radix-8 passes with the values in registers (k_fft_pow2 for
-// double rows; k_fft_pow2_tma for float rows, persistent and fed by bulk copies); other
-// 7-smooth lengths a mixed-radix (8, 4, 2, 3, 5, 7) self-sorting Stockham sequence of passes
-// between two shared row buffers (k_fft_rows).  All read per-pass twiddle tables.  Any
-// other length goes through Bluestein's chirp-z algorithm on power-of-two rows (below).
+// The FP64 form's 7-smooth rows run in block fixed point (fft_fix.cu) unless PIC_DHT_F64_GEMM
+// asks for IEEE float64.  Here: power-of-two lengths use radix-8 passes with the values in
+// registers (k_fft_pow2 for IEEE double rows; k_fft_pow2_tma for float rows, persistent and fed
+// by bulk copies); other 7-smooth lengths a mixed-radix (8, 4, 2, 3, 5, 7) self-sorting Stockham
+// sequence of passes between two shared row buffers (k_fft_rows).  All read per-pass twiddle
+// tables.  Any other length goes through Bluestein's chirp-z algorithm on power-of-two rows.
 // The component combination of the quasi-cylindrical scheme is fused into the row load:
 // out = ca * inA + cb * inB, which forms J_+- = (J_r -+ i J_theta)/2 before the forward
 // transform and E_r = E_+ + E_-, E_theta = i (E_+ - E_-) before the inverse one.
@@ -14,7 +15,6 @@
 #include <type_traits>
 
 #include "pic_internal.cuh"
-#include "dword.cuh"
 #include "tc_common.cuh"
 
 namespace pic {
@@ -23,8 +23,6 @@ namespace {
 template <typename R> struct Vec2;
 template <> struct Vec2<double> { using T = double2; };
 template <> struct Vec2<float> { using T = float2; };
-
-template <> struct Vec2<dw> { using T = dw2; };
 
 template <typename T> __device__ __forceinline__ T cmul(T a, T b) {
   T r;
@@ -76,9 +74,6 @@ __device__ __forceinline__ void row_coefs(const RowCombine& rc, int comp, C2& ca
   if constexpr (sizeof(R) == 4) {
     ca.x = rc.fcaRe[comp]; ca.y = rc.fcaIm[comp];
     cb.x = rc.fcbRe[comp]; cb.y = rc.fcbIm[comp];
-  } else if constexpr (std::is_same<R, dw>::value) {   // the coefficients are exact in float
-    ca.x = dw(rc.fcaRe[comp], 0.f); ca.y = dw(rc.fcaIm[comp], 0.f);
-    cb.x = dw(rc.fcbRe[comp], 0.f); cb.y = dw(rc.fcbIm[comp], 0.f);
   } else {
     ca.x = rc.caRe[comp]; ca.y = rc.caIm[comp];
     cb.x = rc.cbRe[comp]; cb.y = rc.cbIm[comp];
@@ -86,31 +81,6 @@ __device__ __forceinline__ void row_coefs(const RowCombine& rc, int comp, C2& ca
   ka = rc.kindA[comp]; kb = rc.kindB[comp];
   ua = rc.unitA[comp]; ub = rc.unitB[comp];
 }
-
-// 1/sqrt(2) and 1/N in the row arithmetic R.
-template <typename R> __device__ __forceinline__ R inv_sqrt2() { return (R)0.70710678118654752440; }
-template <> __device__ __forceinline__ dw inv_sqrt2<dw>() { return dw(0.70710676908493042f, 1.2101617485882343e-08f); }
-template <typename R> __device__ __forceinline__ R inv_len(int N) { return (R)1 / (R)N; }
-template <> __device__ __forceinline__ dw inv_len<dw>(int N) { return dw(1.f / (float)N, 0.f); }   // N a power of two
-
-
-// Element type of the rows in global memory for row arithmetic R (double-word rows are
-// stored as doubles), and the conversions between the two.
-template <typename R> struct GlobalOf { using T = typename Vec2<R>::T; };
-template <> struct GlobalOf<dw> { using T = double2; };
-template <typename C2, typename G2> __device__ __forceinline__ C2 from_global(const G2& v) {
-  if constexpr (std::is_same<C2, G2>::value) {
-    return v;
-  } else {
-    C2 r;
-    r.x = dw_from_double(v.x);
-    r.y = dw_from_double(v.y);
-    return r;
-  }
-}
-__device__ __forceinline__ double2 to_global(const dw2& v) { return make_double2(dw_to_double(v.x), dw_to_double(v.y)); }
-__device__ __forceinline__ float2 to_global(const float2& v) { return v; }
-__device__ __forceinline__ double2 to_global(const double2& v) { return v; }
 
 struct FftPlan {
   int N;
@@ -163,7 +133,7 @@ template <typename C2, bool INV> __device__ __forceinline__ void dft4(C2* v) {
 // b_r = (v_r - v_{r+4}) w_8^r.
 template <typename C2, bool INV> __device__ __forceinline__ void dft8(C2* v) {
   using R = decltype(v[0].x);
-  const R h = inv_sqrt2<R>();
+  const R h = (R)0.70710678118654752440;
   C2 a[4], b[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -191,13 +161,12 @@ template <typename C2, bool INV> __device__ __forceinline__ void dft8(C2* v) {
 }
 
 // Per-row context of the power-of-two kernel.
-template <typename C2, typename G2 = C2> struct RowCtx {
-  const G2* a;    // source rows of the combination (b may be null), in global memory
-  const G2* b;
+template <typename C2> struct RowCtx {
+  const C2* a;    // source rows of the combination (b may be null), in global memory
+  const C2* b;
   C2 ca, cb;
   int ka, kb, ua, ub;   // coefficient kinds and units (coef_mul)
-  G2* o;          // destination row
-  float4* odw;    // double-word copy of the destination row (double-word rows only; may be null)
+  C2* o;          // destination row
   C2* buf;        // padded shared row buffer
   int N, tr, TR;
   bool active;    // false for the idle row slots of the last CTA
@@ -206,8 +175,8 @@ template <typename C2, typename G2 = C2> struct RowCtx {
 template <int PS> __device__ __forceinline__ int padded(int i) { return i + (i >> PS); }
 
 // Inputs of the first pass (radix 8): v[8q + r] = (ca a + cb b)[t + r N/8], t = tr + q TR.
-template <typename C2, int E, typename G2>
-__device__ __forceinline__ void pow2_load_global(C2 (&v)[E], const RowCtx<C2, G2>& c) {
+template <typename C2, int E>
+__device__ __forceinline__ void pow2_load_global(C2 (&v)[E], const RowCtx<C2>& c) {
   using Re = decltype(v[0].x);
   const int N8 = c.N >> 3;
 #pragma unroll
@@ -218,8 +187,8 @@ __device__ __forceinline__ void pow2_load_global(C2 (&v)[E], const RowCtx<C2, G2
       C2 x;
       x.x = (Re)0; x.y = (Re)0;
       if (c.active) {
-        x = coef_mul(c.ca, c.ka, c.ua, from_global<C2>(c.a[idx]));
-        if (c.b) x = cadd(x, coef_mul(c.cb, c.kb, c.ub, from_global<C2>(c.b[idx])));
+        x = coef_mul(c.ca, c.ka, c.ua, c.a[idx]);
+        if (c.b) x = cadd(x, coef_mul(c.cb, c.kb, c.ub, c.b[idx]));
       }
       v[q * 8 + r] = x;
     }
@@ -227,8 +196,8 @@ __device__ __forceinline__ void pow2_load_global(C2 (&v)[E], const RowCtx<C2, G2
 }
 
 // Inputs of a later pass of radix R from the shared row buffer.
-template <typename C2, int E, int R, int PS, typename G2>
-__device__ __forceinline__ void pow2_load_shared(C2 (&v)[E], const RowCtx<C2, G2>& c) {
+template <typename C2, int E, int R, int PS>
+__device__ __forceinline__ void pow2_load_shared(C2 (&v)[E], const RowCtx<C2>& c) {
   const int NR = c.N / R;
 #pragma unroll
   for (int q = 0; q < E / R; ++q) {
@@ -265,8 +234,8 @@ __device__ __forceinline__ void pass_twiddles(C2 (&w)[R], const C2* __restrict__
 }
 
 // Twiddles and the R-point DFTs of a pass.
-template <typename C2, bool INV, int E, int R, typename G2>
-__device__ __forceinline__ void pow2_butterflies(C2 (&v)[E], const RowCtx<C2, G2>& c, const C2* __restrict__ twp,
+template <typename C2, bool INV, int E, int R>
+__device__ __forceinline__ void pow2_butterflies(C2 (&v)[E], const RowCtx<C2>& c, const C2* __restrict__ twp,
                                                  int L) {
 #pragma unroll
   for (int q = 0; q < E / R; ++q) {
@@ -285,10 +254,10 @@ __device__ __forceinline__ void pow2_butterflies(C2 (&v)[E], const RowCtx<C2, G2
 
 // Outputs of a pass: out[j L R + s L + k] = y_s, to the shared buffer or (last pass, L =
 // N/R) to the destination row, scaled by 1/N for the inverse transform.
-template <typename C2, bool INV, int E, int R, int PS, typename G2>
-__device__ __forceinline__ void pow2_store(C2 (&v)[E], const RowCtx<C2, G2>& c, int L, int lgL, bool last) {
+template <typename C2, bool INV, int E, int R, int PS>
+__device__ __forceinline__ void pow2_store(C2 (&v)[E], const RowCtx<C2>& c, int L, int lgL, bool last) {
   using Re = decltype(v[0].x);
-  const Re scale = INV ? inv_len<Re>(c.N) : (Re)1;
+  const Re scale = INV ? (Re)1 / (Re)c.N : (Re)1;
 #pragma unroll
   for (int q = 0; q < E / R; ++q) {
     const int t = c.tr + q * c.TR;
@@ -303,10 +272,7 @@ __device__ __forceinline__ void pow2_store(C2 (&v)[E], const RowCtx<C2, G2>& c, 
             y.x = y.x * scale;
             y.y = y.y * scale;
           }
-          c.o[idx] = to_global(y);
-          if constexpr (std::is_same<C2, dw2>::value) {
-            if (c.odw) c.odw[idx] = make_float4(y.x.hi, y.x.lo, y.y.hi, y.y.lo);
-          }
+          c.o[idx] = y;
         }
       } else {
         c.buf[padded<PS>(idx)] = v[q * R + s2];
@@ -315,8 +281,8 @@ __device__ __forceinline__ void pow2_store(C2 (&v)[E], const RowCtx<C2, G2>& c, 
   }
 }
 
-template <typename C2, bool INV, int E, int R, int PS, typename G2>
-__device__ __forceinline__ void pow2_pass(C2 (&v)[E], const RowCtx<C2, G2>& c, const C2* __restrict__ twp, int L,
+template <typename C2, bool INV, int E, int R, int PS>
+__device__ __forceinline__ void pow2_pass(C2 (&v)[E], const RowCtx<C2>& c, const C2* __restrict__ twp, int L,
                                           int lgL, bool last) {
   pow2_butterflies<C2, INV, E, R>(v, c, twp, L);
   pow2_store<C2, INV, E, R, PS>(v, c, L, lgL, last);
@@ -325,16 +291,15 @@ __device__ __forceinline__ void pow2_pass(C2 (&v)[E], const RowCtx<C2, G2>& c, c
 // Double rows: one CTA of 256 threads transforms 256 E / N rows (N <= 2048: E = 8; N = 4096,
 // 8192: one row with E = 16, 32).  Float rows take k_fft_pow2_tma below.
 template <typename R, bool INV, int E>
-__global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R>(E)) k_fft_pow2(const typename GlobalOf<R>::T* __restrict__ in,
-                                                          typename GlobalOf<R>::T* __restrict__ out,
+__global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R>(E)) k_fft_pow2(const typename Vec2<R>::T* __restrict__ in,
+                                                          typename Vec2<R>::T* __restrict__ out,
                                                           const typename Vec2<R>::T* __restrict__ twp,
                                                           RowCombine rc, int N, int lgN, int rows,
                                                           int rows_per_comp) {
   using C2 = typename Vec2<R>::T;
-  using G2 = typename GlobalOf<R>::T;
   constexpr int PS = sizeof(R) == 4 ? 4 : 3;   // one pad element per 128 bytes
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  RowCtx<C2, G2> c;
+  RowCtx<C2> c;
   c.N = N;
   c.TR = N / E;
   const int lr = threadIdx.x / c.TR;
@@ -350,10 +315,6 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R>(E)) k_fft_pow2(co
   c.b = sb >= 0 ? in + ((size_t)sb * rows_per_comp + rr) * N : nullptr;
   row_coefs<R>(rc, comp, c.ca, c.cb, c.ka, c.kb, c.ua, c.ub);
   c.o = out + (size_t)rrow * N;
-  c.odw = nullptr;
-  if constexpr (std::is_same<C2, dw2>::value) {
-    if (rc.out_dw) c.odw = reinterpret_cast<float4*>(rc.out_dw) + (size_t)rrow * N;
-  }
   C2 v[E];
   const int n8 = lgN / 3, rem = lgN - 3 * n8;   // n8 >= 1 radix-8 passes, then radix 2^rem
   pow2_load_global<C2, E>(v, c);
@@ -554,10 +515,6 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R>(E)) k_fft_blue(
   c.b = sb >= 0 ? in + ((size_t)sb * rows_per_comp + rr) * N : nullptr;
   row_coefs<R>(rc, comp, c.ca, c.cb, c.ka, c.kb, c.ua, c.ub);
   c.o = out + (size_t)rrow * N;
-  c.odw = nullptr;
-  if constexpr (std::is_same<C2, dw2>::value) {
-    if (rc.out_dw) c.odw = reinterpret_cast<float4*>(rc.out_dw) + (size_t)rrow * N;
-  }
   C2 v[E];
   const int n8 = lgM / 3, rem = lgM - 3 * n8;
   // forward FFT_M of the chirped, zero-padded row; every pass ends in the shared buffer
@@ -853,6 +810,7 @@ pic_status fft_configure_device() {
   PIC_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lock(mu);
   if (dev >= 0 && dev < 64 && done[dev]) return PIC_OK;
+  if (const pic_status st = fft_fix_configure_device()) return st;
   PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
@@ -864,13 +822,9 @@ pic_status fft_configure_device() {
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2_tma<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_tma_smem(1024)));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<double, false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4608 * 16));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<double, true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4608 * 16));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<dw, false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4608 * 16));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<dw, true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4608 * 16));
   // float64 rows of 8192 (one row per CTA, 32 values per thread): 8192 + 1024 padded doubles
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<double, false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 9216 * 16));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<double, true, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 9216 * 16));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<dw, false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 9216 * 16));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2<dw, true, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 9216 * 16));
   // Bluestein rows of length M = 8192 (float) / 4096 (double)
   PIC_CUDA(cudaFuncSetAttribute(k_fft_blue<float, false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8704 * 8));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_blue<float, true, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8704 * 8));
@@ -892,8 +846,7 @@ void launch_pow2(Sim* s, int N, const void* in, void* out, const void* twp, cons
   const int rpc = kFftThreads / (N / E);
   const size_t smem = (size_t)rpc * (N + (N >> PS)) * sizeof(C2);
   const int grid = (rows + rpc - 1) / rpc;
-  using G2 = typename GlobalOf<R>::T;
-  k_fft_pow2<R, INV, E><<<grid, kFftThreads, smem, s->stream>>>((const G2*)in, (G2*)out, (const C2*)twp, rc, N,
+  k_fft_pow2<R, INV, E><<<grid, kFftThreads, smem, s->stream>>>((const C2*)in, (C2*)out, (const C2*)twp, rc, N,
                                                                 lgN, rows, rows_per_comp);
 }
 
@@ -973,6 +926,7 @@ static void finish_row_combine(RowCombine& rc) {
 }
 
 pic_status launch_fft_rows(Sim* s, const void* in, void* out, const RowCombine& rc_in, bool inverse) {
+  if (fft_fix_active(s)) return launch_fft_fix(s, in, out, rc_in, inverse);
   RowCombine rc = rc_in;
   finish_row_combine(rc);
   const pic_config& c = s->cfg;
@@ -986,14 +940,10 @@ pic_status launch_fft_rows(Sim* s, const void* in, void* out, const RowCombine& 
                    : launch_bluestein<float, false>(s, in, out, rc, rows, rows_per_comp);
   }
   if (fft_is_pow2(c.Nz)) {
-    if (c.precision == PIC_FP64 && s->dht_path == PIC_DHT_F64_GEMM) {   // IEEE float64 throughout
+    if (c.precision == PIC_FP64) {
       const void* twp = s->at<double2>(s->lay.twp);
       if (inverse) launch_pow2_e<double, true>(s, c.Nz, in, out, twp, rc, rows, rows_per_comp);
       else launch_pow2_e<double, false>(s, c.Nz, in, out, twp, rc, rows, rows_per_comp);
-    } else if (c.precision == PIC_FP64) {   // double-word butterflies on the float32 units
-      const void* twp = s->at<dw2>(s->lay.twp_dw);
-      if (inverse) launch_pow2_e<dw, true>(s, c.Nz, in, out, twp, rc, rows, rows_per_comp);
-      else launch_pow2_e<dw, false>(s, c.Nz, in, out, twp, rc, rows, rows_per_comp);
     } else {
       const void* twp = s->at<float2>(s->lay.twp_f);
       if (inverse) launch_pow2_tma<true>(s, c.Nz, in, out, twp, rc, rows_per_comp);

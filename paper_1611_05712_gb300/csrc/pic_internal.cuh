@@ -36,7 +36,7 @@ struct Layout {
   size_t kperp, binv, mfwd, svd_w, svd_v, svd_d;                // DHT tables and scratch
   size_t kzmod, tz, tr, coef;                                    // PSATD tables
   size_t twp;        // per-pass twiddle tables of the row FFT (radix-8 or mixed-radix plan)
-  size_t twp_dw;     // the same as double words (hi, lo float pairs), FP64 form
+  size_t twp_fx;     // the same in fixed point (FP64 form, fft_fix.cu)
   // FP64 form with power-of-two Nz (0 otherwise): E, B as double words, [6][Nm][Nr][Nz]
   // float4 (re.hi, re.lo, im.hi, im.lo), written beside E, B by the inverse row FFT and read
   // by the gather
@@ -183,12 +183,17 @@ struct RowCombine {
   // float copies for the float rows (no float64 conversions in those kernels)
   int8_t kindA[6], kindB[6], unitA[6], unitB[6];
   float fcaRe[6], fcaIm[6], fcbRe[6], fcbIm[6];
-  // optional second destination of the double-word rows (power-of-two FP64 rows): the
-  // outputs as float4 (re.hi, re.lo, im.hi, im.lo) in the layout of `out`; null for none
+  // optional second destination of the fixed-point FP64 rows: the outputs as double words,
+  // float4 (re.hi, re.lo, im.hi, im.lo) in the layout of `out`; null for none
   void* out_dw;
 };
 pic_status launch_fft_rows(Sim* s, const void* in, void* out, const RowCombine& rc, bool inverse);
-// The double-word copy of E, B is kept (FP64 form, power-of-two rows in double words).
+// FP64 rows of 7-smooth length in block fixed point (fft_fix.cu)
+bool fft_fix_active(const Sim* s);      // taken unless PIC_DHT_F64_GEMM asks for IEEE rows
+pic_status fft_fix_configure_device();
+pic_status launch_fft_fix_setup(Sim* s);   // twiddles (after those of launch_setup_twiddles)
+pic_status launch_fft_fix(Sim* s, const void* in, void* out, const RowCombine& rc, bool inverse);
+// The double-word copy of E, B is kept (FP64 form, power-of-two rows, not PIC_DHT_F64_GEMM).
 bool eb_dw_active(const Sim* s);
 pic_status refresh_eb_dw(Sim* s);       // rebuild it from E, B after a write of those
 pic_status fft_configure_device();      // once per device, before any FFT launch

@@ -649,9 +649,8 @@ pic_status launch_setup_twiddles(Sim* s) {
   const size_t n2 = 2 * (size_t)s->cfg.Nz;
   if (s->cfg.precision != PIC_FP64) {
     k_to_float<<<conv_grid(n2), 256, 0, s->stream>>>(s->at<double>(s->lay.twp), s->at<float>(s->lay.twp_f), n2);
-  } else {   // double words for the FP64 rows: hi = float(x), lo = float(x - hi)
-    k_to_double_word<<<conv_grid(n2), 256, 0, s->stream>>>(s->at<double>(s->lay.twp), s->at<float2>(s->lay.twp_dw),
-                                                           n2);
+  } else {
+    return launch_fft_fix_setup(s);
   }
   PIC_LAUNCHED(s);
   return PIC_OK;
