@@ -51,13 +51,69 @@ GridGeom geom_of(const Sim* s) {
 
 constexpr double kInvC2 = 1.0 / (kC * kC);   // gamma from u without a float64 division
 
-// r, cos(theta), sin(theta) of (x, y) from one reciprocal square root (CUDA's rsqrt, within
-// one ulp): with q = x^2 + y^2, r = q rsqrt(q) and (cos, sin) = (x, y) rsqrt(q), within about
-// two ulps, without a square root and a division.  The axis (q = 0) takes theta = 0.
+// The FP64 particle kernels are bound by the float64 unit (2 lanes a clock and SM), on which
+// comparisons, minima, roundings and conversions of float64 values run as well as sums and
+// products.  The helpers below keep all but the arithmetic itself on the integer units.
+__device__ __forceinline__ bool is_zero(double x) {
+  return (((unsigned)__double2hiint(x) & 0x7fffffffu) | (unsigned)__double2loint(x)) == 0u;
+}
+__device__ __forceinline__ bool is_finite(double x) { return (~__double2hiint(x) & 0x7ff00000) != 0; }
+// a >= b for b > 0 (positive float64 order like their bits; a negative a is below them)
+__device__ __forceinline__ bool at_least(double a, double b) { return __double_as_longlong(a) >= __double_as_longlong(b); }
+__device__ __forceinline__ bool below_zero(double x) { return __double2hiint(x) < 0 && !is_zero(x); }
+
+// x with an exponent field of e (x positive and normal), and the float32 nearest below it.
+__device__ __forceinline__ double with_exponent(double x, int e) {
+  return __hiloint2double((__double2hiint(x) & 0xfffff) | (e << 20), __double2loint(x));
+}
+__device__ __forceinline__ float cut_to_float(double x) {   // 1 <= x < 4
+  const int hi = __double2hiint(x);
+  return __int_as_float(((hi - (896 << 20)) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double widen_float(float f) {   // normal, positive
+  const int b = __float_as_int(f);
+  return __hiloint2double((b >> 3) + (896 << 20), b << 29);
+}
+
+// 1/sqrt(x), x > 0, within about one ulp: the float32 unit's approximation (2^-22) and one step of
+// third order, y + y (e/2 + 3 e^2/8) with e = 1 - x y^2 (error 5 e^3/16 < 2^-64): 5 float64
+// operations.  x is scaled to [1, 4) by an even power of two; zero, subnormal, infinite and NaN x
+// take CUDA's function.
+__device__ __forceinline__ double inv_sqrt(double x) {
+  const int e = __double2hiint(x) >> 20;
+  if ((unsigned)(e - 1) >= 2046u) return rsqrt(x);   // also any negative x
+  const int k = (e - 1023) >> 1;                     // 4^k <= x < 4^(k+1)
+  const double xs = with_exponent(x, e - 2 * k);
+  float f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(cut_to_float(xs)));
+  const double y = widen_float(f);
+  const double r = __fma_rn(-__dmul_rn(xs, y), y, 1.0);
+  const double z = __fma_rn(y, __dmul_rn(r, __fma_rn(r, 0.375, 0.5)), y);
+  return __hiloint2double(__double2hiint(z) - k * (1 << 20), __double2loint(z));
+}
+
+// 2/d for d >= 1, within about one ulp: the float32 unit's reciprocal (2^-23) and one step of
+// third order, y + y (e + e^2), e = 1 - d y: 3 float64 operations where a division is a long
+// sequence.
+__device__ __forceinline__ double two_over(double d) {
+  const int e = __double2hiint(d) >> 20;
+  if ((unsigned)(e - 1023) >= 1000u) return 2.0 / d;
+  const double ds = with_exponent(d, 1023);          // d 2^-(e - 1023), in [1, 2)
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(cut_to_float(ds)));
+  const double y = widen_float(f);
+  const double r = __fma_rn(-ds, y, 1.0);
+  const double z = __fma_rn(y, __fma_rn(r, r, r), y);
+  return __hiloint2double(__double2hiint(z) + (1024 - e) * (1 << 20), __double2loint(z));
+}
+
+// r, cos(theta), sin(theta) of (x, y) from one reciprocal square root: with q = x^2 + y^2,
+// r = q / sqrt(q) and (cos, sin) = (x, y) / sqrt(q), within about two ulps, without a square root
+// and a division.  The axis (q = 0) takes theta = 0.
 __device__ __forceinline__ void polar(double x, double y, double& r, double& c, double& s) {
   const double r2 = __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y));
-  if (r2 > 0.0) {
-    const double ir = rsqrt(r2);
+  if (!is_zero(r2)) {
+    const double ir = inv_sqrt(r2);
     r = r2 * ir; c = x * ir; s = y * ir;
   } else {
     r = 0.0; c = 1.0; s = 0.0;
@@ -79,27 +135,42 @@ __device__ __forceinline__ double div_rn(double x, double d, double inv_d) {
   return __fma_rn(__fma_rn(-q, d, x), inv_d, q);
 }
 
+// floor(u) and u - floor(u), |u| < 2^31: a sum with 1.5 2^52 rounded down leaves floor(u) in the
+// low word (three float64 additions, no rounding and conversion instructions).
+__device__ __forceinline__ int floor_frac(double u, double& frac) {
+  constexpr double kM = 6755399441055744.0;
+  const double t = __dadd_rd(u, kM);
+  frac = __dsub_rn(u, __dsub_rn(t, kM));
+  return __double2loint(t);
+}
+
 __device__ __forceinline__ Stencil stencil(const GridGeom& g, double z, double r) {
   Stencil st;
-  double u = div_rn(z, g.dz, g.inv_dz);
-  double fi = floor(u);
-  double sz = u - fi;
-  long long i0 = (long long)fi;
-  if (i0 < 0 || i0 >= g.Nz) {   // z outside [0, L): wrap (the push keeps z inside)
-    i0 %= g.Nz;
+  // z / dz stays correctly rounded (one ulp of it is ~Nz ulps of a weight); r / dr (r < R)
+  // as a product with 1/dr
+  const double u = div_rn(z, g.dz, g.inv_dz), v = r * g.inv_dr - 0.5;
+  double sz, t;
+  if (((__double2hiint(u) >> 20) & 0x7ff) < 1023 + 30 && ((__double2hiint(v) >> 20) & 0x7ff) < 1023 + 30) {
+    st.i0 = floor_frac(u, sz);
+    st.j0 = floor_frac(v, t);
+    if ((unsigned)st.i0 >= (unsigned)g.Nz) {   // z outside [0, L): wrap (the push keeps z inside)
+      st.i0 %= g.Nz;
+      if (st.i0 < 0) st.i0 += g.Nz;
+    }
+  } else {   // far outside the box
+    const double fi = floor(u), fj = floor(v);
+    sz = u - fi;
+    t = v - fj;
+    long long i0 = (long long)fi % g.Nz;
     if (i0 < 0) i0 += g.Nz;
+    st.i0 = (int)i0;
+    st.j0 = (int)fmin(fmax(fj, -1.0), (double)g.Nr);
   }
-  st.i0 = (int)i0;
+  // r >= 0 gives j0 >= -1; beyond the last node every weight is dropped anyway
+  st.j0 = min(max(st.j0, -1), g.Nr);
   st.i1 = st.i0 + 1 == g.Nz ? 0 : st.i0 + 1;
   st.wz0 = 1.0 - sz;
   st.wz1 = sz;
-  // z / dz stays correctly rounded (one ulp of it is ~Nz ulps of a weight); r / dr (r < R)
-  // as a product with 1/dr
-  double v = r * g.inv_dr - 0.5;
-  double fj = floor(v);
-  double t = v - fj;
-  // r >= 0 gives fj >= -1; beyond the last node every weight is dropped anyway
-  st.j0 = (int)fmin(fmax(fj, -1.0), (double)g.Nr);
   st.wr0 = 1.0 - t;
   st.wr1 = t;
   return st;
@@ -233,6 +304,39 @@ __device__ __forceinline__ void count_inactive(int32_t* count, int key, bool ina
   if (inactive && (threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(count + key, __popc(m));
 }
 
+// floor(u) when u, off by a relative 2^-50 at most, lies so far from the cell boundaries that the
+// exact quotient has the same floor (u < 2^20); else -1.
+__device__ __forceinline__ int clear_floor(double u) {
+  double frac;
+  const int i = floor_frac(u, frac);
+  // 2^-28 <= frac < 1 - 2^-20 by the high words
+  const int f = __double2hiint(frac);
+  return f >= (1023 - 28) * (1 << 20) && f < 0x3feffffe ? i : -1;
+}
+
+// Cell key iz Nr + ir with iz = floor(z / dz), ir = floor(sqrt(x x + y y) / dr) of the rounded
+// sum, root and quotients.  Nearly every particle lies clear of the cell boundaries, where
+// products with 1/dz, 1/dr and an approximate root decide; the others take the exact sequence.
+__device__ __forceinline__ int cell_key(const GridGeom& g, double x, double y, double z, int32_t* err) {
+  const double r2 = __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y));
+  const double uz = z * g.inv_dz;
+  if (is_finite(r2) && !is_zero(r2) && __double2hiint(uz) >= 0 && __double2hiint(uz) < (1023 + 20) << 20) {
+    const double ur = (r2 * inv_sqrt(r2)) * g.inv_dr;
+    if (__double2hiint(ur) < (1023 + 20) << 20) {
+      const int iz = clear_floor(uz), ir = clear_floor(ur);
+      if (iz >= 0 && ir >= 0) return min(iz, g.Nz - 1) * g.Nr + min(ir, g.Nr - 1);
+    }
+  }
+  double fz = floor(div_rn(z, g.dz, g.inv_dz)), fr = floor(div_rn(sqrt(r2), g.dr, g.inv_dr));
+  if (!(fz == fz) || !(fr == fr) || isinf(fz) || isinf(fr)) {
+    atomicOr(err, kErrNumeric);
+    fz = 0.0; fr = 0.0;
+  }
+  const int iz = (int)fmin(fmax(fz, 0.0), (double)(g.Nz - 1));
+  const int ir = (int)fmin(fmax(fr, 0.0), (double)(g.Nr - 1));
+  return iz * g.Nr + ir;
+}
+
 // WIN (moving window on): inactive particles take the tail keys.
 template <bool WIN>
 __global__ void k_keys(const Parts p, int64_t np, GridGeom g, int32_t* keys, int32_t* count,
@@ -248,16 +352,7 @@ __global__ void k_keys(const Parts p, int64_t np, GridGeom g, int32_t* keys, int
         continue;
       }
     }
-    double x = p.x[i], y = p.y[i], z = p.z[i];
-    double r = sqrt(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)));
-    double fz = floor(div_rn(z, g.dz, g.inv_dz)), fr = floor(div_rn(r, g.dr, g.inv_dr));
-    if (!(fz == fz) || !(fr == fr) || isinf(fz) || isinf(fr)) {
-      atomicOr(err, kErrNumeric);
-      fz = 0.0; fr = 0.0;
-    }
-    int iz = (int)fmin(fmax(fz, 0.0), (double)(g.Nz - 1));
-    int ir = (int)fmin(fmax(fr, 0.0), (double)(g.Nr - 1));
-    int key = iz * g.Nr + ir;
+    const int key = cell_key(g, p.x[i], p.y[i], p.z[i], err);
     keys[i] = key;
     atomicAdd(count + key, 1);
   }
@@ -477,11 +572,20 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     rad[dj] = keep ? (dj ? st.wr1 : st.wr0) * (invV[jn[dj]] * qw) : 0.0;
   }
   const double vr = c * vx + s * vy, vt = c * vy - s * vx;
+  double pr[kMaxModes - 1], pi[kMaxModes - 1];   // e^{+i m theta}, m = 1 ..
+  pr[0] = c;
+  pi[0] = s;
+#pragma unroll
+  for (int m = 1; m < kMaxModes - 1; ++m) {
+    if (m + 1 >= g.Nm) break;
+    pr[m] = pr[m - 1] * c - pi[m - 1] * s;
+    pi[m] = pr[m - 1] * s + pi[m - 1] * c;
+  }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int node = (q + rot) & 3, dz = node >> 1, dj = node & 1;
     const double gq = (dz ? st.wz1 : st.wz0) * (dj ? rad[1] : rad[0]);
-    if (gq == 0.0) continue;
+    if (is_zero(gq)) continue;
     const size_t o = (size_t)(dj ? jn[1] : jn[0]) * g.Nz + (dz ? st.i1 : st.i0);
     const bool fold = ghost && dj == 0;   // the ghost node: fold signs apply
     double gr = 0.0, gt = 0.0, gz = 0.0;
@@ -497,24 +601,21 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
       atomicAdd(reinterpret_cast<double*>(a.J + g.G + o), flip_sign(gt, fold));
       atomicAdd(reinterpret_cast<double*>(a.J + 2 * g.G + o), gz);
     }
-    double pr = c, pi = s;   // e^{+i m theta}
-    for (int m = 1; m < g.Nm; ++m) {
+#pragma unroll
+    for (int m = 1; m < kMaxModes; ++m) {
+      if (m >= g.Nm) break;
       const bool negS = fold && (m & 1), negV = fold && !(m & 1);
       const size_t om = (size_t)m * RZ + o;
+      const double er = pr[m - 1], ei = pi[m - 1];
       if (do_rho) {
         const double v = flip_sign(gq, negS);
-        dep2(a.rho + om, v * pr, v * pi);
+        dep2(a.rho + om, v * er, v * ei);
       }
       if (do_J) {
         const double jr = flip_sign(gr, negV), jt = flip_sign(gt, negV), jz = flip_sign(gz, negS);
-        dep2(a.J + om, jr * pr, jr * pi);
-        dep2(a.J + g.G + om, jt * pr, jt * pi);
-        dep2(a.J + 2 * g.G + om, jz * pr, jz * pi);
-      }
-      if (m + 1 < g.Nm) {
-        const double nr = pr * c - pi * s, ni = pr * s + pi * c;
-        pr = nr;
-        pi = ni;
+        dep2(a.J + om, jr * er, jr * ei);
+        dep2(a.J + g.G + om, jt * er, jt * ei);
+        dep2(a.J + 2 * g.G + om, jz * er, jz * ei);
       }
     }
   }
@@ -538,13 +639,13 @@ __global__ void k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a, cons
     double vx = 0.0, vy = 0.0, vz = 0.0;
     if (do_J) {
       const double ux = p.ux[i], uy = p.uy[i], uz = p.uz[i];
-      const double ig = rsqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
+      const double ig = inv_sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
       vx = ux * ig; vy = uy * ig; vz = uz * ig;
     }
     const double wt = p.w[i];
-    if (wt == 0.0) continue;   // inactive particles add nothing
+    if (is_zero(wt)) continue;   // inactive particles add nothing
     const double x = p.x[i], y = p.y[i], z = p.z[i];
-    if (!isfinite(x) || !isfinite(y) || !isfinite(z)) { atomicOr(err, kErrNumeric); continue; }
+    if (!is_finite(x) || !is_finite(y) || !is_finite(z)) { atomicOr(err, kErrNumeric); continue; }
     deposit_one(g, a, invV, x, y, z, wt, vx, vy, vz, do_rho, do_J);
   }
 }
@@ -566,8 +667,14 @@ __device__ __forceinline__ void win_mark(const WinArgs& wa, int32_t id, int64_t 
 
 // WIN: moving window on (removal behind the back edge); the plain instance has none of it.
 // DWG: gather from the double-word copy of E, B (gather_dw) instead of the float64 grids.
+// Bound by the float64 unit: about 225 operations a particle at two modes are left of 295 once
+// comparisons, roundings and conversions run on the integer units, roots and the quotient of the
+// push take 5 and 3 operations and the cross products are fused.  Three CTAs per SM at 80
+// registers hide its latency better than two at 128: at 1.35 M particles and two modes 846 ->
+// 752 us with two CTAs, 703 us with three; leaving out all atomics gains 20 us more, all
+// deposits 345 us.
 template <bool WIN, bool DWG>
-__global__ void __launch_bounds__(256, 2) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
+__global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
                               const double2* __restrict__ B, const float4* __restrict__ EBdw, double k,
                               double dt, DepArgs dep, const double* invV, int fuse, int32_t* err,
                               WinArgs wa) {
@@ -575,9 +682,9 @@ __global__ void __launch_bounds__(256, 2) k_gather_push(Parts p, int64_t np, Gri
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double w = p.w[i];
-    if (w == 0.0) continue;   // inactive (moving window): neither pushed nor moved
+    if (is_zero(w)) continue;   // inactive (moving window): neither pushed nor moved
     double x = p.x[i], y = p.y[i], z = p.z[i];
-    if (!isfinite(x) || !isfinite(y) || !isfinite(z)) { atomicOr(err, kErrNumeric); continue; }
+    if (!is_finite(x) || !is_finite(y) || !is_finite(z)) { atomicOr(err, kErrNumeric); continue; }
     const double z_old = z;
     double ux = p.ux[i], uy = p.uy[i], uz = p.uz[i];
     double r, c, s;
@@ -621,37 +728,38 @@ __global__ void __launch_bounds__(256, 2) k_gather_push(Parts p, int64_t np, Gri
     }
     const double Ex = F[0] * c - F[1] * s, Ey = F[0] * s + F[1] * c, Ez = F[2];
     const double Bx = F[3] * c - F[4] * s, By = F[3] * s + F[4] * c, Bz = F[5];
-    // Boris with k = q dt / (2 m) (from the host); 1/gamma^- once for the three t
+    // Boris with k = q dt / (2 m) (from the host); 1/gamma^- once for the three t; the cross
+    // products as chains of fused multiply-adds
     const double umx = ux + k * Ex, umy = uy + k * Ey, umz = uz + k * Ez;
-    const double igm = rsqrt(1.0 + (umx * umx + umy * umy + umz * umz) * kInvC2);
-    const double kb = k * igm;
+    const double kb = k * inv_sqrt(1.0 + (umx * umx + umy * umy + umz * umz) * kInvC2);
     const double tx = kb * Bx, ty = kb * By, tz = kb * Bz;
-    const double upx = umx + (umy * tz - umz * ty);
-    const double upy = umy + (umz * tx - umx * tz);
-    const double upz = umz + (umx * ty - umy * tx);
-    const double f = 2.0 / (1.0 + tx * tx + ty * ty + tz * tz);
+    const double upx = fma(-umz, ty, fma(umy, tz, umx));
+    const double upy = fma(-umx, tz, fma(umz, tx, umy));
+    const double upz = fma(-umy, tx, fma(umx, ty, umz));
+    const double f = two_over(1.0 + tx * tx + ty * ty + tz * tz);
     const double sx = f * tx, sy = f * ty, sz = f * tz;
-    ux = umx + (upy * sz - upz * sy) + k * Ex;
-    uy = umy + (upz * sx - upx * sz) + k * Ey;
-    uz = umz + (upx * sy - upy * sx) + k * Ez;
-    const double ig = rsqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
+    ux = fma(k, Ex, fma(-upz, sy, fma(upy, sz, umx)));
+    uy = fma(k, Ey, fma(-upx, sz, fma(upz, sx, umy)));
+    uz = fma(k, Ez, fma(-upy, sx, fma(upx, sy, umz)));
+    const double ig = inv_sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
     const double vx = ux * ig, vy = uy * ig, vz = uz * ig;
     const double hdt = 0.5 * dt;
-    x = __dadd_rn(x, __dmul_rn(hdt, vx));   // no FMA: one ulp of z is ~L/dz ulps of a weight
-    y = __dadd_rn(y, __dmul_rn(hdt, vy));
-    z = __dadd_rn(z, __dmul_rn(hdt, vz));
-    if (z >= g.L) z -= g.L;
-    if (z < 0.0) z += g.L;
+    const double hx = __dmul_rn(hdt, vx), hy = __dmul_rn(hdt, vy), hz = __dmul_rn(hdt, vz);
+    x = __dadd_rn(x, hx);   // no FMA: one ulp of z is ~L/dz ulps of a weight
+    y = __dadd_rn(y, hy);
+    z = __dadd_rn(z, hz);
+    if (at_least(z, g.L)) z -= g.L;
+    if (below_zero(z)) z += g.L;
     if (fuse) deposit_one(g, dep, invV, x, y, z, w, vx, vy, vz, false, true);
-    x = __dadd_rn(x, __dmul_rn(hdt, vx));   // no FMA: one ulp of z is ~L/dz ulps of a weight
-    y = __dadd_rn(y, __dmul_rn(hdt, vy));
-    z = __dadd_rn(z, __dmul_rn(hdt, vz));
-    if (z >= g.L) z -= g.L;
-    if (z < 0.0) z += g.L;
+    x = __dadd_rn(x, hx);
+    y = __dadd_rn(y, hy);
+    z = __dadd_rn(z, hz);
+    if (at_least(z, g.L)) z -= g.L;
+    if (below_zero(z)) z += g.L;
     // one polar decomposition at x^{n+1} serves the wall and the rho deposit
     double r1, c1, s1;
     polar(x, y, r1, c1, s1);
-    if (r1 >= g.R) {   // specular reflection (rare: the particle crossed the wall)
+    if (at_least(r1, g.R)) {   // specular reflection (rare: the particle crossed the wall)
       const double fr = (2.0 * g.R - r1) / r1;
       const double ur = ux * c1 + uy * s1;
       ux = ux - 2.0 * ur * c1;
@@ -666,10 +774,9 @@ __global__ void __launch_bounds__(256, 2) k_gather_push(Parts p, int64_t np, Gri
     if (WIN) {
       // window coordinate after the step: ((z^n - back) mod L) + 2 half moves - s dz
       double zo = z_old - wa.back_z;
-      if (zo < 0.0) zo += g.L;
-      const double d = __dmul_rn(hdt, vz);
-      const double zn = __dsub_rn(__dadd_rn(__dadd_rn(zo, d), d), wa.shift ? g.dz : 0.0);
-      if (zn < 0.0) {   // left through the back edge: inactive from now on
+      if (below_zero(zo)) zo += g.L;
+      const double zn = __dsub_rn(__dadd_rn(__dadd_rn(zo, hz), hz), wa.shift ? g.dz : 0.0);
+      if (below_zero(zn)) {   // left through the back edge: inactive from now on
         p.w[i] = 0.0;
         ux = 0.0; uy = 0.0; uz = 0.0;
         win_mark(wa, p.id[i], i);
