@@ -36,8 +36,8 @@
  * PIC_ERR_TIMEOUT.
  *
  * Asynchrony: all calls enqueue work on the handle's stream and return, except
- * pic_init (synchronises during set-up: after each sweep of the Hankel matrices' Jacobi SVD
- * and at its end), pic_diagnostics, pic_read_particles,
+ * pic_init (synchronises during set-up: after the Hankel matrices' pseudo-inverses and at its
+ * end), pic_diagnostics, pic_read_particles,
  * pic_copy_buffer with a host destination, and pic_sync.
  */
 #ifndef PSATD_RZ_H
@@ -129,8 +129,8 @@ pic_status pic_required_bytes(const pic_config* cfg, size_t* bytes);
 
 /* Validate cfg, carve the workspace and run the setup stage on the GPU (FP64, once):
  * Bessel zeros alpha_{m,n} (Newton from McMahon's expansion), Hankel matrices
- * B_p = J_p(k_{m,n} r_j), their pseudo-inverses (one-sided Jacobi SVD, singular values
- * <= 1e-3 sigma_max dropped), [k_z]_p (Eq. finite_difference / [k_z]) and the PSATD
+ * B_p = J_p(k_{m,n} r_j), their pseudo-inverses (singular values <= 1e-3 sigma_max
+ * dropped), [k_z]_p (Eq. finite_difference / [k_z]) and the PSATD
  * coefficient tables C, S/K, (1-C)/K^2, ... (Eq. psatd-eqE/eqB with [k_z]).
  * workspace: device pointer, >= pic_required_bytes, 256-byte aligned.  stream: a
  * cudaStream_t (NULL = legacy default stream).  Fields start at zero, no particles.

@@ -103,6 +103,7 @@ Layout make_layout(const pic_config& c) {
   L.svd_w = take((size_t)c.Nm * 3 * Nr2 * 8);
   L.svd_v = take((size_t)c.Nm * 3 * Nr2 * 8);
   L.svd_d = take((size_t)c.Nm * 3 * c.Nr * 8);
+  L.pinv = take(pinv_scratch_bytes(c));
   L.kzmod = take((size_t)c.Nz * 8);
   L.tz = take((size_t)c.Nz * 8);
   L.tr = take((size_t)c.Nm * c.Nr * 8);

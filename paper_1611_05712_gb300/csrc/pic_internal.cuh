@@ -33,7 +33,7 @@ enum : int32_t { kErrNumeric = 1, kErrTimeout = 2, kErrRange = 4 };
 // Device workspace layout, all offsets in bytes from the workspace base.
 struct Layout {
   size_t E, B, Eh, Bh, dep, srch, tmp, rho_prev_h, rho_ion;   // grids
-  size_t kperp, binv, mfwd, svd_w, svd_v, svd_d;                // DHT tables and scratch
+  size_t kperp, binv, mfwd, svd_w, svd_v, svd_d, pinv;          // DHT tables and scratch
   size_t kzmod, tz, tr, coef;                                    // PSATD tables
   size_t twp;        // per-pass twiddle tables of the row FFT (radix-8 or mixed-radix plan)
   size_t twp_fx;     // the same in fixed point (FP64 form, fft_fix.cu)
@@ -169,6 +169,12 @@ pic_status cuda_status(cudaError_t e, const char* what);
 pic_status launch_setup_hankel(Sim* s);          // zeros, B_p, pinv(B_p)
 pic_status launch_setup_tables(Sim* s, int32_t order_p);   // [k_z]_p and PSATD coefficients
 pic_status launch_setup_twiddles(Sim* s);
+// ---- launchers (pinv.cu) ----
+// mfwd <- pinv(binv) of every matrix up to a Newton-Schulz step, and the check of that step;
+// *bad is raised where the SVD has to be taken instead.
+size_t pinv_scratch_bytes(const pic_config& c);
+pic_status launch_pinv(Sim* s, int32_t* bad);
+pic_status launch_pinv_check(Sim* s, const double* before, const double* after, int32_t* bad);
 pic_status convert_hankel_tables(Sim* s);                    // mixed form: float/split copies
 pic_status convert_psatd_tables(Sim* s);
 

@@ -2,8 +2,9 @@
 //   * Bessel zeros alpha_{m,n} and k_{m,n} = alpha_{m,n}/R (quasi-cylindrical Hankel grid,
 //     section "Finite order pseudo-spectral solvers": Hankel transform along r);
 //   * inverse Hankel matrices B_p[j][n] = J_p(k_{m,n} r_j), p = m-1, m, m+1;
-//   * forward matrices M_p = pinv(B_p) by a one-sided (Hestenes) Jacobi SVD, dropping
-//     singular values <= 1e-3 sigma_max (B_{m-1} lacks the k=0 Dini function);
+//   * forward matrices M_p = pinv(B_p), dropping singular values <= 1e-3 sigma_max (B_{m-1}
+//     lacks the k=0 Dini function): by elimination with the dropped directions projected out
+//     (pinv.cu), or by the one-sided (Hestenes) Jacobi SVD here where its checks ask for it;
 //   * [k_z]_p from Eq. finite_difference and the [k_z] equation, and the PSATD
 //     coefficient tables of Eq. psatd-eqE / psatd-eqB with k_z -> [k_z]_p;
 //   * the FFT twiddle table.
@@ -503,18 +504,12 @@ pic_status convert_psatd_tables(Sim* s) {
   return PIC_OK;
 }
 
-pic_status launch_setup_hankel(Sim* s) {
+// mfwd = pinv(B) by the Jacobi SVD of all matrices.
+static pic_status pinv_by_svd(Sim* s) {
   const pic_config& c = s->cfg;
   const int Nm = c.Nm, Nr = c.Nr;
-  double* kperp = s->at<double>(s->lay.kperp);
-  double* binv = s->at<double>(s->lay.binv);
-  int32_t* err = s->at<int32_t>(s->lay.err);
-  k_bessel_zeros<<<blocks_for((size_t)Nm * Nr, 128), 128, 0, s->stream>>>(kperp, Nm, Nr, Nr * c.dr, err);
-  PIC_LAUNCHED(s);
-  size_t tot = (size_t)Nm * 3 * Nr * Nr;
-  k_hankel_inv<<<(int)std::min<size_t>(blocks_for(tot, 256), 152 * 16), 256, 0, s->stream>>>(
-      binv, kperp, Nm, Nr, c.dr);
-  PIC_LAUNCHED(s);
+  const double* binv = s->at<double>(s->lay.binv);
+  double* mfwd = s->at<double>(s->lay.mfwd);
   double* wt = s->at<double>(s->lay.svd_w);
   double* vt = s->at<double>(s->lay.svd_v);
   double* d = s->at<double>(s->lay.svd_d);
@@ -546,13 +541,19 @@ pic_status launch_setup_hankel(Sim* s) {
   }
   k_svd_values<<<nmat, kSvdThreads, 0, s->stream>>>(wt, d, Nr);
   PIC_LAUNCHED(s);
-  double* mfwd = s->at<double>(s->lay.mfwd);
   dim3 g(blocks_for(Nr, 32), blocks_for(Nr, 32), Nm * 3);
   k_pinv_assemble<<<g, dim3(32, 32), 0, s->stream>>>(wt, vt, d, mfwd, Nr);
   PIC_LAUNCHED(s);
-  // One Newton-Schulz step M <- M (2I - B M): the Jacobi result is accurate to about
-  // tol * cond; the step squares the error on the kept subspace, while components along
-  // dropped directions (of size ~tol |M|) only double.  W and V are free again here.
+  return PIC_OK;
+}
+
+// One Newton-Schulz step M <- M (2I - B M): the step squares the error on the kept subspace,
+// while components along dropped directions only double.  W and V are scratch.  bad (may be
+// null) is raised if the step was not a small one.
+static pic_status newton_schulz(Sim* s, int32_t* bad) {
+  const int Nm = s->cfg.Nm, Nr = s->cfg.Nr;
+  double *binv = s->at<double>(s->lay.binv), *mfwd = s->at<double>(s->lay.mfwd);
+  double *wt = s->at<double>(s->lay.svd_w), *vt = s->at<double>(s->lay.svd_v);
   const size_t Nr2 = (size_t)Nr * Nr;
   DhtBatch bm{}, mt{};
   for (int k = 0; k < Nm * 3; ++k) {
@@ -566,7 +567,37 @@ pic_status launch_setup_hankel(Sim* s) {
       wt, Nm * 3, Nr);                                  // W = 2I - W
   PIC_LAUNCHED(s);
   if ((st = launch_gemm_f64(s, mt, Nr)) != PIC_OK) return st;   // V = M W
+  if (bad && (st = launch_pinv_check(s, mfwd, vt, bad)) != PIC_OK) return st;
   PIC_CUDA(cudaMemcpyAsync(mfwd, vt, Nm * 3 * Nr2 * sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
+  return PIC_OK;
+}
+
+pic_status launch_setup_hankel(Sim* s) {
+  const pic_config& c = s->cfg;
+  const int Nm = c.Nm, Nr = c.Nr;
+  double* kperp = s->at<double>(s->lay.kperp);
+  double* binv = s->at<double>(s->lay.binv);
+  int32_t* err = s->at<int32_t>(s->lay.err);
+  k_bessel_zeros<<<blocks_for((size_t)Nm * Nr, 128), 128, 0, s->stream>>>(kperp, Nm, Nr, Nr * c.dr, err);
+  PIC_LAUNCHED(s);
+  size_t tot = (size_t)Nm * 3 * Nr * Nr;
+  k_hankel_inv<<<(int)std::min<size_t>(blocks_for(tot, 256), 152 * 16), 256, 0, s->stream>>>(
+      binv, kperp, Nm, Nr, c.dr);
+  PIC_LAUNCHED(s);
+  // pseudo-inverses by elimination (pinv.cu), checked; by the SVD where the checks ask for it.
+  // The sort's counter words are free during set-up: one records the checks
+  int32_t* bad = s->at<int32_t>(s->lay.big_count);
+  int32_t h = 0;
+  PIC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int32_t), s->stream));
+  pic_status st = launch_pinv(s, bad);
+  if (st != PIC_OK) return st;
+  if ((st = newton_schulz(s, bad)) != PIC_OK) return st;
+  PIC_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+  PIC_CUDA(cudaStreamSynchronize(s->stream));
+  if (h != 0) {
+    if ((st = pinv_by_svd(s)) != PIC_OK) return st;
+    if ((st = newton_schulz(s, nullptr)) != PIC_OK) return st;
+  }
   k_tr_table<<<blocks_for((size_t)Nm * Nr, 128), 128, 0, s->stream>>>(s->at<double>(s->lay.tr), kperp,
                                                                        Nm * Nr, c.dr);
   PIC_LAUNCHED(s);
