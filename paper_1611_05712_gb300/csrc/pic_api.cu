@@ -699,6 +699,34 @@ pic_status pic_selftest_wait_timeout(pic_sim* sim, int32_t max_polls) {
   return launch_wait_selftest(s, (uint32_t)max_polls);
 }
 
+namespace {
+
+// Array k of a particle set on its way in or out: the staging area (mixed forms) or the
+// particles' own array.
+double* stage_array(const Sim* s, int k) {
+  return s->cfg.precision != PIC_FP64 ? s->at<double>(s->lay.stage64) + (size_t)k * (size_t)s->cfg.np_capacity
+                                      : s->at<double>(s->lay.part[s->cur][k]);
+}
+
+// Whether a kernel of this handle may work on the caller's device arrays themselves: every array
+// given lies on the workspace's own device, apart from the workspace, and is aligned to its
+// elements (a copy by the runtime needs none of this).
+bool readable_in_place(const Sim* s, const double* const* soa, const int32_t* id) {
+  cudaPointerAttributes own, a;
+  if (cudaPointerGetAttributes(&own, s->ws) != cudaSuccess) { cudaGetLastError(); return false; }
+  for (int k = 0; k < 8; ++k) {
+    const void* p = k < 7 ? (soa ? static_cast<const void*>(soa[k]) : nullptr) : static_cast<const void*>(id);
+    if (!p) continue;
+    const char* c = static_cast<const char*>(p);
+    if (reinterpret_cast<uintptr_t>(p) % (k < 7 ? 8 : 4) || (c >= s->ws && c < s->ws + s->ws_bytes)) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (a.type != cudaMemoryTypeDevice || a.device != own.device) return false;
+  }
+  return true;
+}
+
+}  // namespace
+
 pic_status pic_write_particles(pic_sim* sim, const double* const soa[7], const int32_t* id, int64_t n,
                                int32_t on_host) {
   Sim* s = reinterpret_cast<Sim*>(sim);
@@ -711,21 +739,22 @@ pic_status pic_write_particles(pic_sim* sim, const double* const soa[7], const i
   if (n > 0 && (!soa || !id)) { set_error("particle pointers are NULL"); return PIC_ERR_ARG; }
   const cudaMemcpyKind kind = on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const bool mixed = s->cfg.precision != PIC_FP64;
-  const size_t cap = (size_t)s->cfg.np_capacity;
-  for (int k = 0; k < 7 && n > 0; ++k) {
+  for (int k = 0; k < 7 && n > 0; ++k)
     if (!soa[k]) { set_error("particle array %d is NULL", k); return PIC_ERR_ARG; }
-    char* dst = mixed ? s->ws + s->lay.stage64 + k * cap * 8 : s->ws + s->lay.part[s->cur][k];
-    PIC_CUDA(cudaMemcpyAsync(dst, soa[k], n * 8, kind, s->stream));
-  }
-  if (n > 0) {
-    // ids go straight to their final place (FP64 form) or to the perm scratch (mixed form)
-    char* dst = mixed ? s->ws + s->lay.perm_tmp : s->ws + s->lay.pid[s->cur];
-    PIC_CUDA(cudaMemcpyAsync(dst, id, n * 4, kind, s->stream));
+  const bool direct = n > 0 && !on_host && readable_in_place(s, soa, id);
+  double* staged[7];
+  for (int k = 0; k < 7; ++k) staged[k] = stage_array(s, k);
+  int32_t* ids = mixed ? s->at<int32_t>(s->lay.perm_tmp) : s->at<int32_t>(s->lay.pid[s->cur]);
+  if (n > 0 && !direct) {   // straight to their final place (FP64 form) or to the staging area
+    for (int k = 0; k < 7; ++k) PIC_CUDA(cudaMemcpyAsync(staged[k], soa[k], n * 8, kind, s->stream));
+    PIC_CUDA(cudaMemcpyAsync(ids, id, n * 4, kind, s->stream));
   }
   s->np = n;
   s->win.on = 0;   // new particles: the window's template and ids no longer apply
-  if (mixed) {
-    pic_status st = launch_particles_in(s, s->at<int32_t>(s->lay.perm_tmp), n);
+  if (direct || mixed) {
+    const double* from[7];
+    for (int k = 0; k < 7; ++k) from[k] = direct ? soa[k] : staged[k];
+    pic_status st = launch_particles_in(s, from, direct ? id : ids, n);
     if (st != PIC_OK) return st;
   }
   if (on_host) PIC_CUDA(cudaStreamSynchronize(s->stream));
@@ -798,15 +827,9 @@ pic_status pic_take_particles(pic_sim* sim) {
   const int32_t* ids = reinterpret_cast<const int32_t*>(g.buf + (size_t)7 * st * 8);
   s->np = n;
   s->win.on = 0;   // new particles: the window's template and ids no longer apply
-  if (s->cfg.precision != PIC_FP64) {
-    pic_status r = launch_particles_in(s, ids, n, src, st);
-    if (r != PIC_OK) return r;
-  } else if (n > 0) {
-    for (int k = 0; k < 7; ++k)
-      PIC_CUDA(cudaMemcpyAsync(s->ws + s->lay.part[s->cur][k], src + (size_t)k * st, (size_t)n * 8,
-                               cudaMemcpyDeviceToDevice, s->stream));
-    PIC_CUDA(cudaMemcpyAsync(s->ws + s->lay.pid[s->cur], ids, (size_t)n * 4, cudaMemcpyDeviceToDevice, s->stream));
-  }
+  const double* from[7];
+  for (int k = 0; k < 7; ++k) from[k] = src + (size_t)k * st;
+  if (const pic_status r = launch_particles_in(s, from, ids, n)) return r;
   PIC_CUDA(cudaEventRecord(g.free_, s->stream));
   return PIC_OK;
 }
@@ -818,19 +841,20 @@ pic_status pic_read_particles(pic_sim* sim, double* const soa[7], int32_t* id, i
   if (n < 0 || n > s->np) { set_error("n=%lld exceeds the %lld particles held", (long long)n, (long long)s->np); return PIC_ERR_ARG; }
   const cudaMemcpyKind kind = on_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   const bool mixed = s->cfg.precision != PIC_FP64;
-  const size_t cap = (size_t)s->cfg.np_capacity;
+  if (n > 0 && !on_host && readable_in_place(s, soa, id)) {
+    pic_status st = launch_particles_out(s, soa, id, n);
+    return st != PIC_OK ? st : pic_sync(sim);
+  }
+  double* staged[7];
+  for (int k = 0; k < 7; ++k) staged[k] = stage_array(s, k);
+  int32_t* ids = mixed ? s->at<int32_t>(s->lay.perm_tmp) : s->at<int32_t>(s->lay.pid[s->cur]);
   if (mixed) {
-    pic_status st = launch_particles_out(s, s->at<int32_t>(s->lay.perm_tmp), n);
+    pic_status st = launch_particles_out(s, staged, ids, n);
     if (st != PIC_OK) return st;
   }
-  for (int k = 0; k < 7 && n > 0; ++k) {
-    const char* src = mixed ? s->ws + s->lay.stage64 + k * cap * 8 : s->ws + s->lay.part[s->cur][k];
-    if (soa && soa[k]) PIC_CUDA(cudaMemcpyAsync(soa[k], src, n * 8, kind, s->stream));
-  }
-  if (id && n > 0) {
-    const char* src = mixed ? s->ws + s->lay.perm_tmp : s->ws + s->lay.pid[s->cur];
-    PIC_CUDA(cudaMemcpyAsync(id, src, n * 4, kind, s->stream));
-  }
+  for (int k = 0; k < 7 && n > 0; ++k)
+    if (soa && soa[k]) PIC_CUDA(cudaMemcpyAsync(soa[k], staged[k], n * 8, kind, s->stream));
+  if (id && n > 0) PIC_CUDA(cudaMemcpyAsync(id, ids, n * 4, kind, s->stream));
   return pic_sync(sim);
 }
 

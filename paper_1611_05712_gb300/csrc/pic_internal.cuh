@@ -265,11 +265,10 @@ pic_status launch_diag(Sim* s, int32_t id_lo, int32_t id_hi, pic_diag* out, doub
                        int32_t max_slices);
 pic_status build_inv_volume(Sim* s);                        // once, at init
 pic_status particles_configure_device();                    // once per device
-// mixed: float64 SoA (7 arrays of `stride` doubles from src; stage64 with the capacity as
-// stride when src is null) -> FP32
-pic_status launch_particles_in(Sim* s, const int32_t* id_dev, int64_t n, const double* src = nullptr,
-                               int64_t stride = 0);
-pic_status launch_particles_out(Sim* s, int32_t* id_dev, int64_t n);        // mixed: FP32 -> stage64
+// The current particles <- device arrays v[0..6] (x y z ux uy uz w, float64) and id, and back
+// (null arrays are left out); the mixed forms convert.  The arrays are aligned to their elements.
+pic_status launch_particles_in(Sim* s, const double* const v[7], const int32_t* id, int64_t n);
+pic_status launch_particles_out(Sim* s, double* const v[7], int32_t* id, int64_t n);
 
 // ---- moving window (particles.cu: particle side; window.cu: field side) ----
 // Byte offsets of the window workspace for a template of n_tpl particles.
