@@ -546,98 +546,162 @@ __device__ __forceinline__ void dep2(double2* p, double re, double im) {
   atomicAdd(d + 1, im);
 }
 
-// Deposit of one particle: rho (do_rho) and/or J (do_J) with weight e^{+i m theta} per mode,
-// linear weights; the ghost node r = -dr/2 of the axis cell is node 0 seen across the axis
-// (fold sign (-1)^m for rho and J_z, (-1)^{m+1} for J_r and J_theta) and node Nr is dropped.
-// The mode-independent products are formed once per node: g = q w w_z w_r / V_j and g v_k;
-// each mode multiplies them by its phase (mode 0: real, so its imaginary parts, which would
-// receive zeros, are left alone).  Lanes visit the 4 nodes in an order rotated by the lane
-// index, so that lanes of one cell (same nodes) add to different nodes in one instruction.
-// deposit_at takes the particle's radius and azimuth (r, cos, sin) already formed.
+// Products of the deposits on the integer units.  A particle adds 12 (2 Nm - 1) + 4 (2 Nm - 1)
+// products of five factors to the grids, half of the push kernel's float64 operations when the
+// float64 unit forms them.  Here a factor is its 53-bit mantissa as a 62-bit integer in two
+// halves of 31 bits, its exponent and its sign: a product takes three wide multiply-adds and four
+// shifts (the low halves' product is left out), keeps 57 bits or more over the chain of four
+// (each product may start one bit lower), and is rounded to float64 once at the end, where
+// the float64 products rounded each time.
+struct Sf {
+  unsigned h, l;   // mantissa h 2^31 + l, in [2^61, 2^62) for a converted number; 0 for zero
+  int e;           // biased exponent: the value is mantissa 2^(e - 1023 - 61)
+  unsigned s;      // sign in bit 31
+};
+
+__device__ __forceinline__ Sf sf_from(double x) {   // subnormal x count as zero
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  Sf r;
+  r.h = e ? (((hi & 0xfffffu) | 0x100000u) << 10) | (lo >> 22) : 0u;
+  r.l = e ? (lo << 9) & 0x7fffffffu : 0u;
+  r.e = e ? e : -100000;   // products with zero fall out of the exponent range (sf_far)
+  r.s = hi & 0x80000000u;
+  return r;
+}
+
+__device__ __forceinline__ unsigned long long sf_mantissa(const Sf& a) { return ((unsigned long long)a.h << 31) | a.l; }
+
+__device__ __forceinline__ unsigned long long sf_product(const Sf& a, const Sf& b) {   // mantissas' product >> 62
+  const unsigned long long t = (unsigned long long)a.h * b.l + (unsigned long long)a.l * b.h;   // below 2^63
+  return (unsigned long long)a.h * b.h + (t >> 31);
+}
+
+__device__ __forceinline__ Sf operator*(const Sf& a, const Sf& b) {
+  const unsigned long long p = sf_product(a, b);
+  return Sf{(unsigned)(p >> 31), (unsigned)p & 0x7fffffffu, a.e + b.e - 1022, a.s ^ b.s};
+}
+
+// sf_double of zero and of results outside the normal range (NaN factors: e is large).
+__device__ __noinline__ double sf_far(unsigned long long m, int e, unsigned s) {
+  if (m == 0ull) return 0.0;
+  if (e > 3000) return __longlong_as_double(0x7ff8000000000000ll);
+  const double v = ldexp((double)m, e - 1023 - 61);
+  return s ? -v : v;
+}
+
+// Mantissa m (0, or 2^56 <= m < 2^62) with biased exponent e and sign s as a float64.
+__device__ __forceinline__ double sf_double(unsigned long long m, int e, unsigned s) {
+  const int lz = __clz((int)(unsigned)(m >> 32));
+  const unsigned long long r = ((m << (lz - 1)) + 0x200u) >> 10;   // 53 bits, rounded (2^53 carries on)
+  const int ex = e + 2 - lz;                                       // exponent field of the result
+  if ((unsigned)(ex - 1) >= 2044u) return sf_far(m, e, s);
+  return __hiloint2double((int)((unsigned)(r >> 32) + ((unsigned)(ex - 1) << 20) | s), (int)(unsigned)r);
+}
+
+// Deposit of one particle: rho (RHO) and/or J (CUR) with weight e^{+i m theta} per mode, linear
+// weights; the ghost node r = -dr/2 of the axis cell is node 0 seen across the axis (fold sign
+// (-1)^m for rho and J_z, (-1)^{m+1} for J_r and J_theta) and node Nr is dropped.  The
+// mode-independent products are formed once per node: g = q w w_z w_r / V_j and g v_k; each mode
+// multiplies them by its phase (mode 0: real, so its imaginary parts, which would receive zeros,
+// are left alone).  Lanes visit the 4 nodes in an order rotated by the lane index, so that lanes
+// of one cell (same nodes) add to different nodes in one instruction.  deposit_at takes the
+// particle's radius and azimuth (r, cos, sin) already formed; MODES: modes it has room for.
+template <int MODES, bool RHO, bool CUR>
 __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* invV, double r,
-                           double c, double s, double z, double w, double vx, double vy, double vz,
-                           bool do_rho, bool do_J) {
+                           double c, double s, double z, double w, double vx, double vy, double vz) {
   const Stencil st = stencil(g, z, r);
   const size_t RZ = (size_t)g.Nr * g.Nz;
   const int rot = threadIdx.x & 3;
   const bool ghost = st.j0 < 0;
   const double qw = a.q * w;
-  double rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (0 for the dropped node Nr)
-  int jn[2];       // their grid rows (the ghost node j = -1 is row 0)
+  Sf rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (0 for the dropped node Nr)
+  int jn[2];   // their grid rows (the ghost node j = -1 is row 0)
 #pragma unroll
   for (int dj = 0; dj < 2; ++dj) {
     const int j = st.j0 + dj;
     const bool keep = j < g.Nr;
     jn[dj] = (j < 0 || !keep) ? 0 : j;
-    rad[dj] = keep ? (dj ? st.wr1 : st.wr0) * (invV[jn[dj]] * qw) : 0.0;
+    rad[dj] = sf_from(keep ? (dj ? st.wr1 : st.wr0) : 0.0) * sf_from(invV[jn[dj]] * qw);
   }
-  const double vr = c * vx + s * vy, vt = c * vy - s * vx;
-  double pr[kMaxModes - 1], pi[kMaxModes - 1];   // e^{+i m theta}, m = 1 ..
-  pr[0] = c;
-  pi[0] = s;
-#pragma unroll
-  for (int m = 1; m < kMaxModes - 1; ++m) {
-    if (m + 1 >= g.Nm) break;
-    pr[m] = pr[m - 1] * c - pi[m - 1] * s;
-    pi[m] = pr[m - 1] * s + pi[m - 1] * c;
+  Sf v[3], pr[MODES > 1 ? MODES - 1 : 1], pi[MODES > 1 ? MODES - 1 : 1];   // velocity; e^{+i m theta}, m = 1 ..
+  if (CUR) {
+    v[0] = sf_from(c * vx + s * vy);
+    v[1] = sf_from(c * vy - s * vx);
+    v[2] = sf_from(vz);
   }
+  // a NaN or an infinity among the factors makes every product of the particle NaN
+  if (!is_finite(qw) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
+  {
+    double er = c, ei = s;
 #pragma unroll
+    for (int m = 1; m < MODES; ++m) {
+      if (m >= g.Nm) break;
+      pr[m - 1] = sf_from(er);
+      pi[m - 1] = sf_from(ei);
+      const double nr = er * c - ei * s;
+      ei = er * s + ei * c;
+      er = nr;
+    }
+  }
+  const Sf z0 = sf_from(st.wz0), z1 = sf_from(st.wz1);
+#pragma unroll 1
   for (int q = 0; q < 4; ++q) {
     const int node = (q + rot) & 3, dz = node >> 1, dj = node & 1;
-    const double gq = (dz ? st.wz1 : st.wz0) * (dj ? rad[1] : rad[0]);
-    if (is_zero(gq)) continue;
+    const Sf gq = (dj ? rad[1] : rad[0]) * (dz ? z1 : z0);
+    if ((gq.h | gq.l) == 0u) continue;
     const size_t o = (size_t)(dj ? jn[1] : jn[0]) * g.Nz + (dz ? st.i1 : st.i0);
-    const bool fold = ghost && dj == 0;   // the ghost node: fold signs apply
-    double gr = 0.0, gt = 0.0, gz = 0.0;
-    if (do_J) {
-      gr = gq * vr;
-      gt = gq * vt;
-      gz = gq * vz;
-    }
-    // mode 0: fold +1 for rho and J_z, -1 for J_r and J_theta
-    if (do_rho) atomicAdd(reinterpret_cast<double*>(a.rho + o), gq);
-    if (do_J) {
-      atomicAdd(reinterpret_cast<double*>(a.J + o), flip_sign(gr, fold));
-      atomicAdd(reinterpret_cast<double*>(a.J + g.G + o), flip_sign(gt, fold));
-      atomicAdd(reinterpret_cast<double*>(a.J + 2 * g.G + o), gz);
-    }
+    const unsigned fold = ghost && dj == 0 ? 0x80000000u : 0u;   // the ghost node: fold signs apply
+    auto add = [&](double2* grid, size_t at, const Sf& f, unsigned flip) {   // mode 0
+      atomicAdd(reinterpret_cast<double*>(grid + at), sf_double(sf_mantissa(f), f.e, f.s ^ flip));
+    };
+    auto add_phase = [&](double2* grid, size_t at, const Sf& f, int m, unsigned flip) {
+      const Sf &er = pr[m - 1], &ei = pi[m - 1];
+      dep2(grid + at, sf_double(sf_product(f, er), f.e + er.e - 1022, f.s ^ er.s ^ flip),
+           sf_double(sf_product(f, ei), f.e + ei.e - 1022, f.s ^ ei.s ^ flip));
+    };
+    if (RHO) {   // fold +1 in mode 0, (-1)^m
+      add(a.rho, o, gq, 0u);
 #pragma unroll
-    for (int m = 1; m < kMaxModes; ++m) {
-      if (m >= g.Nm) break;
-      const bool negS = fold && (m & 1), negV = fold && !(m & 1);
-      const size_t om = (size_t)m * RZ + o;
-      const double er = pr[m - 1], ei = pi[m - 1];
-      if (do_rho) {
-        const double v = flip_sign(gq, negS);
-        dep2(a.rho + om, v * er, v * ei);
+      for (int m = 1; m < MODES; ++m) {
+        if (m >= g.Nm) break;
+        add_phase(a.rho, (size_t)m * RZ + o, gq, m, (m & 1) ? fold : 0u);
       }
-      if (do_J) {
-        const double jr = flip_sign(gr, negV), jt = flip_sign(gt, negV), jz = flip_sign(gz, negS);
-        dep2(a.J + om, jr * er, jr * ei);
-        dep2(a.J + g.G + om, jt * er, jt * ei);
-        dep2(a.J + 2 * g.G + om, jz * er, jz * ei);
+    }
+    if (CUR) {   // J_r and J_theta: fold -1 in mode 0, (-1)^{m+1}; J_z as rho
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const Sf gk = gq * v[k];
+        double2* J = a.J + k * g.G;
+        add(J, o, gk, k < 2 ? fold : 0u);
+#pragma unroll
+        for (int m = 1; m < MODES; ++m) {
+          if (m >= g.Nm) break;
+          add_phase(J, (size_t)m * RZ + o, gk, m, ((m & 1) != 0) == (k == 2) ? fold : 0u);
+        }
       }
     }
   }
 }
 
+template <int MODES, bool RHO, bool CUR>
 __device__ __forceinline__ void deposit_one(const GridGeom& g, const DepArgs& a, const double* invV,
                                             double x, double y, double z, double w, double vx,
-                                            double vy, double vz, bool do_rho, bool do_J) {
+                                            double vy, double vz) {
   double r, c, s;
   polar(x, y, r, c, s);
-  deposit_at(g, a, invV, r, c, s, z, w, vx, vy, vz, do_rho, do_J);
+  deposit_at<MODES, RHO, CUR>(g, a, invV, r, c, s, z, w, vx, vy, vz);
 }
 
-__global__ void k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a, const double* invV,
-                          int32_t* err) {
-  const bool do_rho = a.rho != nullptr, do_J = a.J != nullptr;
+template <int MODES, bool RHO, bool CUR>
+__global__ void __launch_bounds__(256, 3) k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a,
+                                                    const double* invV, int32_t* err) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t id = p.id[i];
     if (id < a.id_lo || id >= a.id_hi) continue;
     double vx = 0.0, vy = 0.0, vz = 0.0;
-    if (do_J) {
+    if (CUR) {
       const double ux = p.ux[i], uy = p.uy[i], uz = p.uz[i];
       const double ig = inv_sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
       vx = ux * ig; vy = uy * ig; vz = uz * ig;
@@ -646,7 +710,7 @@ __global__ void k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a, cons
     if (is_zero(wt)) continue;   // inactive particles add nothing
     const double x = p.x[i], y = p.y[i], z = p.z[i];
     if (!is_finite(x) || !is_finite(y) || !is_finite(z)) { atomicOr(err, kErrNumeric); continue; }
-    deposit_one(g, a, invV, x, y, z, wt, vx, vy, vz, do_rho, do_J);
+    deposit_one<MODES, RHO, CUR>(g, a, invV, x, y, z, wt, vx, vy, vz);
   }
 }
 
@@ -667,13 +731,14 @@ __device__ __forceinline__ void win_mark(const WinArgs& wa, int32_t id, int64_t 
 
 // WIN: moving window on (removal behind the back edge); the plain instance has none of it.
 // DWG: gather from the double-word copy of E, B (gather_dw) instead of the float64 grids.
-// Bound by the float64 unit: about 225 operations a particle at two modes are left of 295 once
-// comparisons, roundings and conversions run on the integer units, roots and the quotient of the
-// push take 5 and 3 operations and the cross products are fused.  Three CTAs per SM at 80
-// registers hide its latency better than two at 128: at 1.35 M particles and two modes 846 ->
-// 752 us with two CTAs, 703 us with three; leaving out all atomics gains 20 us more, all
-// deposits 345 us.
-template <bool WIN, bool DWG>
+// Bound by the float64 unit (63 % busy) and by latency at 24 warps per SM: about 165 operations a
+// particle are left of 295 at two modes once comparisons, roundings and conversions run on the
+// integer units, roots and the quotient of the push take 5 and 3 operations, the cross products
+// are fused and the deposits' products are formed by the integer units (Sf).  Three CTAs per SM
+// at 80 registers hide its latency better than two at 128.  1.35 M particles, two modes: 846 us
+// at first, 703 with the float64 unit's own work reduced, 593 with the integer products; 1.64 M
+// particles, three modes: 959, 793, 764.  Leaving out all atomics would gain 20 us.
+template <int MODES, bool WIN, bool DWG>
 __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
                               const double2* __restrict__ B, const float4* __restrict__ EBdw, double k,
                               double dt, DepArgs dep, const double* invV, int fuse, int32_t* err,
@@ -750,7 +815,7 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     z = __dadd_rn(z, hz);
     if (at_least(z, g.L)) z -= g.L;
     if (below_zero(z)) z += g.L;
-    if (fuse) deposit_one(g, dep, invV, x, y, z, w, vx, vy, vz, false, true);
+    if (fuse) deposit_one<MODES, false, true>(g, dep, invV, x, y, z, w, vx, vy, vz);
     x = __dadd_rn(x, hx);
     y = __dadd_rn(y, hy);
     z = __dadd_rn(z, hz);
@@ -770,7 +835,7 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     }
     // rho^{n+1} at x^{n+1} (without the moving window; with it the deposit stage runs after
     // the injection)
-    if (!WIN && dep.rho) deposit_at(g, dep, invV, r1, c1, s1, z, w, 0.0, 0.0, 0.0, true, false);
+    if (!WIN && dep.rho) deposit_at<MODES, true, false>(g, dep, invV, r1, c1, s1, z, w, 0.0, 0.0, 0.0);
     if (WIN) {
       // window coordinate after the step: ((z^n - back) mod L) + 2 half moves - s dz
       double zo = z_old - wa.back_z;
@@ -2265,6 +2330,15 @@ __global__ void __launch_bounds__(kWinBlock) k_win_inject_f32(int32_t* flag, int
 
 bool is_mixed(const Sim* s) { return s->cfg.precision != PIC_FP64; }
 
+// Kernel instances of the FP64 form by the modes they have room for.
+template <int MODES> auto deposit_kernel64(const DepArgs& a) {
+  return !a.J ? k_deposit<MODES, true, false> : !a.rho ? k_deposit<MODES, false, true> : k_deposit<MODES, true, true>;
+}
+template <int MODES> auto push_kernel64(bool win, bool dwg) {
+  return win ? (dwg ? k_gather_push<MODES, true, true> : k_gather_push<MODES, true, false>)
+             : (dwg ? k_gather_push<MODES, false, true> : k_gather_push<MODES, false, false>);
+}
+
 // Kernel instances of the mixed form by mode count (1..kMaxModes).
 using DepositKernel = void (*)(const PartsF, int64_t, GeomF, DepArgsF, const float*, int32_t*, BandArgs);
 using GatherPushKernel = void (*)(PartsF, int64_t, GeomF, const float2* __restrict__, float, float, float, float,
@@ -2439,7 +2513,9 @@ pic_status launch_deposit(Sim* s, int32_t what, int32_t id_lo, int32_t id_hi, vo
     a.J = (what & PIC_DEP_J) ? s->at<double2>(s->lay.dep) + G : nullptr;
     if (a.J) PIC_CUDA(cudaMemsetAsync(a.J, 0, 3 * G * sizeof(double2), s->stream));
     if (s->np == 0) return PIC_OK;
-    k_deposit<<<pgrid(s->np), 256, 0, s->stream>>>(parts_of(s, s->cur), s->np, geom_of(s), a, inv_volume(s), err);
+    if (!a.rho && !a.J) return PIC_OK;
+    auto* kern = s->cfg.Nm <= 2 ? deposit_kernel64<2>(a) : s->cfg.Nm == 3 ? deposit_kernel64<3>(a) : deposit_kernel64<4>(a);
+    kern<<<pgrid(s->np), 256, 0, s->stream>>>(parts_of(s, s->cur), s->np, geom_of(s), a, inv_volume(s), err);
   }
   PIC_LAUNCHED(s);
   return PIC_OK;
@@ -2505,19 +2581,13 @@ pic_status launch_gather_push(Sim* s, int32_t fuse_current, const WinArgs& wa, b
     const float4* ebdw = eb_dw_active(s) ? s->at<float4>(s->lay.ebdw) : nullptr;
     const Parts p = parts_of(s, s->cur);
     const GridGeom g = geom_of(s);
-    const int grid = pgrid(s->np);
-    if (wa.on && ebdw)
-      k_gather_push<true, true><<<grid, 256, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s),
-                                                             fuse_current, err, wa);
-    else if (wa.on)
-      k_gather_push<true, false><<<grid, 256, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s),
-                                                              fuse_current, err, wa);
-    else if (ebdw)
-      k_gather_push<false, true><<<grid, 256, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s),
-                                                              fuse_current, err, wa);
-    else
-      k_gather_push<false, false><<<grid, 256, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a,
-                                                               inv_volume(s), fuse_current, err, wa);
+    // one particle per thread: an even last wave.  Sets that leave SMs idle are spread over more,
+    // smaller CTAs (36 k particles: 38 us with 256 threads, 35 us with 128)
+    const int threads = s->np < 152 * 1024 ? 128 : 256;
+    const int grid = (int)((s->np + threads - 1) / threads);
+    const bool win = wa.on != 0, dwg = ebdw != nullptr;
+    auto* kern = c.Nm <= 2 ? push_kernel64<2>(win, dwg) : c.Nm == 3 ? push_kernel64<3>(win, dwg) : push_kernel64<4>(win, dwg);
+    kern<<<grid, threads, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s), fuse_current, err, wa);
   }
   PIC_LAUNCHED(s);
   return PIC_OK;
