@@ -11,8 +11,8 @@
 // The component combination of the quasi-cylindrical scheme is fused into the row load:
 // out = ca * inA + cb * inB, which forms J_+- = (J_r -+ i J_theta)/2 before the forward
 // transform and E_r = E_+ + E_-, E_theta = i (E_+ - E_-) before the inverse one.
+#include <algorithm>
 #include <mutex>
-#include <type_traits>
 
 #include "pic_internal.cuh"
 #include "tc_common.cuh"
@@ -207,9 +207,9 @@ __device__ __forceinline__ void pow2_load_shared(C2 (&v)[E], const RowCtx<C2>& c
 }
 
 // Twiddles w^r = w_{LR}^{rk}, r = 1 .. R-1, of butterfly k of pass (R, L).  Float rows read
-// w^1 from the table and form the other powers with at most three products each (w^2 = w w,
-// w^3 = w^2 w, w^4 = w^2 w^2, w^5 = w^4 w, w^6 = w^4 w^2, w^7 = w^4 w^3), a few float
-// roundings from the tabulated values: one table read per butterfly instead of R - 1, which
+// w^1 from the table (and w^4, w^8 beyond 8 points) and form the other powers with at most three
+// products each (w^2 = w w, w^3 = w^2 w, w^4 = w^2 w^2 up to 8 points, w^{4a+b} = w^{4a} w^b), a
+// few float roundings from the tabulated values: one to three table reads instead of R - 1, which
 // the register budget of 16 and 32 values per thread could not keep in flight.  Double rows
 // read every power: their products would run on the float64 unit, which bounds those rows.
 template <typename C2, int R>
@@ -221,12 +221,12 @@ __device__ __forceinline__ void pass_twiddles(C2 (&w)[R], const C2* __restrict__
       w[2] = cmul(w[1], w[1]);
       w[3] = cmul(w[2], w[1]);
     }
-    if constexpr (R > 4) {
-      w[4] = cmul(w[2], w[2]);
-      w[5] = cmul(w[4], w[1]);
-      w[6] = cmul(w[4], w[2]);
-      w[7] = cmul(w[4], w[3]);
-    }
+    if constexpr (R > 4) w[4] = R > 8 ? twp[L - 1 + 3 * L + k] : cmul(w[2], w[2]);
+    if constexpr (R > 8) w[8] = twp[L - 1 + 7 * L + k];
+    if constexpr (R > 12) w[12] = cmul(w[8], w[4]);
+#pragma unroll
+    for (int r = 5; r < R; ++r)
+      if (r & 3) w[r] = cmul(w[r & ~3], w[r & 3]);
   } else {
 #pragma unroll
     for (int r = 1; r < R; ++r) w[r] = twp[L - 1 + (r - 1) * L + k];
@@ -585,15 +585,20 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_ctas<R>(E)) k_fft_blue(
 }
 
 // ---- any 7-smooth length ----
-// Stockham passes of the plan's radices (8, 4, 2, 3, 5, 7 in the plan's order), one row per
-// CTA; each thread takes butterflies t, t + 256, ... of a pass and holds a butterfly's R
+// Stockham passes of the plan's radices (plan_radix), one row per CTA; each thread takes
+// butterflies t, t + blockDim, ... of a pass and holds a butterfly's R
 // values in registers.  The first pass reads the combined row straight from global memory
 // and the last pass writes the row there (L = N / R, so its butterflies store in natural
 // order); the passes between exchange values through two shared row buffers.  Twiddles as
 // in the power-of-two rows (pass_twiddles); the R-point DFTs of odd R use the symmetric
 // form y_m, y_{R-m} = v_0 + sum_s (v_s + v_{R-s}) cos(2 pi s m / R)
 // -+ i sum_s (v_s - v_{R-s}) sin(2 pi s m / R) (s = 1 .. (R-1)/2), with the cosines and
-// sines of the R-th roots of unity as constants.
+// sines of the R-th roots of unity as constants.  Float rows take products of those radices too
+// (6 to 16): the rows are bound by instructions, and every pass adds its indices, twiddles and
+// exchange to them.  The 35840 rows of 3600 points of four field cycles on 2 modes x 448 radial
+// points took 936 us in six passes of 8, 2, 3, 3, 5, 5 and take 661 us in three of 15, 15, 16
+// (80 registers), 675 us at four CTAs an SM (64 registers, about 160 bytes spilled for radices
+// 14 to 16); the 96000 shorter rows of eight grids of a parameter scan 1074, 1065 and 976 us.
 // cos(2 pi j / R) and sin(2 pi j / R), 0 <= j <= (R - 1) / 2, R = 3, 5, 7.
 __host__ __device__ constexpr double root_cos(int R, int j) {
   return j == 0 ? 1.0
@@ -644,6 +649,80 @@ template <typename C2, bool INV, int R> __device__ __forceinline__ void dft_odd(
   v[0] = y0;
 }
 
+// cos and sin of 2 pi k / R at compile time, by their power series on [-pi, pi].
+__host__ __device__ constexpr double unit_angle(int R, int k) {
+  k %= R;
+  if (2 * k > R) k -= R;
+  return 6.283185307179586476925 * k / R;
+}
+__host__ __device__ constexpr double unit_cos(int R, int k) {
+  const double x = unit_angle(R, k);
+  double t = 1.0, sum = 1.0;
+  for (int i = 1; i < 20; ++i) {
+    t *= -x * x / ((2 * i - 1) * (2 * i));
+    sum += t;
+  }
+  return sum;
+}
+__host__ __device__ constexpr double unit_sin(int R, int k) {
+  const double x = unit_angle(R, k);
+  double t = x, sum = x;
+  for (int i = 1; i < 20; ++i) {
+    t *= -x * x / ((2 * i) * (2 * i + 1));
+    sum += t;
+  }
+  return sum;
+}
+
+template <typename C2, bool INV, int R> __device__ __forceinline__ void dft_any(C2* v);
+
+// R = R1 R2 points: R2 DFTs of R1 points, their outputs turned by w_R^{n2 k1}, R1 DFTs of R2.
+template <typename C2, bool INV, int R1, int R2> __device__ __forceinline__ void dft_product(C2* v) {
+  using Re = decltype(v[0].x);
+  constexpr int R = R1 * R2;
+  C2 t[R];
+#pragma unroll
+  for (int n2 = 0; n2 < R2; ++n2) {
+    C2 u[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) u[n1] = v[R2 * n1 + n2];
+    dft_any<C2, INV, R1>(u);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) {
+      if (n2 * k1 != 0) {
+        C2 w;
+        w.x = (Re)unit_cos(R, n2 * k1);
+        w.y = INV ? (Re)unit_sin(R, n2 * k1) : -(Re)unit_sin(R, n2 * k1);
+        u[k1] = cmul(u[k1], w);
+      }
+      t[n2 * R1 + k1] = u[k1];
+    }
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < R1; ++k1) {
+    C2 u[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) u[n2] = t[n2 * R1 + k1];
+    dft_any<C2, INV, R2>(u);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) v[k1 + R1 * k2] = u[k2];
+  }
+}
+
+template <typename C2, bool INV, int R> __device__ __forceinline__ void dft_any(C2* v) {
+  if constexpr (R == 2) dft2<C2, INV>(v);
+  else if constexpr (R == 4) dft4<C2, INV>(v);
+  else if constexpr (R == 8) dft8<C2, INV>(v);
+  else if constexpr (R == 6) dft_product<C2, INV, 2, 3>(v);
+  else if constexpr (R == 9) dft_product<C2, INV, 3, 3>(v);
+  else if constexpr (R == 10) dft_product<C2, INV, 2, 5>(v);
+  else if constexpr (R == 12) dft_product<C2, INV, 4, 3>(v);
+  else if constexpr (R == 14) dft_product<C2, INV, 2, 7>(v);
+  else if constexpr (R == 15) dft_product<C2, INV, 3, 5>(v);
+  else if constexpr (R == 16) dft_product<C2, INV, 4, 4>(v);
+  else dft_odd<C2, INV, R>(v);
+}
+
 // Sources and destinations of a pass: the shared buffers, or (first pass) the combined
 // input row / (last pass) the output row scaled for the inverse transform.
 template <typename C2> struct MixedIO {
@@ -684,10 +763,7 @@ __device__ __forceinline__ void mixed_pass(const C2* __restrict__ src, C2* __res
 #pragma unroll
       for (int r = 1; r < R; ++r) v[r] = cmul(v[r], conj_if<C2, INV>(w[r]));
     }
-    if constexpr (R == 2) dft2<C2, INV>(v);
-    else if constexpr (R == 4) dft4<C2, INV>(v);
-    else if constexpr (R == 8) dft8<C2, INV>(v);
-    else dft_odd<C2, INV, R>(v);
+    dft_any<C2, INV, R>(v);
     const int base = j * L * R + k;
 #pragma unroll
     for (int s2 = 0; s2 < R; ++s2) {
@@ -706,6 +782,18 @@ __device__ __forceinline__ void mixed_pass(const C2* __restrict__ src, C2* __res
 template <typename C2, bool INV, bool FIRST, bool LAST>
 __device__ __forceinline__ void mixed_pass_r(int Rdx, const C2* src, C2* dst, const C2* __restrict__ twp,
                                              const MixedIO<C2>& io, int N, int L) {
+  if constexpr (sizeof(io.scale) == 4) {   // the float plans' products of radices
+    switch (Rdx) {
+      case 6: mixed_pass<C2, INV, 6, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 9: mixed_pass<C2, INV, 9, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 10: mixed_pass<C2, INV, 10, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 12: mixed_pass<C2, INV, 12, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 14: mixed_pass<C2, INV, 14, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 15: mixed_pass<C2, INV, 15, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 16: mixed_pass<C2, INV, 16, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      default: break;
+    }
+  }
   switch (Rdx) {
     case 2: mixed_pass<C2, INV, 2, FIRST, LAST>(src, dst, twp, io, N, L); break;
     case 3: mixed_pass<C2, INV, 3, FIRST, LAST>(src, dst, twp, io, N, L); break;
@@ -717,10 +805,11 @@ __device__ __forceinline__ void mixed_pass_r(int Rdx, const C2* src, C2* dst, co
 }
 
 template <typename R, bool INV>
-__global__ void __launch_bounds__(256) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
-                                                  typename Vec2<R>::T* __restrict__ out,
-                                                  const typename Vec2<R>::T* __restrict__ twp, RowCombine rc,
-                                                  FftPlan plan, int rows_per_comp) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
+                                                                             typename Vec2<R>::T* __restrict__ out,
+                                                                             const typename Vec2<R>::T* __restrict__ twp,
+                                                                             RowCombine rc, FftPlan plan,
+                                                                             int rows_per_comp) {
   using C2 = typename Vec2<R>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = plan.N;
@@ -736,29 +825,29 @@ __global__ void __launch_bounds__(256) k_fft_rows(const typename Vec2<R>::T* __r
   row_coefs<R>(rc, comp, io.ca, io.cb, io.ka, io.kb, io.ua, io.ub);
   io.o = out + (size_t)row * N;
   io.scale = INV ? (R)1 / (R)N : (R)1;
-  // radices packed 4 bits each (a parameter array indexed at run time would be copied to
-  // the stack)
+  // radices (less one) packed 4 bits each (a parameter array indexed at run time would be copied
+  // to the stack)
   unsigned long long radix = 0;
 #pragma unroll
-  for (int p = 0; p < kMaxRadixPasses; ++p) radix |= (unsigned long long)plan.radix[p] << (4 * p);
+  for (int p = 0; p < kMaxRadixPasses; ++p) radix |= (unsigned long long)((plan.radix[p] - 1) & 15) << (4 * p);
   const int np = plan.n_pass;
   if (np == 1) {
-    mixed_pass_r<C2, INV, true, true>((int)(radix & 15), buf0, buf1, twp, io, N, 1);
+    mixed_pass_r<C2, INV, true, true>((int)(radix & 15) + 1, buf0, buf1, twp, io, N, 1);
     return;
   }
-  mixed_pass_r<C2, INV, true, false>((int)(radix & 15), buf0, buf0, twp, io, N, 1);
+  mixed_pass_r<C2, INV, true, false>((int)(radix & 15) + 1, buf0, buf0, twp, io, N, 1);
   __syncthreads();
   C2* src = buf0;
   C2* dst = buf1;
-  int L = (int)(radix & 15);
+  int L = (int)(radix & 15) + 1;
   for (int p = 1; p < np - 1; ++p) {
-    const int Rp = (int)((radix >> (4 * p)) & 15);
+    const int Rp = (int)((radix >> (4 * p)) & 15) + 1;
     mixed_pass_r<C2, INV, false, false>(Rp, src, dst, twp, io, N, L);
     __syncthreads();
     C2* t2 = src; src = dst; dst = t2;
     L *= Rp;
   }
-  mixed_pass_r<C2, INV, false, true>((int)((radix >> (4 * (np - 1))) & 15), src, dst, twp, io, N, L);
+  mixed_pass_r<C2, INV, false, true>((int)((radix >> (4 * (np - 1))) & 15) + 1, src, dst, twp, io, N, L);
 }
 
 // ---- any other length: Bluestein's chirp-z algorithm ----
@@ -782,19 +871,60 @@ int bluestein_length(int Nz, int precision) {
   return M <= (precision == PIC_FP64 ? 4096 : 8192) ? M : 0;
 }
 
-// Factor Nz into passes of radix 8, 4, 2, 3, 5, 7 (the Stockham order is free).
-bool plan_radix(int N, int32_t* radix, int32_t* n_pass) {
-  int n = N, k = 0;
-  const int order[6] = {8, 4, 2, 3, 5, 7};
-  for (int f : order) {
-    while (n % f == 0) {
-      if (k >= kMaxRadixPasses) return false;
-      radix[k++] = f;
-      n /= f;
+namespace {
+
+// The factorisation of a 7-smooth length into the fewest radices (any needs fewer than
+// kMaxRadixPasses), in falling order, and among those the one of the smallest first radix.
+struct RadixSearch {
+  int n, r[kMaxRadixPasses];
+
+  void search(int rest, int from, RadixSearch& best) {
+    constexpr int kR[] = {16, 15, 14, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
+    if (rest == 1) {
+      if (n < best.n || (n == best.n && r[0] < best.r[0])) best = *this;
+      return;
     }
+    if (n + 1 > best.n) return;
+    for (int i = from; i < 13; ++i)
+      if (rest % kR[i] == 0) {
+        r[n++] = kR[i];
+        search(rest / kR[i], i, best);
+        --n;
+      }
+  }
+};
+
+}  // namespace
+
+// Factor Nz into passes (the Stockham order is free).  FP64 rows: radices 8, 4, 2, 3, 5, 7.
+// Float rows of lengths that are no powers of two: the fewest passes of radices up to 16 (each
+// pass costs about as many instructions for indices, twiddles and the exchange as for its
+// butterflies), and among those the smallest largest radix; the pass whose radix shares the
+// smallest power of two with the shared memory's 16 double banks comes first, since its stores
+// step by the radix (odd radices meet no bank conflicts).
+bool plan_radix(int N, int precision, int32_t* radix, int32_t* n_pass) {
+  int n = N;
+  for (int f : {2, 3, 5, 7})
+    while (n > 1 && n % f == 0) n /= f;
+  if (n != 1) return false;
+  int k = 0;
+  n = N;
+  if (precision == PIC_FP64 || (N & (N - 1)) == 0) {
+    for (int f : {8, 4, 2, 3, 5, 7})
+      while (n % f == 0) {
+        if (k >= kMaxRadixPasses) return false;
+        radix[k++] = f;
+        n /= f;
+      }
+  } else {
+    RadixSearch best{}, cur{};
+    best.n = kMaxRadixPasses;
+    cur.search(N, 0, best);
+    std::stable_sort(best.r, best.r + best.n, [](int a, int b) { return (a & -a) < (b & -b); });
+    for (; k < best.n; ++k) radix[k] = best.r[k];
   }
   *n_pass = k;
-  return n == 1;
+  return true;
 }
 
 // The shared-memory limit of the FFT kernels is raised once per device to the largest row
@@ -968,13 +1098,13 @@ pic_status launch_fft_rows(Sim* s, const void* in, void* out, const RowCombine& 
                                                                 plan, rows_per_comp);
     }
   } else {
-    if (inverse) {
-      k_fft_rows<float, true><<<rows, 256, smem, s->stream>>>((const float2*)in, (float2*)out, twf, rc,
-                                                              plan, rows_per_comp);
-    } else {
-      k_fft_rows<float, false><<<rows, 256, smem, s->stream>>>((const float2*)in, (float2*)out, twf, rc,
-                                                               plan, rows_per_comp);
-    }
+    // as many threads as share the butterflies of the smallest radix evenly, at most 256
+    int least = plan.radix[0];
+    for (int i = 1; i < plan.n_pass; ++i) least = std::min(least, plan.radix[i]);
+    const int most = c.Nz / least, turns = (most + 255) / 256;
+    const int threads = std::max(64, ((most + turns - 1) / turns + 31) / 32 * 32);
+    auto* k = inverse ? k_fft_rows<float, true> : k_fft_rows<float, false>;
+    k<<<rows, threads, smem, s->stream>>>((const float2*)in, (float2*)out, twf, rc, plan, rows_per_comp);
   }
   PIC_LAUNCHED(s);
   return PIC_OK;
