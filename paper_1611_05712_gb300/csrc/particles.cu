@@ -1124,7 +1124,15 @@ __device__ __forceinline__ float fx_value(int32_t hi, int32_t lo) {
 }
 
 // Largest |w| and radial stencil range over particles [b0, b1) (all threads of the CTA;
-// non-finite weights raise the numeric error bit and count as 0).
+// non-finite weights raise the numeric error bit and count as 0); MOMENTA: the momenta are read
+// afterwards.
+// Starts the read of *p into L2.  The particle loop reads the arrays that the statistics pass does
+// not need only after a chain of dependent loads: with their lines requested here the push of 1.35 M
+// particles (2048 x 256, 2 modes) takes 160 us where it took 165, the rho deposit of 2.2 M 62.5 us
+// where it took 66.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+template <bool MOMENTA>
 __device__ __forceinline__ ChunkStats chunk_stats(const PartsF& p, const GeomF& g, int64_t b0, int64_t b1,
                                                   ChunkStats* slot, int32_t* err) {
   if (threadIdx.x == 0) *slot = ChunkStats{0u, g.Nr, -1};
@@ -1133,6 +1141,11 @@ __device__ __forceinline__ ChunkStats chunk_stats(const PartsF& p, const GeomF& 
   int jmin = g.Nr, jmax = -1;
   for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
     float a = fabsf(p.w[i]);
+    prefetch_l2(p.iz + i); prefetch_l2(p.fz + i);
+    if (MOMENTA) {
+      prefetch_l2(p.ux + i); prefetch_l2(p.uy + i); prefetch_l2(p.uz + i);
+      prefetch_l2(p.uxl + i); prefetch_l2(p.uyl + i); prefetch_l2(p.uzl + i);
+    }
     if (!(a <= 3.0e38f)) { atomicOr(err, kErrNumeric); a = 0.f; }
     mx = fmaxf(mx, a);
     float x, y;
@@ -1184,11 +1197,11 @@ __device__ __forceinline__ BandF make_band(int32_t* smem, int iz_first, int iz_l
                ldexpf(1.f, S0)};
 }
 
-// Zero a band (all threads of the CTA).
+// Zero a band (all threads of the CTA; 16-byte stores).
 __device__ __forceinline__ void band_zero(const BandF& bd) {
   if (!bd.tile) return;
-  const int n = bd.TZ * bd.RS;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) bd.tile[k] = 0;
+  const int n = bd.TZ * bd.RS / 4;   // RS is a multiple of 8 words
+  for (int k = threadIdx.x; k < n; k += blockDim.x) reinterpret_cast<int4*>(bd.tile)[k] = make_int4(0, 0, 0, 0);
 }
 
 // Fixed-point adds of one node: rho (DO_RHO, component 0) and J (DO_J, components NC-3..NC-1).
@@ -1440,7 +1453,7 @@ __global__ void __launch_bounds__(kBandThreads, 2) k_deposit_f32(const PartsF p,
   const int64_t b1 = b0 + ba.chunk < np ? b0 + ba.chunk : np;
   BandF band{nullptr, 0, 0, 0, 0, 1, 0, 1.f, 1.f};
   if (ba.tz > 0) {
-    const ChunkStats cs = chunk_stats(p, g, b0, b1, &stats_slot, err);
+    const ChunkStats cs = chunk_stats<DO_J>(p, g, b0, b1, &stats_slot, err);
     const float qw = fabsf(a.q) * __uint_as_float(cs.wmax_bits);
     if (cs.wmax_bits != 0u)   // a chunk of inactive particles deposits nothing: no band
       band = make_band(band_smem, p.iz[b0], p.iz[b1 - 1], g, ba.tz, band_node_words(NM, NC), cs, ba.jw_max,
@@ -1505,7 +1518,7 @@ __global__ void __launch_bounds__(kBandThreads, 2) k_gather_push_f32(PartsF p, i
   const int64_t b1 = b0 + ba.chunk < np ? b0 + ba.chunk : np;
   BandF band{nullptr, 0, 0, 0, 0, 1, 0, 1.f, 1.f};
   if (fuse && ba.tz > 0) {
-    const ChunkStats cs = chunk_stats(p, g, b0, b1, &stats_slot, err);
+    const ChunkStats cs = chunk_stats<true>(p, g, b0, b1, &stats_slot, err);
     const float qw = fabsf(dep.q) * __uint_as_float(cs.wmax_bits);
     if (cs.wmax_bits != 0u)   // a chunk of inactive particles deposits nothing: no band
       band = make_band(band_smem, p.iz[b0], p.iz[b1 - 1], g, ba.tz, band_node_words(NM, NC), cs, ba.jw_max,
@@ -2373,8 +2386,8 @@ GatherPushKernel gather_push_kernel(int nm, bool win, bool rho) {
   }
 }
 
-// Shared-memory bands for the deposits: chunks of cell-sorted particles per CTA (1024, or
-// the tuned size: a power of two) and a
+// Shared-memory bands for the deposits: chunks of cell-sorted particles per CTA (at most 1024,
+// or the tuned size: a power of two) and a
 // band of ncomp components (all modes, 16 bytes per complex node) within kBandBudget, so
 // that two CTAs fit on an SM: 8 or 4 full z-rows when they fit, else 4 rows of as many r
 // nodes as fit (at least 16).  jmargin: r nodes a particle can move before it deposits.
@@ -2385,9 +2398,18 @@ struct BandPlan {
 };
 BandPlan band_plan(const Sim* s, int ncomp, int jmargin) {
   const pic_config& c = s->cfg;
-  const int64_t chunk = s->tune_chunk > 0 ? s->tune_chunk : 1024;
+  int64_t chunk = s->tune_chunk > 0 ? s->tune_chunk : 1024;
   int lg = 0;
   while ((int64_t(1) << lg) < chunk) ++lg;
+  // Up to three waves of CTAs (two per SM): chunks shortened so that the last wave is full.  Pushes
+  // of the sets of a parameter scan at 0.17, 0.8, 1.3, 1.4, 2.3, 2.5, 2.6 waves took 16.8, 67, 62,
+  // 77, 129, 262, 69 us and take 10.9, 59, 58, 78, 129, 237, 66; at 4.3 waves (2048 x 256, 2 modes)
+  // the additional bands cost more than the last wave (160 -> 167 us).
+  const int64_t slots = 2 * 152, waves = (s->np + slots * chunk - 1) / (slots * chunk);
+  if (waves >= 1 && waves <= 3) {
+    const int64_t even = ((s->np + slots * waves - 1) / (slots * waves) + 31) & ~int64_t(31);
+    chunk = std::min(chunk, std::max<int64_t>(even, 128));
+  }
   BandPlan bp{BandArgs{chunk, 0, 0, jmargin, lg}, 0};
   if (ncomp <= 0) return bp;
   // one r node of one row: re hi, re lo for every mode, im hi, im lo for the modes m >= 1,
