@@ -297,11 +297,16 @@ constexpr int kTailBins = 64;
 
 __device__ __forceinline__ int tail_key(int ncell, int64_t i) { return ncell + (int)((i >> 5) & (kTailBins - 1)); }
 
-// Warp-aggregated count of the inactive lanes of this iteration (all share one sub-bin).
-__device__ __forceinline__ void count_inactive(int32_t* count, int key, bool inactive) {
+// Counts the inactive lanes of this iteration (all share one sub-bin) with one atomic; returns an
+// inactive lane's place among the sub-bin's entries.
+__device__ __forceinline__ int32_t count_inactive(int32_t* count, int key, bool inactive) {
   const unsigned am = __activemask();
   const unsigned m = __ballot_sync(am, inactive);
-  if (inactive && (threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(count + key, __popc(m));
+  if (!inactive) return 0;
+  const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+  int32_t b = 0;
+  if (lane == leader) b = atomicAdd(count + key, __popc(m));
+  return __shfl_sync(m, b, leader) + __popc(m & ((1u << lane) - 1u));
 }
 
 // floor(u) when u, off by a relative 2^-50 at most, lies so far from the cell boundaries that the
@@ -337,24 +342,26 @@ __device__ __forceinline__ int cell_key(const GridGeom& g, double x, double y, d
   return iz * g.Nr + ir;
 }
 
-// WIN (moving window on): inactive particles take the tail keys.
+// Keys, the particles per key, and each particle's place among those of its key in the order of the
+// atomics (any order).  WIN (moving window on): inactive particles take the tail keys.
 template <bool WIN>
-__global__ void k_keys(const Parts p, int64_t np, GridGeom g, int32_t* keys, int32_t* count,
+__global__ void k_keys(const Parts p, int64_t np, GridGeom g, int32_t* keys, int32_t* count, int32_t* place,
                        int32_t* err) {
   const int ncell = g.Nz * g.Nr;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (WIN) {
       const bool inactive = p.w[i] == 0.0;
-      count_inactive(count, tail_key(ncell, i), inactive);
+      const int32_t at = count_inactive(count, tail_key(ncell, i), inactive);
       if (inactive) {
+        place[i] = at;
         keys[i] = tail_key(ncell, i);
         continue;
       }
     }
     const int key = cell_key(g, p.x[i], p.y[i], p.z[i], err);
     keys[i] = key;
-    atomicAdd(count + key, 1);
+    place[i] = atomicAdd(count + key, 1);
   }
 }
 
@@ -386,8 +393,10 @@ __device__ int32_t block_exclusive_scan(int32_t v, int32_t* total) {
   return excl;
 }
 
+// Exclusive scan within each block and the block totals; empties the list of crowded cells.
 __global__ void __launch_bounds__(kScanThreads) k_scan_local(const int32_t* count, int32_t* start,
-                                                              int32_t* blk, int n) {
+                                                              int32_t* blk, int n, int32_t* big_count) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *big_count = 0;
   const int base = blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
   int32_t v[kScanPer], sum = 0;
   for (int q = 0; q < kScanPer; ++q) {
@@ -403,127 +412,110 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_local(const int32_t* coun
   if (threadIdx.x == 0) blk[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(int32_t* blk, int nblk, int32_t* start,
-                                                               int n) {
-  // one block: exclusive scan of up to 4096 block totals
-  const int base = threadIdx.x * kScanPer;
-  int32_t v[kScanPer], sum = 0;
-  for (int q = 0; q < kScanPer; ++q) {
-    v[q] = (base + q < nblk) ? blk[base + q] : 0;
-    sum += v[q];
+// Adds to the elements of each block of the scan the totals of the blocks before it (every CTA, of a
+// quarter of a block, sums them itself: a launch of one CTA for them took 2.7 us), writes start[n],
+// and lists the cells of more than kWarpCellMax particles.
+__global__ void __launch_bounds__(256) k_scan_add(const int32_t* __restrict__ count, int32_t* __restrict__ start,
+                                                  const int32_t* __restrict__ blk, int n, int ncell,
+                                                  int32_t* __restrict__ big_list, int32_t* __restrict__ big_count) {
+  constexpr int kPer = kScanBlock / 4 / 256;
+  __shared__ int32_t warp_sums[8];
+  const int nb = blockIdx.x / 4;
+  int32_t v[kPer], c[kPer], sum = 0;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int i = blockIdx.x * (kScanBlock / 4) + q * 256 + threadIdx.x;
+    v[q] = i < n ? start[i] : 0;
+    c[q] = i < ncell ? count[i] : 0;
   }
-  int32_t tot;
-  int32_t ex = block_exclusive_scan(sum, &tot);
-  for (int q = 0; q < kScanPer; ++q) {
-    if (base + q < nblk) blk[base + q] = ex;
-    ex += v[q];
-  }
-  if (threadIdx.x == 0) start[n] = tot;
-}
-
-__global__ void k_scan_add(int32_t* start, const int32_t* blk, int n, int32_t* cursor) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    int32_t v = start[i] + blk[i / kScanBlock];
-    start[i] = v;
-    cursor[i] = v;
-  }
-}
-
-// Counting-sort scatter; the inactive lanes of a warp iteration (one sub-bin, see tail_key)
-// take their places with one atomic.
-template <bool WIN>
-__global__ void k_scatter(const int32_t* keys, int64_t np, int32_t* cursor, int32_t* tmp, int32_t ncell) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t key = keys[i];
-    if (!WIN) {
-      tmp[atomicAdd(cursor + key, 1)] = (int32_t)i;
-      continue;
-    }
-    const bool t = key >= ncell;
-    const unsigned am = __activemask();
-    const unsigned m = __ballot_sync(am, t);
-    int32_t pos;
-    if (t) {
-      const int leader = __ffs(m) - 1;
-      int32_t b = 0;
-      if (lane == leader) b = atomicAdd(cursor + key, __popc(m));
-      b = __shfl_sync(m, b, leader);
-      pos = b + __popc(m & ((1u << lane) - 1u));
-    } else {
-      pos = atomicAdd(cursor + key, 1);
-    }
-    tmp[pos] = (int32_t)i;
+  for (int b = threadIdx.x; b < nb; b += 256) sum += blk[b];
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  int32_t before = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) before += warp_sums[w];
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int i = blockIdx.x * (kScanBlock / 4) + q * 256 + threadIdx.x;
+    if (i < n) start[i] = v[q] + before;
+    if (i == n - 1) start[n] = before + blk[nb];
+    if (c[q] > kWarpCellMax) big_list[atomicAdd(big_count, 1)] = i;
   }
 }
 
-// Within each cell, order the particle indices ascending (this makes the counting sort
-// stable and deterministic).  Cells with <= 16 particles: insertion sort by one thread;
-// cells up to kWarpCellMax are queued at the front of big_list for a warp each, larger
-// ones at its back for a CTA each (big_count[0], big_count[1]; cell_sort.cuh).
-constexpr int kSmallCell = 16;
-__global__ void k_cell_sort_small(const int32_t* start, const int32_t* tmp, int32_t* perm, int ncell,
-                                  int32_t* big_list, int32_t* big_count) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-    const int s0 = start[c], n = start[c + 1] - s0;
-    if (n == 0) continue;
-    if (n > kSmallCell) {
-      if (n <= kWarpCellMax) big_list[atomicAdd(big_count, 1)] = c;
-      else big_list[ncell - 1 - atomicAdd(big_count + 1, 1)] = c;
-      continue;
-    }
-    int32_t v[kSmallCell];
-    for (int k = 0; k < n; ++k) {
-      int32_t e = tmp[s0 + k];
-      int q = k;
-      while (q > 0 && v[q - 1] > e) { v[q] = v[q - 1]; --q; }
-      v[q] = e;
-    }
-    for (int k = 0; k < n; ++k) perm[s0 + k] = v[k];
-  }
+// Counting-sort scatter into the cells, in the order of the keys' atomics.
+__global__ void k_scatter(const int32_t* __restrict__ keys, const int32_t* __restrict__ place,
+                          const int32_t* __restrict__ start, int64_t np, int32_t* __restrict__ tmp) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x)
+    tmp[start[keys[i]] + place[i]] = (int32_t)i;
 }
 
-// With tail = 1 the inactive sub-bins past the ncell cells are copied over as they are
-// (nothing depends on the order of inactive particles).  The cells queued at the back of
-// big_list are sorted by whole CTAs, which use the cell's range of tmp as their second
-// buffer.
+// Cells of more than kWarpCellMax particles: their indices in ascending order into perm, a CTA a
+// cell, with the cell's range of tmp as the second buffer (cell_sort.cuh).
 __global__ void __launch_bounds__(256) k_cell_sort_big(const int32_t* start, int32_t* tmp, int32_t* perm,
-                                                       const int32_t* big_list, const int32_t* big_count,
-                                                       int ncell, int tail) {
+                                                       const int32_t* big_list, const int32_t* big_count) {
   __shared__ int32_t sm[kCellChunk];
-  if (tail) {
-    const int32_t b = start[ncell], e = start[ncell + kTailBins];
-    for (int32_t i = b + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) perm[i] = tmp[i];
-  }
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int nmid = big_count[0], nhuge = big_count[1];
-  for (int b = gw; b < nmid; b += nw) {
-    const int c = big_list[b];
-    const int s0 = start[c];
-    warp_rank_cell(tmp + s0, perm + s0, start[c + 1] - s0);
-  }
-  for (int b = blockIdx.x; b < nhuge; b += gridDim.x) {
-    const int c = big_list[ncell - 1 - b];
-    const int s0 = start[c];
-    cta_sort_cell(tmp + s0, perm + s0, tmp + s0, start[c + 1] - s0, sm);
+  const int nbig = *big_count;
+  for (int b = blockIdx.x; b < nbig; b += gridDim.x) {
+    const int s0 = start[big_list[b]];
+    cta_sort_cell(tmp + s0, perm + s0, tmp + s0, start[big_list[b] + 1] - s0, sm);
   }
 }
 
-// dst[i] = src[perm[i]]; with a moving window (slot non-null) the array index of every
-// inactive particle is recorded by id for the next injection.
+// The sorted place of the particle at scattered place i and its index e: within a cell the indices
+// ascend (which makes the counting sort stable and deterministic).  An entry of a cell of up to
+// kWarpCellMax particles counts the smaller ones among the cell's, which the neighbouring threads
+// read too; crowded cells are in order in perm already; inactive particles stay as they are
+// (nothing depends on their order).  The count runs while the particle's own values are in flight,
+// so the permutation waits for memory no longer than without it; by a kernel before it (an insertion
+// sort by a thread a cell) it took as long as a third of the permutation.  Both, before and now: 16.8 ->
+// 4.8 us at 256 x 64 cells and 36 000 particles, 69 -> 33 us at 1.6 M particles (FP64), 42 -> 29 us
+// at 2048 x 256 cells and 1.3 M particles, 48 -> 40 us at 2.2 M particles (mixed form).
+struct Sorted {
+  const int32_t* keys;
+  const int32_t* start;
+  const int32_t* tmp;
+  int32_t* perm;
+  int ncell;
+};
+__device__ __forceinline__ int32_t sorted_place(const Sorted& so, int32_t i, int32_t& e) {
+  const int32_t key = so.keys[e];
+  int32_t at = i;
+  if (key < so.ncell) {
+    const int32_t s0 = so.start[key], n = so.start[key + 1] - s0;
+    if (n > kWarpCellMax) {
+      e = so.perm[i];
+      return i;
+    }
+    at = s0;
+    for (int32_t q = 0; q < n; ++q) at += so.tmp[s0 + q] < e;
+  }
+  so.perm[at] = e;
+  return at;
+}
+
+// dst[at] = src[e] in the sorted order; with a moving window (slot non-null) the array index of
+// every inactive particle is recorded by id for the next injection.
 template <bool WIN>
-__global__ void k_permute(const Parts src, Parts dst, const int32_t* perm, int64_t np, int32_t* slot) {
+__global__ void k_permute(const Parts src, Parts dst, const Sorted so, int64_t np, int32_t* slot) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t k = perm[i];
-    const double w = src.w[k];
-    const int32_t id = src.id[k];
-    dst.x[i] = src.x[k]; dst.y[i] = src.y[k]; dst.z[i] = src.z[k];
-    dst.ux[i] = src.ux[k]; dst.uy[i] = src.uy[k]; dst.uz[i] = src.uz[k];
-    dst.w[i] = w; dst.id[i] = id;
-    if (WIN && w == 0.0) slot[id] = (int32_t)i;
+    const int32_t k0 = so.tmp[i];
+    double x, y, z, ux, uy, uz, w;
+    int32_t id;
+    auto load = [&](int32_t j) {
+      x = src.x[j]; y = src.y[j]; z = src.z[j]; ux = src.ux[j]; uy = src.uy[j]; uz = src.uz[j];
+      w = src.w[j]; id = src.id[j];
+    };
+    load(k0);   // in flight while the place is found
+    int32_t k = k0;
+    const int32_t at = sorted_place(so, (int32_t)i, k);
+    if (k != k0) load(k);
+    dst.x[at] = x; dst.y[at] = y; dst.z[at] = z;
+    dst.ux[at] = ux; dst.uy[at] = uy; dst.uz[at] = uz;
+    dst.w[at] = w; dst.id[at] = id;
+    if (WIN && w == 0.0) slot[id] = at;
   }
 }
 
@@ -1363,14 +1355,16 @@ __global__ void k_inv_volume_f(float* invV, int Nr, double dr, double dz) {
 }
 
 template <bool WIN>
-__global__ void k_keys_f32(const PartsF p, int64_t np, GeomF g, int32_t* keys, int32_t* count, int32_t* err) {
+__global__ void k_keys_f32(const PartsF p, int64_t np, GeomF g, int32_t* keys, int32_t* count, int32_t* place,
+                           int32_t* err) {
   const int ncell = g.Nz * g.Nr;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (WIN) {
       const bool inactive = p.w[i] == 0.f;
-      count_inactive(count, tail_key(ncell, i), inactive);
+      const int32_t at = count_inactive(count, tail_key(ncell, i), inactive);
       if (inactive) {
+        place[i] = at;
         keys[i] = tail_key(ncell, i);
         continue;
       }
@@ -1388,47 +1382,32 @@ __global__ void k_keys_f32(const PartsF p, int64_t np, GeomF g, int32_t* keys, i
     const int ir = (int)fminf(fmaxf(fr, 0.f), (float)(g.Nr - 1));
     const int key = iz * g.Nr + ir;
     keys[i] = key;
-    atomicAdd(count + key, 1);
+    place[i] = atomicAdd(count + key, 1);
   }
 }
 
-// dst[i] = src[perm[i]] for the 13 arrays; four particles per thread, all loads issued
-// before the stores (the gathered reads are latency-bound).
+// dst[at] = src[e] in the sorted order (sorted_place) for the 13 arrays.
 template <bool WIN>
-__global__ void k_permute_f32(const PartsF src, PartsF dst, const int32_t* __restrict__ perm, int64_t np,
-                              int32_t* slot) {
-  constexpr int U = 4;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < np; i0 += U * stride) {
-    int32_t k[U];
-    bool ok[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t i = i0 + u * stride;
-      ok[u] = i < np;
-      k[u] = ok[u] ? perm[i] : 0;
-    }
-    int32_t iz[U], ixy[U], id[U];
-    float fz[U], fx[U], fy[U], ux[U], uy[U], uz[U], uxl[U], uyl[U], uzl[U], w[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!ok[u]) continue;
-      const int32_t j = k[u];
-      iz[u] = src.iz[j]; fz[u] = src.fz[j]; ixy[u] = src.ixy[j]; fx[u] = src.fx[j]; fy[u] = src.fy[j];
-      ux[u] = src.ux[j]; uy[u] = src.uy[j]; uz[u] = src.uz[j];
-      uxl[u] = src.uxl[j]; uyl[u] = src.uyl[j]; uzl[u] = src.uzl[j];
-      w[u] = src.w[j]; id[u] = src.id[j];
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!ok[u]) continue;
-      const int64_t i = i0 + u * stride;
-      dst.iz[i] = iz[u]; dst.fz[i] = fz[u]; dst.ixy[i] = ixy[u]; dst.fx[i] = fx[u]; dst.fy[i] = fy[u];
-      dst.ux[i] = ux[u]; dst.uy[i] = uy[u]; dst.uz[i] = uz[u];
-      dst.uxl[i] = uxl[u]; dst.uyl[i] = uyl[u]; dst.uzl[i] = uzl[u];
-      dst.w[i] = w[u]; dst.id[i] = id[u];
-      if (WIN && w[u] == 0.f) slot[id[u]] = (int32_t)i;   // moving window: inactive slot by id
-    }
+__global__ void k_permute_f32(const PartsF src, PartsF dst, const Sorted so, int64_t np, int32_t* slot) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t k0 = so.tmp[i];
+    int32_t iz, ixy, id;
+    float fz, fx, fy, ux, uy, uz, uxl, uyl, uzl, w;
+    auto load = [&](int32_t j) {
+      iz = src.iz[j]; fz = src.fz[j]; ixy = src.ixy[j]; fx = src.fx[j]; fy = src.fy[j];
+      ux = src.ux[j]; uy = src.uy[j]; uz = src.uz[j];
+      uxl = src.uxl[j]; uyl = src.uyl[j]; uzl = src.uzl[j];
+      w = src.w[j]; id = src.id[j];
+    };
+    load(k0);   // in flight while the place is found
+    int32_t k = k0;
+    const int32_t at = sorted_place(so, (int32_t)i, k);
+    if (k != k0) load(k);
+    dst.iz[at] = iz; dst.fz[at] = fz; dst.ixy[at] = ixy; dst.fx[at] = fx; dst.fy[at] = fy;
+    dst.ux[at] = ux; dst.uy[at] = uy; dst.uz[at] = uz;
+    dst.uxl[at] = uxl; dst.uyl[at] = uyl; dst.uzl[at] = uzl;
+    dst.w[at] = w; dst.id[at] = id;
+    if (WIN && w == 0.f) slot[id] = at;   // moving window: inactive slot by id
   }
 }
 
@@ -2443,52 +2422,45 @@ pic_status launch_sort(Sim* s) {
   int32_t* big_list = s->at<int32_t>(s->lay.big_list);
   int32_t* big_count = s->at<int32_t>(s->lay.big_count);
   int32_t* err = s->at<int32_t>(s->lay.err);
-  int32_t* cursor = reinterpret_cast<int32_t*>(s->at<char>(s->lay.scan_blk) + 4 * 4096 * sizeof(int32_t));
   int32_t* slot = s->win.on ? reinterpret_cast<int32_t*>(s->win.ws + s->win.slot) : nullptr;
   PIC_CUDA(cudaMemsetAsync(count, 0, sizeof(int32_t) * (ncell + kTailBins + 1), s->stream));   // cells + inactive
-  PIC_CUDA(cudaMemsetAsync(big_count, 0, 2 * sizeof(int32_t), s->stream));
   if (np == 0) return PIC_OK;
   const bool win = slot != nullptr;
+  // perm holds the particles' places within their keys until the scatter has read them
   if (is_mixed(s)) {
     if (win)
-      k_keys_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), np, geomf_of(s), keys, count, err);
+      k_keys_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), np, geomf_of(s), keys, count, perm, err);
     else
-      k_keys_f32<false><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), np, geomf_of(s), keys, count, err);
+      k_keys_f32<false><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), np, geomf_of(s), keys, count, perm, err);
   } else {
     if (win)
-      k_keys<true><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), np, geom_of(s), keys, count, err);
+      k_keys<true><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), np, geom_of(s), keys, count, perm, err);
     else
-      k_keys<false><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), np, geom_of(s), keys, count, err);
+      k_keys<false><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), np, geom_of(s), keys, count, perm, err);
   }
   PIC_LAUNCHED(s);
   const int nbin = ncell + kTailBins;
   const int nblk = (nbin + kScanBlock - 1) / kScanBlock;
-  k_scan_local<<<nblk, kScanThreads, 0, s->stream>>>(count, start, blk, nbin);
+  k_scan_local<<<nblk, kScanThreads, 0, s->stream>>>(count, start, blk, nbin, big_count);
   PIC_LAUNCHED(s);
-  k_scan_blocks<<<1, kScanThreads, 0, s->stream>>>(blk, nblk, start, nbin);
+  k_scan_add<<<(nbin + kScanBlock / 4 - 1) / (kScanBlock / 4), 256, 0, s->stream>>>(count, start, blk, nbin, ncell, big_list, big_count);
   PIC_LAUNCHED(s);
-  k_scan_add<<<pgrid(nbin), 256, 0, s->stream>>>(start, blk, nbin, cursor);
+  k_scatter<<<pgrid(np), 256, 0, s->stream>>>(keys, perm, start, np, tmp);
   PIC_LAUNCHED(s);
-  if (win)
-    k_scatter<true><<<pgrid(np), 256, 0, s->stream>>>(keys, np, cursor, tmp, ncell);
-  else
-    k_scatter<false><<<pgrid(np), 256, 0, s->stream>>>(keys, np, cursor, tmp, ncell);
+  k_cell_sort_big<<<152 * 4, 256, 0, s->stream>>>(start, tmp, perm, big_list, big_count);
   PIC_LAUNCHED(s);
-  k_cell_sort_small<<<pgrid(ncell), 256, 0, s->stream>>>(start, tmp, perm, ncell, big_list, big_count);
-  PIC_LAUNCHED(s);
-  k_cell_sort_big<<<152 * 4, 256, 0, s->stream>>>(start, tmp, perm, big_list, big_count, ncell, win ? 1 : 0);
-  PIC_LAUNCHED(s);
+  const Sorted so{keys, start, tmp, perm, ncell};
   if (is_mixed(s))
     if (win)
-      k_permute_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), perm, np,
+      k_permute_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), so, np,
                                                             slot);
     else
-      k_permute_f32<false><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), perm, np,
+      k_permute_f32<false><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), so, np,
                                                              slot);
   else if (win)
-    k_permute<true><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), perm, np, slot);
+    k_permute<true><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), so, np, slot);
   else
-    k_permute<false><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), perm, np, slot);
+    k_permute<false><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), so, np, slot);
   PIC_LAUNCHED(s);
   s->cur = 1 - s->cur;
   return PIC_OK;

@@ -163,7 +163,7 @@ Layout make_layout(const pic_config& c) {
   L.perm_tmp = take(cap * 4);
   L.count = take((ncell + 66) * 4);   // cells plus 64 sub-bins of inactive particles (+1)
   L.start = take((ncell + 66) * 4);
-  L.scan_blk = take(4 * 4096 * 4 + (ncell + 66) * 4);   // block totals, then the scatter cursor
+  L.scan_blk = take(4 * 4096 * 4);   // block totals
   L.big_list = take(ncell * 4);
   L.big_count = take(256);
   L.diag_acc = take(diag_acc_doubles() * 8);
