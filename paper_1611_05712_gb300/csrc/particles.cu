@@ -41,11 +41,27 @@ struct GridGeom {
   size_t G;      // Nm*Nr*Nz
   double inv_dr; // 1/dr, 1/dz correctly rounded (float64 divisions are long sequences on
   double inv_dz; // GB300's float64 unit)
+  unsigned long long mz, mr;   // 1/dz = mz 2^(ez + 1074), 1/dr = mr 2^(er + 1074), mantissas of 64 bits
+  int ez, er;
 };
+
+// 1/d, cut to 64 bits, as m 2^(e + 1074): e is such that x / d = (X m / 2^64) 2^(f + e) for x with
+// exponent field f and its 53-bit mantissa X at the top of a 64-bit word.
+void reciprocal64(double d, unsigned long long& m, int& e) {
+  int k = 0;
+  const unsigned long long M = (unsigned long long)std::ldexp(std::frexp(d, &k), 53);   // d = M 2^(k - 53)
+  const unsigned __int128 q = ((unsigned __int128)1 << 116) / M;                        // in (2^63, 2^64]
+  const bool pow2 = (unsigned long long)(q >> 64) != 0;
+  m = pow2 ? 1ull << 63 : (unsigned long long)q;
+  e = -1138 - (k - 53) + (pow2 ? 1 : 0);
+}
 
 GridGeom geom_of(const Sim* s) {
   const pic_config& c = s->cfg;
-  GridGeom g{c.Nz, c.Nr, c.Nm, c.dz, c.dr, c.Nz * c.dz, c.Nr * c.dr, s->grid_elems(), 1.0 / c.dr, 1.0 / c.dz};
+  GridGeom g{c.Nz, c.Nr, c.Nm, c.dz, c.dr, c.Nz * c.dz, c.Nr * c.dr, s->grid_elems(), 1.0 / c.dr, 1.0 / c.dz,
+             0, 0, 0, 0};
+  reciprocal64(c.dz, g.mz, g.ez);
+  reciprocal64(c.dr, g.mr, g.er);
   return g;
 }
 
@@ -176,6 +192,150 @@ __device__ __forceinline__ Stencil stencil(const GridGeom& g, double z, double r
   return st;
 }
 
+// Products of the deposits on the integer units.  A particle adds 12 (2 Nm - 1) + 4 (2 Nm - 1)
+// products of five factors to the grids, half of the push kernel's float64 operations when the
+// float64 unit forms them.  Here a factor is its 53-bit mantissa as a 62-bit integer in two
+// halves of 31 bits, its exponent and its sign: a product takes three wide multiply-adds and four
+// shifts (the low halves' product is left out) and may start one bit lower; the chain of them keeps
+// 56 bits or more and is rounded to float64 once at the end, where the float64 products rounded
+// each time.
+struct Sf {
+  unsigned h, l;   // mantissa h 2^31 + l, in [2^61, 2^62) for a converted number; 0 for zero
+  int e;           // biased exponent: the value is mantissa 2^(e - 1023 - 61)
+  unsigned s;      // sign in bit 31
+};
+
+__device__ __forceinline__ Sf sf_from(double x) {   // subnormal x count as zero
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  Sf r;
+  r.h = e ? (((hi & 0xfffffu) | 0x100000u) << 10) | (lo >> 22) : 0u;
+  r.l = e ? (lo << 9) & 0x7fffffffu : 0u;
+  r.e = e ? e : -100000;   // products with zero fall out of the exponent range (sf_far)
+  r.s = hi & 0x80000000u;
+  return r;
+}
+
+__device__ __forceinline__ unsigned long long sf_mantissa(const Sf& a) { return ((unsigned long long)a.h << 31) | a.l; }
+
+__device__ __forceinline__ unsigned long long sf_product(const Sf& a, const Sf& b) {   // mantissas' product >> 62
+  const unsigned long long t = (unsigned long long)a.h * b.l + (unsigned long long)a.l * b.h;   // below 2^63
+  return (unsigned long long)a.h * b.h + (t >> 31);
+}
+
+__device__ __forceinline__ Sf operator*(const Sf& a, const Sf& b) {
+  const unsigned long long p = sf_product(a, b);
+  return Sf{(unsigned)(p >> 31), (unsigned)p & 0x7fffffffu, a.e + b.e - 1022, a.s ^ b.s};
+}
+
+// sf_double of zero and of results outside the normal range (NaN factors: e is large).  In line: a
+// call here would have the kernels keep their values in memory around it.
+__device__ __forceinline__ double sf_far(unsigned long long m, int e, unsigned s) {
+  unsigned long long r;
+  if (e > 12) {
+    r = m == 0ull ? 0ull : e > 3000 ? 0x7ff8000000000000ull : 0x7ff0000000000000ull;
+  } else {   // m 2^(e - 10) units of the subnormal numbers
+    const int sh = 10 - e;
+    r = sh < 64 && sh > 0 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
+  }
+  return __longlong_as_double((long long)(r | (unsigned long long)s << 32));
+}
+
+// Mantissa m (0, or 2^55 <= m < 2^62) with biased exponent e and sign s as a float64.
+__device__ __forceinline__ double sf_double(unsigned long long m, int e, unsigned s) {
+  const int lz = __clz((int)(unsigned)(m >> 32));
+  const unsigned long long r = ((m << (lz - 1)) + 0x200u) >> 10;   // 53 bits, rounded (2^53 carries on)
+  const int ex = e + 2 - lz;                                       // exponent field of the result
+  if ((unsigned)(ex - 1) >= 2044u) return sf_far(m, e, s);
+  return __hiloint2double((int)((unsigned)(r >> 32) + ((unsigned)(ex - 1) << 20) | s), (int)(unsigned)r);
+}
+
+// A fraction w 2^-62, 0 <= w <= 2^62, as a factor (2^62 itself as 2^62 - 1).
+constexpr unsigned long long kOne62 = 1ull << 62;
+__device__ __forceinline__ Sf sf_fraction(unsigned long long w) {
+  if (w == kOne62) --w;
+  const int n = __clzll((long long)w);
+  const unsigned long long m = w << (n - 2 & 63);
+  return Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, w == 0ull ? -100000 : 1024 - n, 0u};
+}
+
+// a with its mantissa's leading bit at 2^61 again (a is zero or a product: at least 2^55).
+__device__ __forceinline__ Sf sf_normal(const Sf& a) {
+  const int n = __clz((int)a.h) - 1;   // h < 2^31
+  const unsigned long long m = sf_mantissa(a) << (a.h ? n : 0);
+  return Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, a.e - n, a.s};
+}
+
+// A weight (a product of two fractions) as a double word: 24 bits cut, the rest rounded.
+__device__ __forceinline__ dw dw_weight(const Sf& a) {
+  const Sf p = sf_normal(a);
+  if (p.h == 0u || p.e < 960) return dw(0.f, 0.f);   // weights below 2^-63 count as zero
+  const unsigned long long m = sf_mantissa(p);
+  const float lo = __uint2float_rn((unsigned)(m >> 6)  /* bits 37 .. 6 */);
+  return dw(__uint_as_float(((unsigned)(p.e - 896) << 23) | ((unsigned)(m >> 38) & 0x7fffffu)),
+            __fmul_rn(lo, __uint_as_float((unsigned)(p.e - 951) << 23)));
+}
+
+// u = x / d >= 0 as i + f 2^-62 from the bits, with d's reciprocal in 64 bits: off by less than u
+// 2^-61 below the quotient, where the rounded float64 quotient is off by up to u 2^-53.  False unless
+// 0 <= u < 2^31.
+__device__ __forceinline__ bool cell_fraction(double x, unsigned long long m, int e, int& i, unsigned long long& f) {
+  const unsigned hi = (unsigned)__double2hiint(x), ex = hi >> 20;   // a sign makes ex >= 2048
+  const unsigned long long X = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 43) |
+                               ((unsigned long long)(unsigned)__double2loint(x) << 11);
+  const unsigned long long P = __umul64hi(X, m);
+  const int n = -((int)ex + e);   // u = P 2^-n
+  if (ex >= 2047u || n < 33) return false;
+  const bool small = n >= 64;     // u < 1
+  i = small ? 0 : (int)(P >> (n & 63));
+  f = small ? (n < 128 ? P >> (n & 63) : 0ull) : P << (64 - n & 63);
+  f >>= 2;
+  return true;
+}
+
+// The cells and fractions of a particle's stencil: rows i0, i1 with weights 1 - fz, fz, radial nodes
+// j0, j0 + 1 with weights 1 - fr, fr (fz, fr in units of 2^-62).
+struct Stencil62 {
+  int i0, i1, j0;
+  unsigned long long fz, fr;
+};
+
+// ... of coordinates outside the box, infinite and NaN, by the stencil above (out of line: rare).
+__device__ __noinline__ Stencil62 stencil62_far(int Nz, int Nr, double dz, double inv_dz, double inv_dr, double z,
+                                                double r) {
+  GridGeom g;
+  g.Nz = Nz; g.Nr = Nr; g.dz = dz; g.inv_dz = inv_dz; g.inv_dr = inv_dr;
+  const Stencil d = stencil(g, z, r);
+  Stencil62 st;
+  st.i0 = d.i0; st.i1 = d.i1; st.j0 = d.j0;
+  st.fz = min((unsigned long long)__double2ull_rz(d.wz1 * 4611686018427387904.0), kOne62 - 1);
+  st.fr = min((unsigned long long)__double2ull_rz(d.wr1 * 4611686018427387904.0), kOne62 - 1);
+  return st;
+}
+
+// The stencil without the float64 unit (the one above takes 14 operations of it, three times a
+// particle: a quarter of what the push did there).  Without them, with the weights' products in integers: push of
+// 1.35 M particles 583 -> 536 us, rho deposit of 1.64 M 192 -> 181.
+__device__ __forceinline__ Stencil62 stencil62(const GridGeom& g, double z, double r) {
+  Stencil62 st;
+  int jr;
+  unsigned long long fr;
+  if (cell_fraction(z, g.mz, g.ez, st.i0, st.fz) && st.i0 < g.Nz && cell_fraction(r, g.mr, g.er, jr, fr)) {
+    const bool up = fr >= kOne62 / 2;   // node j sits at r = (j + 1/2) dr
+    st.j0 = min(up ? jr : jr - 1, g.Nr);
+    st.fr = up ? fr - kOne62 / 2 : fr + kOne62 / 2;
+    st.i1 = st.i0 + 1 == g.Nz ? 0 : st.i0 + 1;
+    return st;
+  }
+  return stencil62_far(g.Nz, g.Nr, g.dz, g.inv_dz, g.inv_dr, z, r);
+}
+
+// Starts the read of *p into L2.  The particle loop reads the arrays that the statistics pass does
+// not need only after a chain of dependent loads: with their lines requested here the push of 1.35 M
+// particles (2048 x 256, 2 modes) takes 160 us where it took 165, the rho deposit of 2.2 M 62.5 us
+// where it took 66.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Gather weights of a particle's 4 nodes n = 2 dz + dj (rows i0, i1; radial nodes j0, j0 + 1):
 // w_z w_r, 0 for a dropped node (j >= Nr, read at a valid address); the ghost node r = -dr/2
 // of the axis cell (j0 = -1) is read at node 0 and takes its field's fold sign.
@@ -211,6 +371,29 @@ __device__ __forceinline__ GatherNodes gather_nodes(const GridGeom& g, const Ste
 // plus the operands' own double-word rounding), against the n 2^-53 of a float64 sum;
 // GB300 runs float64 at 1/64 of its float32 rate, and the float64 unit bounds the particle
 // pass.
+// The weights come from the stencil's fractions by integer products.
+struct GatherNodesDw {
+  dw w[4];
+  unsigned off[4];
+  bool ghost;
+};
+
+__device__ __forceinline__ GatherNodesDw gather_nodes_dw(const GridGeom& g, const Stencil62& st) {
+  GatherNodesDw gn;
+  const Sf z0 = sf_fraction(kOne62 - st.fz), z1 = sf_fraction(st.fz);
+  const Sf r0 = sf_fraction(kOne62 - st.fr), r1 = sf_fraction(st.fr);
+#pragma unroll
+  for (int n = 0; n < 4; ++n) {
+    const int dz = n >> 1, dj = n & 1;
+    const int j = st.j0 + dj;
+    const bool keep = j < g.Nr;
+    gn.w[n] = keep ? dw_weight((dz ? z1 : z0) * (dj ? r1 : r0)) : dw(0.f, 0.f);
+    gn.off[n] = (unsigned)(j < 0 || !keep ? 0 : j) * g.Nz + (dz ? st.i1 : st.i0);
+  }
+  gn.ghost = st.j0 < 0;
+  return gn;
+}
+
 struct Dot2 {
   float s, c;   // running sum and collected errors: the value is s + c
 };
@@ -230,54 +413,42 @@ __device__ __forceinline__ dw dw_twice(dw x) { return dw(__fmul_rn(2.f, x.hi), _
 // F_k = Re sum_m mult_m e^{-i m theta} sum_n w_n F_{k,m}(node n) as in k_gather_push, with
 // 2 Re(e^{-i m theta} v) = 2 cos(m theta) Re v + 2 sin(m theta) Im v; the inner nodes (n = 0,
 // 2) take their field's fold sign through sign-flipped copies of their weights.
-__device__ __forceinline__ void gather_dw(const GridGeom& g, const GatherNodes& gn, double c, double s,
+__device__ __forceinline__ void gather_dw(const GridGeom& g, const GatherNodesDw& gn, double c, double s,
                                           const float4* __restrict__ EB, double (&F)[6]) {
   const size_t RZ = (size_t)g.Nr * g.Nz;
-  dw w[4];
-#pragma unroll
-  for (int n = 0; n < 4; ++n) w[n] = dw_from_double(gn.w[n]);
   Dot2 acc[6];
-  {   // mode 0: real part; fold +1 for z components, -1 for r and theta
-    const dw f0 = neg_if(w[0], gn.ghost), f2 = neg_if(w[2], gn.ghost);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {   // real parts only: (re.hi, re.lo) of each float4
-      const float2* base = reinterpret_cast<const float2*>(EB + (size_t)k * g.G);
-      const bool zc = (k % 3) == 2;
-      const float2 v0 = base[2 * gn.off[0]], v1 = base[2 * gn.off[1]], v2 = base[2 * gn.off[2]],
-                   v3 = base[2 * gn.off[3]];
-      acc[k].s = 0.f;
-      acc[k].c = 0.f;
-      dot2_add(acc[k], zc ? w[0] : f0, v0.x, v0.y);
-      dot2_add(acc[k], w[1], v1.x, v1.y);
-      dot2_add(acc[k], zc ? w[2] : f2, v2.x, v2.y);
-      dot2_add(acc[k], w[3], v3.x, v3.y);
+  for (int k = 0; k < 6; ++k) acc[k].s = acc[k].c = 0.f;
+  // node by node, so that one node's factors are in registers at a time
+#pragma unroll
+  for (int n = 0; n < 4; ++n) {   // mode 0: real part; fold +1 for z components, -1 for r and theta
+    const float2* base = reinterpret_cast<const float2*>(EB + gn.off[n]);   // (re.hi, re.lo) of a float4
+    const dw wz = gn.w[n], wv = neg_if(wz, !(n & 1) && gn.ghost);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const float2 v = base[2 * (size_t)k * g.G];
+      dot2_add(acc[k], (k % 3) == 2 ? wz : wv, v.x, v.y);
     }
   }
   const dw c1 = dw_from_double(c), s1 = dw_from_double(s);
   dw cm = c1, sm = s1;   // cos(m theta), sin(m theta)
   for (int m = 1; m < g.Nm; ++m) {
     const dw c2 = dw_twice(cm), s2 = dw_twice(sm);
-    dw A[4], S[4];
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-      A[n] = w[n] * c2;
-      S[n] = w[n] * s2;
-    }
-    // fold signs of the inner nodes: z components (-1)^m, r and theta (-1)^{m+1}
-    const bool negZ = gn.ghost && (m & 1), negV = gn.ghost && !(m & 1);
+      const float4* base = EB + (size_t)m * RZ + gn.off[n];
+      // fold signs of the inner nodes: z components (-1)^m, r and theta (-1)^{m+1}
+      const bool ghost = !(n & 1) && gn.ghost;
+      const dw A = gn.w[n] * c2, S = gn.w[n] * s2;
+      const dw az = neg_if(A, ghost && (m & 1)), sz = neg_if(S, ghost && (m & 1));
+      const dw av = neg_if(A, ghost && !(m & 1)), sv = neg_if(S, ghost && !(m & 1));
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const float4* base = EB + (size_t)k * g.G + (size_t)m * RZ;
-      const bool neg = (k % 3) == 2 ? negZ : negV;
-      const float4 v0 = base[gn.off[0]], v1 = base[gn.off[1]], v2 = base[gn.off[2]], v3 = base[gn.off[3]];
-      dot2_add(acc[k], neg_if(A[0], neg), v0.x, v0.y);
-      dot2_add(acc[k], neg_if(S[0], neg), v0.z, v0.w);
-      dot2_add(acc[k], A[1], v1.x, v1.y);
-      dot2_add(acc[k], S[1], v1.z, v1.w);
-      dot2_add(acc[k], neg_if(A[2], neg), v2.x, v2.y);
-      dot2_add(acc[k], neg_if(S[2], neg), v2.z, v2.w);
-      dot2_add(acc[k], A[3], v3.x, v3.y);
-      dot2_add(acc[k], S[3], v3.z, v3.w);
+      for (int k = 0; k < 6; ++k) {
+        const float4 v = base[(size_t)k * g.G];
+        const bool zc = (k % 3) == 2;
+        dot2_add(acc[k], zc ? az : av, v.x, v.y);
+        dot2_add(acc[k], zc ? sz : sv, v.z, v.w);
+      }
     }
     const dw nc = cm * c1 - sm * s1, ns = sm * c1 + cm * s1;   // times e^{i theta}
     cm = nc;
@@ -538,59 +709,6 @@ __device__ __forceinline__ void dep2(double2* p, double re, double im) {
   atomicAdd(d + 1, im);
 }
 
-// Products of the deposits on the integer units.  A particle adds 12 (2 Nm - 1) + 4 (2 Nm - 1)
-// products of five factors to the grids, half of the push kernel's float64 operations when the
-// float64 unit forms them.  Here a factor is its 53-bit mantissa as a 62-bit integer in two
-// halves of 31 bits, its exponent and its sign: a product takes three wide multiply-adds and four
-// shifts (the low halves' product is left out), keeps 57 bits or more over the chain of four
-// (each product may start one bit lower), and is rounded to float64 once at the end, where
-// the float64 products rounded each time.
-struct Sf {
-  unsigned h, l;   // mantissa h 2^31 + l, in [2^61, 2^62) for a converted number; 0 for zero
-  int e;           // biased exponent: the value is mantissa 2^(e - 1023 - 61)
-  unsigned s;      // sign in bit 31
-};
-
-__device__ __forceinline__ Sf sf_from(double x) {   // subnormal x count as zero
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  Sf r;
-  r.h = e ? (((hi & 0xfffffu) | 0x100000u) << 10) | (lo >> 22) : 0u;
-  r.l = e ? (lo << 9) & 0x7fffffffu : 0u;
-  r.e = e ? e : -100000;   // products with zero fall out of the exponent range (sf_far)
-  r.s = hi & 0x80000000u;
-  return r;
-}
-
-__device__ __forceinline__ unsigned long long sf_mantissa(const Sf& a) { return ((unsigned long long)a.h << 31) | a.l; }
-
-__device__ __forceinline__ unsigned long long sf_product(const Sf& a, const Sf& b) {   // mantissas' product >> 62
-  const unsigned long long t = (unsigned long long)a.h * b.l + (unsigned long long)a.l * b.h;   // below 2^63
-  return (unsigned long long)a.h * b.h + (t >> 31);
-}
-
-__device__ __forceinline__ Sf operator*(const Sf& a, const Sf& b) {
-  const unsigned long long p = sf_product(a, b);
-  return Sf{(unsigned)(p >> 31), (unsigned)p & 0x7fffffffu, a.e + b.e - 1022, a.s ^ b.s};
-}
-
-// sf_double of zero and of results outside the normal range (NaN factors: e is large).
-__device__ __noinline__ double sf_far(unsigned long long m, int e, unsigned s) {
-  if (m == 0ull) return 0.0;
-  if (e > 3000) return __longlong_as_double(0x7ff8000000000000ll);
-  const double v = ldexp((double)m, e - 1023 - 61);
-  return s ? -v : v;
-}
-
-// Mantissa m (0, or 2^56 <= m < 2^62) with biased exponent e and sign s as a float64.
-__device__ __forceinline__ double sf_double(unsigned long long m, int e, unsigned s) {
-  const int lz = __clz((int)(unsigned)(m >> 32));
-  const unsigned long long r = ((m << (lz - 1)) + 0x200u) >> 10;   // 53 bits, rounded (2^53 carries on)
-  const int ex = e + 2 - lz;                                       // exponent field of the result
-  if ((unsigned)(ex - 1) >= 2044u) return sf_far(m, e, s);
-  return __hiloint2double((int)((unsigned)(r >> 32) + ((unsigned)(ex - 1) << 20) | s), (int)(unsigned)r);
-}
-
 // Deposit of one particle: rho (RHO) and/or J (CUR) with weight e^{+i m theta} per mode, linear
 // weights; the ghost node r = -dr/2 of the axis cell is node 0 seen across the axis (fold sign
 // (-1)^m for rho and J_z, (-1)^{m+1} for J_r and J_theta) and node Nr is dropped.  The
@@ -602,11 +720,11 @@ __device__ __forceinline__ double sf_double(unsigned long long m, int e, unsigne
 template <int MODES, bool RHO, bool CUR>
 __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* invV, double r,
                            double c, double s, double z, double w, double vx, double vy, double vz) {
-  const Stencil st = stencil(g, z, r);
+  const Stencil62 st = stencil62(g, z, r);
   const size_t RZ = (size_t)g.Nr * g.Nz;
   const int rot = threadIdx.x & 3;
   const bool ghost = st.j0 < 0;
-  const double qw = a.q * w;
+  const Sf qw = sf_from(a.q) * sf_from(w);
   Sf rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (0 for the dropped node Nr)
   int jn[2];   // their grid rows (the ghost node j = -1 is row 0)
 #pragma unroll
@@ -614,7 +732,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     const int j = st.j0 + dj;
     const bool keep = j < g.Nr;
     jn[dj] = (j < 0 || !keep) ? 0 : j;
-    rad[dj] = sf_from(keep ? (dj ? st.wr1 : st.wr0) : 0.0) * sf_from(invV[jn[dj]] * qw);
+    rad[dj] = sf_normal(sf_fraction(keep ? (dj ? st.fr : kOne62 - st.fr) : 0ull) * (sf_from(invV[jn[dj]]) * qw));
   }
   Sf v[3], pr[MODES > 1 ? MODES - 1 : 1], pi[MODES > 1 ? MODES - 1 : 1];   // velocity; e^{+i m theta}, m = 1 ..
   if (CUR) {
@@ -623,7 +741,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     v[2] = sf_from(vz);
   }
   // a NaN or an infinity among the factors makes every product of the particle NaN
-  if (!is_finite(qw) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
+  if (!is_finite(w) || !is_finite(a.q) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
   {
     double er = c, ei = s;
 #pragma unroll
@@ -636,7 +754,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
       er = nr;
     }
   }
-  const Sf z0 = sf_from(st.wz0), z1 = sf_from(st.wz1);
+  const Sf z0 = sf_fraction(kOne62 - st.fz), z1 = sf_fraction(st.fz);
 #pragma unroll 1
   for (int q = 0; q < 4; ++q) {
     const int node = (q + rot) & 3, dz = node >> 1, dj = node & 1;
@@ -723,15 +841,19 @@ __device__ __forceinline__ void win_mark(const WinArgs& wa, int32_t id, int64_t 
 
 // WIN: moving window on (removal behind the back edge); the plain instance has none of it.
 // DWG: gather from the double-word copy of E, B (gather_dw) instead of the float64 grids.
-// Bound by the float64 unit (63 % busy) and by latency at 24 warps per SM: about 165 operations a
-// particle are left of 295 at two modes once comparisons, roundings and conversions run on the
-// integer units, roots and the quotient of the push take 5 and 3 operations, the cross products
-// are fused and the deposits' products are formed by the integer units (Sf).  Three CTAs per SM
-// at 80 registers hide its latency better than two at 128.  1.35 M particles, two modes: 846 us
-// at first, 703 with the float64 unit's own work reduced, 593 with the integer products; 1.64 M
-// particles, three modes: 959, 793, 764.  Leaving out all atomics would gain 20 us.
-template <int MODES, bool WIN, bool DWG>
-__global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
+// Bound by the float64 unit (about half of the time) and by latency at 24 warps per SM: about 110
+// operations a particle are left of 295 at two modes once comparisons, roundings and conversions run
+// on the integer units, roots and the quotient of the push take 5 and 3 operations, the cross
+// products are fused, and the stencils, the gather's weights and the deposits' products are formed
+// by the integer units (stencil62, Sf).  Momenta are read after the gather, requested into L2 before
+// it, and written before the deposits, and the gather goes node by node: the kernel needs more
+// registers than three CTAs per SM leave it (80; 236 to 408 bytes of its values go through local
+// memory), which still hides its latency better than two CTAs at 128.  1.35 M particles, two modes:
+// 846 us at first, 703 with the float64 unit's own work reduced, 593 with the integer products, 498
+// now (525 at 128 registers); 1.64 M particles, three modes: 959, 793, 746, 651 (664).  A set that
+// fits the SMs at once with 128 registers takes them (CTAS = 2): 36 000 particles 31.2 -> 28.1 us.
+template <int MODES, bool WIN, bool DWG, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
                               const double2* __restrict__ B, const float4* __restrict__ EBdw, double k,
                               double dt, DepArgs dep, const double* invV, int fuse, int32_t* err,
                               WinArgs wa) {
@@ -743,18 +865,17 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     double x = p.x[i], y = p.y[i], z = p.z[i];
     if (!is_finite(x) || !is_finite(y) || !is_finite(z)) { atomicOr(err, kErrNumeric); continue; }
     const double z_old = z;
-    double ux = p.ux[i], uy = p.uy[i], uz = p.uz[i];
+    prefetch_l2(p.ux + i); prefetch_l2(p.uy + i); prefetch_l2(p.uz + i);
     double r, c, s;
     polar(x, y, r, c, s);
-    const Stencil st = stencil(g, z, r);
     // F = Re sum_m mult_m e^{-i m theta} sum_n w_n F_m(node n), mult_0 = 1, mult_m = 2; per
     // mode the node weights are multiplied by mult e^{-i m theta} once for the 6 components,
     // and the ghost nodes (n = 0, 2) are summed apart so that the fold is one sign flip.
-    const GatherNodes gn = gather_nodes(g, st);
     double F[6];   // E_r, E_t, E_z, B_r, B_t, B_z
     if constexpr (DWG) {
-      gather_dw(g, gn, c, s, EBdw, F);
+      gather_dw(g, gather_nodes_dw(g, stencil62(g, z, r)), c, s, EBdw, F);
     } else {
+    const GatherNodes gn = gather_nodes(g, stencil(g, z, r));
 #pragma unroll
     for (int k = 0; k < 6; ++k) {   // mode 0: real phase, fold +1 for E_z, B_z and -1 for r, theta
       const double2* base = (k < 3 ? E : B) + (size_t)(k % 3) * g.G;
@@ -785,6 +906,7 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     }
     const double Ex = F[0] * c - F[1] * s, Ey = F[0] * s + F[1] * c, Ez = F[2];
     const double Bx = F[3] * c - F[4] * s, By = F[3] * s + F[4] * c, Bz = F[5];
+    double ux = p.ux[i], uy = p.uy[i], uz = p.uz[i];
     // Boris with k = q dt / (2 m) (from the host); 1/gamma^- once for the three t; the cross
     // products as chains of fused multiply-adds
     const double umx = ux + k * Ex, umy = uy + k * Ey, umz = uz + k * Ez;
@@ -800,6 +922,7 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     uz = fma(k, Ez, fma(-upy, sx, fma(upx, sy, umz)));
     const double ig = inv_sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * kInvC2);
     const double vx = ux * ig, vy = uy * ig, vz = uz * ig;
+    p.ux[i] = ux; p.uy[i] = uy; p.uz[i] = uz;   // out of the registers before the deposits
     const double hdt = 0.5 * dt;
     const double hx = __dmul_rn(hdt, vx), hy = __dmul_rn(hdt, vy), hz = __dmul_rn(hdt, vz);
     x = __dadd_rn(x, hx);   // no FMA: one ulp of z is ~L/dz ulps of a weight
@@ -818,13 +941,14 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
     polar(x, y, r1, c1, s1);
     if (at_least(r1, g.R)) {   // specular reflection (rare: the particle crossed the wall)
       const double fr = (2.0 * g.R - r1) / r1;
-      const double ur = ux * c1 + uy * s1;
-      ux = ux - 2.0 * ur * c1;
-      uy = uy - 2.0 * ur * s1;
+      const double ux = p.ux[i], uy = p.uy[i], ur = ux * c1 + uy * s1;
+      p.ux[i] = ux - 2.0 * ur * c1;
+      p.uy[i] = uy - 2.0 * ur * s1;
       x *= fr;
       y *= fr;
       polar(x, y, r1, c1, s1);
     }
+    p.x[i] = x; p.y[i] = y; p.z[i] = z;
     // rho^{n+1} at x^{n+1} (without the moving window; with it the deposit stage runs after
     // the injection)
     if (!WIN && dep.rho) deposit_at<MODES, true, false>(g, dep, invV, r1, c1, s1, z, w, 0.0, 0.0, 0.0);
@@ -835,12 +959,10 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(Parts p, int64_t np, Gri
       const double zn = __dsub_rn(__dadd_rn(__dadd_rn(zo, hz), hz), wa.shift ? g.dz : 0.0);
       if (below_zero(zn)) {   // left through the back edge: inactive from now on
         p.w[i] = 0.0;
-        ux = 0.0; uy = 0.0; uz = 0.0;
+        p.ux[i] = 0.0; p.uy[i] = 0.0; p.uz[i] = 0.0;
         win_mark(wa, p.id[i], i);
       }
     }
-    p.x[i] = x; p.y[i] = y; p.z[i] = z;
-    p.ux[i] = ux; p.uy[i] = uy; p.uz[i] = uz;
   }
 }
 
@@ -1118,12 +1240,6 @@ __device__ __forceinline__ float fx_value(int32_t hi, int32_t lo) {
 // Largest |w| and radial stencil range over particles [b0, b1) (all threads of the CTA;
 // non-finite weights raise the numeric error bit and count as 0); MOMENTA: the momenta are read
 // afterwards.
-// Starts the read of *p into L2.  The particle loop reads the arrays that the statistics pass does
-// not need only after a chain of dependent loads: with their lines requested here the push of 1.35 M
-// particles (2048 x 256, 2 modes) takes 160 us where it took 165, the rho deposit of 2.2 M 62.5 us
-// where it took 66.
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 template <bool MOMENTA>
 __device__ __forceinline__ ChunkStats chunk_stats(const PartsF& p, const GeomF& g, int64_t b0, int64_t b1,
                                                   ChunkStats* slot, int32_t* err) {
@@ -2326,9 +2442,13 @@ bool is_mixed(const Sim* s) { return s->cfg.precision != PIC_FP64; }
 template <int MODES> auto deposit_kernel64(const DepArgs& a) {
   return !a.J ? k_deposit<MODES, true, false> : !a.rho ? k_deposit<MODES, false, true> : k_deposit<MODES, true, true>;
 }
-template <int MODES> auto push_kernel64(bool win, bool dwg) {
-  return win ? (dwg ? k_gather_push<MODES, true, true> : k_gather_push<MODES, true, false>)
-             : (dwg ? k_gather_push<MODES, false, true> : k_gather_push<MODES, false, false>);
+template <int MODES, int CTAS> auto push_kernel64(bool win, bool dwg) {
+  return win ? (dwg ? k_gather_push<MODES, true, true, CTAS> : k_gather_push<MODES, true, false, CTAS>)
+             : (dwg ? k_gather_push<MODES, false, true, CTAS> : k_gather_push<MODES, false, false, CTAS>);
+}
+template <int CTAS> auto push_kernel64_nm(int nm, bool win, bool dwg) {
+  return nm <= 2 ? push_kernel64<2, CTAS>(win, dwg)
+                 : nm == 3 ? push_kernel64<3, CTAS>(win, dwg) : push_kernel64<4, CTAS>(win, dwg);
 }
 
 // Kernel instances of the mixed form by mode count (1..kMaxModes).
@@ -2580,7 +2700,7 @@ pic_status launch_gather_push(Sim* s, int32_t fuse_current, const WinArgs& wa, b
     const int threads = s->np < 152 * 1024 ? 128 : 256;
     const int grid = (int)((s->np + threads - 1) / threads);
     const bool win = wa.on != 0, dwg = ebdw != nullptr;
-    auto* kern = c.Nm <= 2 ? push_kernel64<2>(win, dwg) : c.Nm == 3 ? push_kernel64<3>(win, dwg) : push_kernel64<4>(win, dwg);
+    auto* kern = s->np <= 152 * 512 ? push_kernel64_nm<2>(c.Nm, win, dwg) : push_kernel64_nm<3>(c.Nm, win, dwg);
     kern<<<grid, threads, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s), fuse_current, err, wa);
   }
   PIC_LAUNCHED(s);
