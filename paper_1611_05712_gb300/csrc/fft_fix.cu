@@ -388,18 +388,18 @@ template <bool SHORT> __device__ __forceinline__ void row_or(unsigned* word, uns
   }
 }
 
-// T threads transform 8 T / N rows (at least one).
+// A CTA of up to T threads transforms 8 threads / N rows (at least one).
 template <bool INV, int T, bool SHORT>
 __global__ void __launch_bounds__(T, 1024 / T) k_fft_fix_pow2(const __grid_constant__ FixArgs A, int lgN) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kMaxRows = SHORT ? T : T / 32;   // a row takes one thread at least (N >= 8), or a warp
   __shared__ unsigned top[kMaxRows], bits[5][kMaxRows];
   const int TR = A.N >> 3, lr = threadIdx.x / TR, tr = threadIdx.x - lr * TR;
-  const int rpc = T / TR, row = blockIdx.x * rpc + lr;
+  const int rpc = blockDim.x / TR, row = blockIdx.x * rpc + lr;
   const bool active = row < A.rows;
   fx2* buf = reinterpret_cast<fx2*>(smem_raw) + (size_t)lr * (A.N + (A.N >> 3));
   RowIO io = row_io(A, active ? row : 0);
-  for (int i = threadIdx.x; i < rpc; i += T) {
+  for (int i = threadIdx.x; i < rpc; i += blockDim.x) {
     top[i] = 0;
 #pragma unroll
     for (int p = 0; p < 5; ++p) bits[p][i] = 0;
@@ -570,12 +570,16 @@ template <bool INV> void launch(Sim* s, const FixArgs& A) {
     int lgN = 0;
     while ((1 << lgN) < N) ++lgN;
     const int T = N <= 2048 ? 256 : N >> 3;
-    const int rpc = T / (N >> 3), grid = (A.rows + rpc - 1) / rpc;
+    // few short rows: smaller CTAs, down to 64 threads, until there are two for each SM (512 rows of
+    // 256 points: @@)
+    int t = T;
+    while (t > 64 && t > N >> 3 && (int64_t)A.rows * (N >> 3) < (int64_t)t * 2 * 152) t >>= 1;
+    const int rpc = t / (N >> 3), grid = (A.rows + rpc - 1) / rpc;
     auto* k = N < 256    ? k_fft_fix_pow2<INV, 256, true>
               : T == 256 ? k_fft_fix_pow2<INV, 256, false>
               : T == 512 ? k_fft_fix_pow2<INV, 512, false>
                          : k_fft_fix_pow2<INV, 1024, false>;
-    k<<<grid, T, pow2_smem(N, T), s->stream>>>(A, lgN);
+    k<<<grid, t, pow2_smem(N, t), s->stream>>>(A, lgN);
   } else if (N <= 2048) {
     k_fft_fix_rows<INV, 256><<<A.rows, 256, rows_smem(N), s->stream>>>(A);
   } else {
