@@ -570,8 +570,9 @@ template <bool INV> void launch(Sim* s, const FixArgs& A) {
     int lgN = 0;
     while ((1 << lgN) < N) ++lgN;
     const int T = N <= 2048 ? 256 : N >> 3;
-    // few short rows: smaller CTAs, down to 64 threads, until there are two for each SM (512 rows of
-    // 256 points: @@)
+    // few short rows: smaller CTAs, down to 64 threads, until there are two for each SM (512 and 768
+    // rows of 256 points: 19.5 -> 18.2 and 25.7 -> 24.8 us; 32 threads give no more: a thread's own
+    // chain of three passes over 8 points is what is left)
     int t = T;
     while (t > 64 && t > N >> 3 && (int64_t)A.rows * (N >> 3) < (int64_t)t * 2 * 152) t >>= 1;
     const int rpc = t / (N >> 3), grid = (A.rows + rpc - 1) / rpc;
