@@ -1,15 +1,11 @@
-// Double-word arithmetic: a float64-accurate number as an unevaluated sum of two floats.
-//
-// GB300 runs float64 at 1/64 of its float32 rate, and the FP64 form's row FFT was bound by
-// the float64 unit.  Its butterflies run on the float32 units with each real number an
-// unevaluated sum of two floats, hi + lo with |lo| <= ulp(hi)/2: about 48 significant bits
-// (double-word arithmetic after Dekker, Numer. Math. 18, 1971, with error-free products
-// from fused multiply-adds).  Sum: the exact sum of the high parts (Knuth's two-sum) plus
-// the low parts, renormalised: error below 2u^2 (|x| + |y|), u = 2^-24, an absolute error
-// of the kind an FFT's error bound is made of.  Product: the exact product of the high
-// parts (one fma) plus the cross terms: error below a few u^2 |x y|.  Grids stay doubles
-// in memory; the conversions use integer operations and, on the way out, one float64
-// addition per value.
+// Double-word arithmetic: a number as an unevaluated sum of two floats, hi + lo with |lo| <=
+// ulp(hi)/2, about 48 significant bits (after Dekker, Numer. Math. 18, 1971, with error-free
+// products from fused multiply-adds).  GB300 runs float64 at 1/64 of its float32 rate; the FP64
+// form's gather of E and B from grids of power-of-two rows runs on the float32 units this way.
+// Sum: the exact sum of the high parts (Knuth's two-sum) plus the low parts, renormalised: error
+// below 2u^2 (|x| + |y|), u = 2^-24.  Product: the exact product of the high parts (one fma) plus
+// the cross terms: error below a few u^2 |x y|.  The conversions to and from float64 use integer
+// operations.
 #pragma once
 
 #include <stdint.h>
@@ -20,11 +16,7 @@ struct dw {
   float hi, lo;
   dw() = default;
   __host__ __device__ constexpr dw(float h, float l) : hi(h), lo(l) {}
-  __host__ __device__ constexpr explicit dw(int v) : hi((float)v), lo(0.f) {}
   dw(double) = delete;   // a double converts through dw_from_double, never through int
-};
-struct dw2 {
-  dw x, y;
 };
 
 __device__ __forceinline__ float dw_neg_if(float v, bool neg) {
@@ -107,9 +99,5 @@ __device__ __forceinline__ double dw_widen(float f) {
   }
   return __longlong_as_double((long long)d);
 }
-__device__ __forceinline__ double dw_to_double(dw v) { return dw_widen(v.hi) + dw_widen(v.lo); }
-__device__ __forceinline__ dw& operator+=(dw& x, dw y) { return x = x + y; }
-__device__ __forceinline__ dw& operator-=(dw& x, dw y) { return x = x - y; }
-__device__ __forceinline__ dw& operator*=(dw& x, dw y) { return x = x * y; }
 
 }  // namespace pic
