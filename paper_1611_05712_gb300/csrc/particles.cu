@@ -378,7 +378,9 @@ struct GatherNodesDw {
   bool ghost;
 };
 
-__device__ __forceinline__ GatherNodesDw gather_nodes_dw(const GridGeom& g, const Stencil62& st) {
+__device__ __forceinline__ GatherNodesDw gather_nodes_dw(const GridGeom& g, double z, double r) {
+  const Stencil62 st = stencil62(g, z, r);
+  const bool finite = is_finite(r);   // x^2 + y^2 may overflow: NaN weights, as from the float64 stencil
   GatherNodesDw gn;
   const Sf z0 = sf_fraction(kOne62 - st.fz), z1 = sf_fraction(st.fz);
   const Sf r0 = sf_fraction(kOne62 - st.fr), r1 = sf_fraction(st.fr);
@@ -388,6 +390,7 @@ __device__ __forceinline__ GatherNodesDw gather_nodes_dw(const GridGeom& g, cons
     const int j = st.j0 + dj;
     const bool keep = j < g.Nr;
     gn.w[n] = keep ? dw_weight((dz ? z1 : z0) * (dj ? r1 : r0)) : dw(0.f, 0.f);
+    if (!finite) gn.w[n] = dw(__int_as_float(0x7fffffff), __int_as_float(0x7fffffff));
     gn.off[n] = (unsigned)(j < 0 || !keep ? 0 : j) * g.Nz + (dz ? st.i1 : st.i0);
   }
   gn.ghost = st.j0 < 0;
@@ -741,7 +744,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     v[2] = sf_from(vz);
   }
   // a NaN or an infinity among the factors makes every product of the particle NaN
-  if (!is_finite(w) || !is_finite(a.q) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
+  if (!is_finite(w) || !is_finite(a.q) || !is_finite(r) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
   {
     double er = c, ei = s;
 #pragma unroll
@@ -873,7 +876,7 @@ __global__ void __launch_bounds__(256, CTAS) k_gather_push(Parts p, int64_t np, 
     // and the ghost nodes (n = 0, 2) are summed apart so that the fold is one sign flip.
     double F[6];   // E_r, E_t, E_z, B_r, B_t, B_z
     if constexpr (DWG) {
-      gather_dw(g, gather_nodes_dw(g, stencil62(g, z, r)), c, s, EBdw, F);
+      gather_dw(g, gather_nodes_dw(g, z, r), c, s, EBdw, F);
     } else {
     const GatherNodes gn = gather_nodes(g, stencil(g, z, r));
 #pragma unroll

@@ -64,3 +64,21 @@ def test_weights_at_cell_edges(Nz, Nr, dz, dr):
     s.close()
     for k in ("ux", "uy", "uz"):
         assert rel_err(got[k], st.p[k]) < tol + 2.0 ** -44, k
+
+
+def test_radius_that_overflows():
+    """x^2 + y^2 beyond the largest float64: the weights are NaN, at the axis row, and so is the push."""
+    Nz, Nr, dz = 64, 16, 0.05e-6
+    P = {k: np.zeros(3) for k in ("ux", "uy", "uz")}
+    P.update(x=np.array([dz, 1e200, 3 * dz]), y=np.zeros(3), z=np.array([2.3, 20.4, 40.5]) * dz, w=np.ones(3),
+             id=np.arange(3, dtype=np.int32))
+    s = bd.Sim(bd.make_config(Nz, Nr, 2, dz, dz, dz / O.C_LIGHT, 0, True, bd.PIC_FP64, 3))
+    s.write_particles(P)
+    s.deposit(bd.PIC_DEP_RHO)
+    want = np.zeros((Nr, Nz), bool)
+    want[0, 20:22] = True
+    assert np.array_equal(np.isnan(s.get("DEP")[0]).any(axis=0), want)
+    s.gather_push(fuse_current=False)
+    got = s.read_particles()
+    s.close()
+    assert np.array_equal(np.isnan(got["ux"]), P["x"] == 1e200)
