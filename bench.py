@@ -46,9 +46,6 @@ def fp64_particle_flops(Nm):
     dep_rho = 7 + 7 + 8 + ph + 1 + 2 * (Nm - 1) + 8 * (2 * Nm - 1)
     return gather + push + dep_j + dep_rho
 FP64_PROBE_TFLOPS = 1.1947                     # FMA-loop probe on this machine's GB300 at 1987 MHz
-# DRAM bytes per FP64 DHT launch (k_gemm<double>) on this workload, from one ncu capture of
-# the current kernel (forward 71.42 + 27.50 MB, inverse 106.87 + 60.50 MB, mean of the two)
-DHT_F64_TRAFFIC_BYTES = (71.424 + 27.501568 + 106.872064 + 60.499968) / 2 * 1e6
 # DRAM bytes of one k_gather_push_f32<2, false, true> launch at cfg2 (dram__bytes_read.sum +
 # dram__bytes_write.sum, profiles/k_gather_push_f32__wake_2048x256_m2_mixed.md)
 PUSH_F32_TRAFFIC_BYTES = (148.361984 + 45.164544) * 1e6
@@ -362,25 +359,17 @@ def measure(args, w, P, npl, beams, prec, dist, dev, world, local):
                     "kernel": "k_dht_tc<BF16x6> (6 BF16 split products on tcgen05)",
                     "peak_source": f"{pk['source']}: bf16 sustained {pk['bf16_sustained']} TFLOP/s",
                     "share_of_step": share}
-    elif w.Nr <= 256:
-        # FP64 form, sliced path: 28 BF16 slice products per algorithmic multiply-add on the
-        # tensor cores (executed against the measured BF16 peak), FP64-equivalent rate beside
-        roofline = {"bound": "tensor", "achieved": 28 * achieved, "peak": pk["bf16_sustained"], "unit": "TFLOP/s",
-                    "frac": 28 * achieved / pk["bf16_sustained"], "traffic": None,
+    else:
+        # FP64 form: 21 BF16 digit products (Nr <= 256; 36 beyond) per algorithmic multiply-add on
+        # the tensor cores (executed against the measured BF16 peak), FP64-equivalent rate beside
+        n_prod = 21 if w.Nr <= 256 else 36
+        roofline = {"bound": "tensor", "achieved": n_prod * achieved, "peak": pk["bf16_sustained"], "unit": "TFLOP/s",
+                    "frac": n_prod * achieved / pk["bf16_sustained"], "traffic": None,
                     "fp64_equivalent_tflops": achieved,
                     "fp64_equivalent_vs_fp64_peak": achieved / FP64_PEAK_TFLOPS,
-                    "kernel": "k_f64s_colmax + k_f64s_panel + k_dht_f64s (FP64 DHT from exact BF16 slices on tcgen05)",
+                    "kernel": "k_f64s_panel + k_dht_f64s (FP64 DHT from exact BF16 digits on tcgen05)",
                     "peak_source": f"{pk['source']}: bf16 sustained {pk['bf16_sustained']} TFLOP/s; FP64 SIMT peak "
                                    "derived 152 SMs x 4 FP64 flop/clk x 2070 MHz",
-                    "share_of_step": share}
-    else:
-        roofline = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                    "frac": achieved / FP64_PEAK_TFLOPS, "traffic": DHT_F64_TRAFFIC_BYTES,
-                    "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, mean of the "
-                                      "forward and inverse launch (profiles/k_gemm_f64__wake_2048x256_m2_fp64.md)",
-                    "kernel": "k_gemm<double> (forward and inverse DHT, FP64 SIMT)",
-                    "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2070 MHz (recipe nominal "
-                                   "1.25 TFLOP/s); FMA probe measured 1.195 TFLOP/s",
                     "share_of_step": share}
     roofline_particles = None
     if not mixed:
@@ -393,13 +382,13 @@ def measure(args, w, P, npl, beams, prec, dist, dev, world, local):
             "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
             "algorithmic_flops": flops, "flops_per_particle": fp64_particle_flops(w.Nm),
-            "kernel": "k_gather_push<false, true> (gather in double words, Boris push, J at x^{n+1/2}, "
-                      "rho at x^{n+1}; FP64)",
+            "kernel": "k_gather_push (gather in double words, Boris push, J at x^{n+1/2}, rho at x^{n+1}; FP64)",
             "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2070 MHz (recipe nominal 1.25 TFLOP/s)",
             "share_of_step": stage_ms["gather_push"] / sum(stage_ms.values()),
             "note": "operations counted in float64 as the algorithm states them; the kernel runs the gather's "
-                    "interpolation and mode sum in double words on the FP32 units and the rest on the FP64 "
-                    "pipe, the binding unit (profiles/k_gather_push__wake_2048x256_m2_fp64.md)"}
+                    "interpolation and mode sum in double words on the FP32 units, the stencils and the deposits' "
+                    "products on the integer units and the rest on the FP64 pipe "
+                    "(profiles/k_gather_push__wake_2048x256_m2_fp64.md)"}
     if mixed:
         # the particle kernel (gather, push, J and rho deposits) against the survey's
         # algorithmic bytes: 56 B per particle (FP32 cell-relative state read and written,
