@@ -48,7 +48,7 @@ def fp64_particle_flops(Nm):
 FP64_PROBE_TFLOPS = 1.1947                     # FMA-loop probe on this machine's GB300 at 1987 MHz
 # DRAM bytes of one k_gather_push_f32<2, false, true> launch at cfg2 (dram__bytes_read.sum +
 # dram__bytes_write.sum, profiles/k_gather_push_f32__wake_2048x256_m2_mixed.md)
-PUSH_F32_TRAFFIC_BYTES = (148.361984 + 45.164544) * 1e6
+PUSH_F32_TRAFFIC_BYTES = (145.056256 + 42.143488) * 1e6
 TF32_PER_BF16 = 1.1 / 2.25                     # nominal dense TF32 / BF16 tensor rates
 
 
