@@ -56,7 +56,7 @@ namespace pic {
 namespace {
 
 constexpr int kF64sM = 128;         // panel columns c per tile (TMEM lanes)
-constexpr int kF64sN = 64;          // matrix rows n per tile
+constexpr int kF64sN = 64;          // matrix rows n per tile, at most (F64sParams::nw)
 constexpr int kF64sAcc = 8;         // accumulators in TMEM (kF64sN columns each: all 512)
 constexpr int kF64sKC = 32;         // K elements per stage (one 64-byte swizzle row of BF16)
 constexpr int kF64sKBlock = 256;    // K elements between drains of the accumulators (exactness)
@@ -248,6 +248,7 @@ struct F64sMaps {
 
 struct F64sParams {
   int Nr, Nc, n_tiles, m_tiles, tiles_total;
+  int nw;            // matrix rows n of a tile: 64, or 32 or 16 where 64 would leave SMs without a tile
   int b0;            // first batch item of this launch
   int16_t mat[24];   // compact matrix index of each batch item
 };
@@ -260,7 +261,7 @@ struct F64sTile {
 __device__ __forceinline__ F64sTile f64s_tile(int t, const F64sParams& P) {
   const int nt = t % P.n_tiles;
   const int rest = t / P.n_tiles;
-  return F64sTile{rest / P.m_tiles, nt * kF64sN, (rest % P.m_tiles) * kF64sM};
+  return F64sTile{rest / P.m_tiles, nt * P.nw, (rest % P.m_tiles) * kF64sM};
 }
 
 // The issuing thread of warp W: the products of its accumulators over the digit pairs of one 16-K
@@ -295,12 +296,25 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
 
 __device__ __forceinline__ int acc_int(uint32_t r) { return __float2int_rn(__uint_as_float(r)); }
 
+// (double)v by integer operations (round to nearest, ties to even): the conversion and the test for
+// zero ran on the float64 unit, 4 us of a tile's epilogue where no other tile's products hide it.
+__device__ __forceinline__ double to_double_rn(long long v) {
+  const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+  if (a == 0ull) return 0.0;
+  const int lz = __clzll((long long)a);
+  const unsigned long long t = a << lz, rest = t & 0x7ffull;
+  unsigned long long r = t >> 11;   // 53 bits; the leading one carries into the exponent
+  r += rest > 0x400ull || (rest == 0x400ull && (r & 1ull)) ? 1ull : 0ull;
+  return __longlong_as_double((long long)((((unsigned long long)(1085 - lz)) << 52) + r) |
+                              (v < 0 ? (long long)0x8000000000000000ull : 0ll));
+}
+
 // y = t 2^k (t a float64 near an integer), the scaling as an addition to the exponent field
 // while the result stays normal.
 __device__ __forceinline__ double scale_pow2(double t, int k) {
   const long long bits = __double_as_longlong(t);
   const int ex = (int)((bits >> 52) & 0x7ff) + k;
-  if (t != 0.0 && ex > 0 && ex < 2047) return __longlong_as_double(bits + (long long)k * (1LL << 52));
+  if ((bits << 1) != 0 && ex > 0 && ex < 2047) return __longlong_as_double(bits + (long long)k * (1LL << 52));
   return t * ldexp(1.0, k);   // zero, or a result outside the normal range
 }
 
@@ -350,8 +364,8 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  // kind::f16: D f32, A and B bf16, both K-major; N = 64, M = 128
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kF64sN >> 3) << 17) |
+  // kind::f16: D f32, A and B bf16, both K-major; N = nw, M = 128
+  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.nw >> 3) << 17) |
                          ((uint32_t)(kF64sM >> 4) << 24);
 
   auto fail = [&]() {
@@ -438,7 +452,7 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
     // four warps per TMEM lane quarter (warp % 4 == q: lanes 32q .. 32q + 31), each taking
     // a quarter of the tile's columns
     constexpr int kCols = kF64sN / 4;
-    const int q = warp & 3, jh = ((warp - 4) >> 2) * kCols;
+    const int cols = P.nw / 4, q = warp & 3, jh = ((warp - 4) >> 2) * cols;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)jh;
     uint32_t i = 0;
     bool ok = true;
@@ -456,6 +470,7 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
         for (int j = 0; j < kCols; j += 4) {
+          if (j >= cols) break;
           uint32_t r[kF64sAcc][4];
 #pragma unroll
           for (int a = 0; a < kF64sAcc; ++a) tmem_ld4(taddr + a * kF64sN + j, r[a]);
@@ -494,14 +509,14 @@ __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sP
 #pragma unroll
         for (int e = 0; e < kCols; ++e) {
           const int n = n0 + e;
-          if (n < P.Nr) {
+          if (e < cols && n < P.Nr) {
             double v;
             int k = Ec + rexp[n];
             if constexpr (S == kF64sDigits) {
-              v = (double)hi[e];
+              v = to_double_rn(hi[e]);
               k -= 54;
             } else {
-              v = fma((double)lo[e], 0x1p-32, (double)hi[e]);   // exact conversions, one rounding
+              v = fma(to_double_rn(lo[e]), 0x1p-32, to_double_rn(hi[e]));   // exact conversions, one rounding
               k -= 36;
             }
             Y[(size_t)n * P.Nc + c] =
@@ -616,6 +631,12 @@ pic_status launch_items(Sim* s, const DhtBatch& b, F64sParams P, int items) {
   F64sMaps maps;
   maps.panel = s->f64s_maps[0];
   maps.mats = s->f64s_maps[1];
+  // narrower tiles while all of them still find an SM at once (256 x 64 x 2 modes, 32 and 48 tiles of
+  // 64 rows: 17.3 -> 12.5 us a launch with 16 and 32 rows and the epilogue off the float64 unit)
+  P.nw = kF64sN;
+  const auto tiles = [&](int nw) { return (Nr + nw - 1) / nw * P.m_tiles * items; };
+  while (P.nw > 16 && tiles(P.nw / 2) <= dht_tc_sm_count()) P.nw /= 2;
+  P.n_tiles = (Nr + P.nw - 1) / P.nw;
   P.tiles_total = P.n_tiles * P.m_tiles * items;
   const int grid = std::min(P.tiles_total, dht_tc_sm_count());
   k_dht_f64s<S><<<grid, kF64sThreads, f64s_smem<S>(), s->stream>>>(b, P, maps, colexp,
@@ -638,7 +659,6 @@ pic_status launch_dht_f64s(Sim* s, const DhtBatch& b) {
   F64sParams P{};
   P.Nr = s->cfg.Nr;
   P.Nc = 2 * s->cfg.Nz;
-  P.n_tiles = (P.Nr + kF64sN - 1) / kF64sN;
   P.m_tiles = (P.Nc + kF64sM - 1) / kF64sM;
   for (int i = 0; i < b.n; ++i) {
     const int id = b.mat[i], per = kMaxModes * 3;
