@@ -734,12 +734,13 @@ template <typename C2> struct MixedIO {
   decltype(C2{}.x) scale;
 };
 
-template <typename C2, bool INV, int R, bool FIRST, bool LAST>
+template <typename C2, bool INV, bool COMP, int R, bool FIRST, bool LAST>
 __device__ __forceinline__ void mixed_pass(const C2* __restrict__ src, C2* __restrict__ dst,
                                            const C2* __restrict__ twp, const MixedIO<C2>& io, int N, int L) {
   const int NR = N / R;
   const float invL = 1.0f / (float)L;
-  for (int t = threadIdx.x; t < NR; t += blockDim.x) {
+  const int step = COMP ? blockDim.x : 256;   // a constant keeps the plain radices in 48 registers
+  for (int t = threadIdx.x; t < NR; t += step) {
     // j = t / L, k = t mod L (t, L < 2^13: the float quotient is off by at most one)
     int j = (int)((float)t * invL);
     int k = t - j * L;
@@ -779,37 +780,38 @@ __device__ __forceinline__ void mixed_pass(const C2* __restrict__ src, C2* __res
   }
 }
 
-template <typename C2, bool INV, bool FIRST, bool LAST>
+template <typename C2, bool INV, bool COMP, bool FIRST, bool LAST>
 __device__ __forceinline__ void mixed_pass_r(int Rdx, const C2* src, C2* dst, const C2* __restrict__ twp,
                                              const MixedIO<C2>& io, int N, int L) {
-  if constexpr (sizeof(io.scale) == 4) {   // the float plans' products of radices
+  if constexpr (COMP) {   // the float plans' products of radices
     switch (Rdx) {
-      case 6: mixed_pass<C2, INV, 6, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 9: mixed_pass<C2, INV, 9, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 10: mixed_pass<C2, INV, 10, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 12: mixed_pass<C2, INV, 12, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 14: mixed_pass<C2, INV, 14, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 15: mixed_pass<C2, INV, 15, FIRST, LAST>(src, dst, twp, io, N, L); return;
-      case 16: mixed_pass<C2, INV, 16, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 6: mixed_pass<C2, INV, COMP, 6, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 9: mixed_pass<C2, INV, COMP, 9, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 10: mixed_pass<C2, INV, COMP, 10, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 12: mixed_pass<C2, INV, COMP, 12, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 14: mixed_pass<C2, INV, COMP, 14, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 15: mixed_pass<C2, INV, COMP, 15, FIRST, LAST>(src, dst, twp, io, N, L); return;
+      case 16: mixed_pass<C2, INV, COMP, 16, FIRST, LAST>(src, dst, twp, io, N, L); return;
       default: break;
     }
   }
   switch (Rdx) {
-    case 2: mixed_pass<C2, INV, 2, FIRST, LAST>(src, dst, twp, io, N, L); break;
-    case 3: mixed_pass<C2, INV, 3, FIRST, LAST>(src, dst, twp, io, N, L); break;
-    case 4: mixed_pass<C2, INV, 4, FIRST, LAST>(src, dst, twp, io, N, L); break;
-    case 5: mixed_pass<C2, INV, 5, FIRST, LAST>(src, dst, twp, io, N, L); break;
-    case 7: mixed_pass<C2, INV, 7, FIRST, LAST>(src, dst, twp, io, N, L); break;
-    default: mixed_pass<C2, INV, 8, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    case 2: mixed_pass<C2, INV, COMP, 2, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    case 3: mixed_pass<C2, INV, COMP, 3, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    case 4: mixed_pass<C2, INV, COMP, 4, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    case 5: mixed_pass<C2, INV, COMP, 5, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    case 7: mixed_pass<C2, INV, COMP, 7, FIRST, LAST>(src, dst, twp, io, N, L); break;
+    default: mixed_pass<C2, INV, COMP, 8, FIRST, LAST>(src, dst, twp, io, N, L); break;
   }
 }
 
-template <typename R, bool INV>
+// COMP: room for the composite radices, which take more registers (64, four CTAs an SM); plans
+// without them are faster in the other instance.
+template <typename R, bool INV, bool COMP>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
-                                                                             typename Vec2<R>::T* __restrict__ out,
-                                                                             const typename Vec2<R>::T* __restrict__ twp,
-                                                                             RowCombine rc, FftPlan plan,
-                                                                             int rows_per_comp) {
+                                                                typename Vec2<R>::T* __restrict__ out,
+                                                                const typename Vec2<R>::T* __restrict__ twp,
+                                                                RowCombine rc, FftPlan plan, int rows_per_comp) {
   using C2 = typename Vec2<R>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = plan.N;
@@ -832,22 +834,22 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_fft_rows(const 
   for (int p = 0; p < kMaxRadixPasses; ++p) radix |= (unsigned long long)((plan.radix[p] - 1) & 15) << (4 * p);
   const int np = plan.n_pass;
   if (np == 1) {
-    mixed_pass_r<C2, INV, true, true>((int)(radix & 15) + 1, buf0, buf1, twp, io, N, 1);
+    mixed_pass_r<C2, INV, COMP, true, true>((int)(radix & 15) + 1, buf0, buf1, twp, io, N, 1);
     return;
   }
-  mixed_pass_r<C2, INV, true, false>((int)(radix & 15) + 1, buf0, buf0, twp, io, N, 1);
+  mixed_pass_r<C2, INV, COMP, true, false>((int)(radix & 15) + 1, buf0, buf0, twp, io, N, 1);
   __syncthreads();
   C2* src = buf0;
   C2* dst = buf1;
   int L = (int)(radix & 15) + 1;
   for (int p = 1; p < np - 1; ++p) {
     const int Rp = (int)((radix >> (4 * p)) & 15) + 1;
-    mixed_pass_r<C2, INV, false, false>(Rp, src, dst, twp, io, N, L);
+    mixed_pass_r<C2, INV, COMP, false, false>(Rp, src, dst, twp, io, N, L);
     __syncthreads();
     C2* t2 = src; src = dst; dst = t2;
     L *= Rp;
   }
-  mixed_pass_r<C2, INV, false, true>((int)((radix >> (4 * (np - 1))) & 15) + 1, src, dst, twp, io, N, L);
+  mixed_pass_r<C2, INV, COMP, false, true>((int)((radix >> (4 * (np - 1))) & 15) + 1, src, dst, twp, io, N, L);
 }
 
 // ---- any other length: Bluestein's chirp-z algorithm ----
@@ -873,6 +875,12 @@ int bluestein_length(int Nz, int precision) {
 
 namespace {
 
+bool composite_plan(const int* radix, int n_pass) {
+  for (int i = 0; i < n_pass; ++i)
+    if (radix[i] == 6 || radix[i] > 8) return true;
+  return false;
+}
+
 // The factorisation of a 7-smooth length into the fewest radices (any needs fewer than
 // kMaxRadixPasses), in falling order, and among those the one of the smallest first radix.
 struct RadixSearch {
@@ -896,20 +904,26 @@ struct RadixSearch {
 
 }  // namespace
 
-// Factor Nz into passes (the Stockham order is free).  FP64 rows: radices 8, 4, 2, 3, 5, 7.
-// Float rows of lengths that are no powers of two: the fewest passes of radices up to 16 (each
-// pass costs about as many instructions for indices, twiddles and the exchange as for its
-// butterflies), and among those the smallest largest radix; the pass whose radix shares the
-// smallest power of two with the shared memory's 16 double banks comes first, since its stores
-// step by the radix (odd radices meet no bank conflicts).
-bool plan_radix(int N, int precision, int32_t* radix, int32_t* n_pass) {
+// Factor Nz into passes (the Stockham order is free): radices 8, 4, 2, 3, 5, 7, or, for float rows of
+// lengths that are no powers of two, the fewest passes of radices up to 16 (each pass costs about as
+// many instructions for indices, twiddles and the exchange as for its butterflies), and among
+// those the smallest largest radix; the pass whose radix shares the smallest power of two with the
+// shared memory's 16 double banks comes first, since its stores step by the radix (odd radices meet no
+// bank conflicts).  A composite pass has fewer threads at work, which pays for short rows and where
+// the rows (4 Nm Nr in a forward transform) are twice as many as the SMs hold.  Field cycles of 70
+// lengths on 96 x 2 and 400 x 1 rows against radices up to 8 alone: 1.00 to 1.19 times as fast up to
+// 900 points, 0.98 to 1.08 (mean 1.03) beyond on the composite side of the line; on the other side
+// composites would take 0.90 to 1.17 (mean 0.98).
+bool plan_radix(int N, int precision, int64_t rows, int32_t* radix, int32_t* n_pass) {
   int n = N;
   for (int f : {2, 3, 5, 7})
     while (n > 1 && n % f == 0) n /= f;
   if (n != 1) return false;
   int k = 0;
   n = N;
-  if (precision == PIC_FP64 || (N & (N - 1)) == 0) {
+  const int64_t held = 152 * (int64_t)(227 * 1024 / (16 * N));   // rows on the SMs at once
+  const bool many = N <= 900 || rows >= 2 * held;
+  if (precision == PIC_FP64 || (N & (N - 1)) == 0 || !many) {
     for (int f : {8, 4, 2, 3, 5, 7})
       while (n % f == 0) {
         if (k >= kMaxRadixPasses) return false;
@@ -941,10 +955,12 @@ pic_status fft_configure_device() {
   std::lock_guard<std::mutex> lock(mu);
   if (dev >= 0 && dev < 64 && done[dev]) return PIC_OK;
   if (const pic_status st = fft_fix_configure_device()) return st;
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
-  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<double, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
+  PIC_CUDA(cudaFuncSetAttribute(k_fft_rows<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax));
   // power-of-two rows: one padded row buffer (float: staging areas as well)
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2_tma<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_tma_smem(8192)));
   PIC_CUDA(cudaFuncSetAttribute(k_fft_pow2_tma<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_tma_smem(8192)));
@@ -1091,19 +1107,22 @@ pic_status launch_fft_rows(Sim* s, const void* in, void* out, const RowCombine& 
   const size_t smem = 2 * (size_t)c.Nz * s->cplx_bytes;
   if (c.precision == PIC_FP64) {
     if (inverse) {
-      k_fft_rows<double, true><<<rows, 256, smem, s->stream>>>((const double2*)in, (double2*)out, tw, rc,
+      k_fft_rows<double, true, false><<<rows, 256, smem, s->stream>>>((const double2*)in, (double2*)out, tw, rc,
                                                                plan, rows_per_comp);
     } else {
-      k_fft_rows<double, false><<<rows, 256, smem, s->stream>>>((const double2*)in, (double2*)out, tw, rc,
+      k_fft_rows<double, false, false><<<rows, 256, smem, s->stream>>>((const double2*)in, (double2*)out, tw, rc,
                                                                 plan, rows_per_comp);
     }
   } else {
-    // as many threads as share the butterflies of the smallest radix evenly, at most 256
-    int least = plan.radix[0];
-    for (int i = 1; i < plan.n_pass; ++i) least = std::min(least, plan.radix[i]);
-    const int most = c.Nz / least, turns = (most + 255) / 256;
-    const int threads = std::max(64, ((most + turns - 1) / turns + 31) / 32 * 32);
-    auto* k = inverse ? k_fft_rows<float, true> : k_fft_rows<float, false>;
+    // plans of composite radices: as many threads as share the butterflies of the largest evenly, so
+    // that more rows fit an SM (against the smallest radix: 3 % to 10 % slower up to 1700 points)
+    int top = 0;
+    for (int i = 0; i < plan.n_pass; ++i) top = std::max(top, plan.radix[i]);
+    const bool comp = composite_plan(plan.radix, plan.n_pass);
+    const int few = c.Nz / top, turns = (few + 255) / 256;
+    const int threads = comp ? std::max(64, ((few + turns - 1) / turns + 31) / 32 * 32) : 256;
+    auto* k = comp ? (inverse ? k_fft_rows<float, true, true> : k_fft_rows<float, false, true>)
+                   : (inverse ? k_fft_rows<float, true, false> : k_fft_rows<float, false, false>);
     k<<<rows, threads, smem, s->stream>>>((const float2*)in, (float2*)out, twf, rc, plan, rows_per_comp);
   }
   PIC_LAUNCHED(s);

@@ -31,7 +31,7 @@ pic_status cuda_status(cudaError_t e, const char* what) {
   return PIC_ERR_CUDA;
 }
 
-bool plan_radix(int N, int precision, int32_t* radix, int32_t* n_pass);
+bool plan_radix(int N, int precision, int64_t rows, int32_t* radix, int32_t* n_pass);
 size_t diag_acc_doubles();
 pic_status launch_filter_copy(Sim* s, void* dst, const void* src);
 pic_status launch_scale_copy(Sim* s, void* dst, const void* src, double a, size_t n_cplx);
@@ -52,7 +52,7 @@ pic_status validate(const pic_config* c, int32_t* radix, int32_t* n_pass) {
     set_error("Nz=%d must be in [8, %d]%s", c->Nz, max_nz, max_nz == 4096 ? " (float64 rows of a length that is not a power of two)" : "");
     return PIC_ERR_ARG;
   }
-  if (!plan_radix(c->Nz, c->precision, radix, n_pass)) {
+  if (!plan_radix(c->Nz, c->precision, (int64_t)4 * c->Nm * c->Nr, radix, n_pass)) {
     *n_pass = 0;
     if (bluestein_length(c->Nz, c->precision) == 0) {
       set_error("Nz=%d is not 7-smooth: Bluestein lengths reach Nz <= %d", c->Nz, max_nz / 2);

@@ -43,3 +43,24 @@ def test_float_rows(Nz):
     # 4 times that; the matrices' products add about as much
     assert per_slice_err(fwd, np.stack(O.forward_sources(g, h, *dep))) < 3e-6
     assert per_slice_err(inv, np.stack(O.inverse_vector(g, h, *eh))) < 3e-6
+
+
+@pytest.mark.parametrize("Nz,Nr", [(1500, 700), (2187, 480), (3600, 320), (6300, 180), (7776, 160)])
+def test_float_rows_of_many(Nz, Nr):
+    """Beyond 900 points the composite radices need more rows than the SMs hold."""
+    g = O.Grid(Nz, Nr, 1, DZ, DZ, DZ / O.C_LIGHT)
+    s = bd.Sim(bd.make_config(Nz, Nr, 1, DZ, DZ, g.dt, 0, True, bd.PIC_MIXED_TF32X3, 0))
+    h = O.hankel_setup(g)
+    rng = np.random.default_rng(Nz)
+    dep = rng.normal(size=(4, 1, Nr, Nz)) + 1j * rng.normal(size=(4, 1, Nr, Nz))
+    eh = rng.normal(size=(3, 1, Nr, Nz)) + 1j * rng.normal(size=(3, 1, Nr, Nz))
+    s.set("DEP", dep)
+    s.forward_transform()
+    fwd = s.get("SRC_H")
+    s.set("EH", eh)
+    s.inverse_transform()
+    inv = s.get("E")
+    s.close()
+    # as above; the matrices' float products are sums of up to Nr terms here
+    assert per_slice_err(fwd, np.stack(O.forward_sources(g, h, *dep))) < 1e-5
+    assert per_slice_err(inv, np.stack(O.inverse_vector(g, h, *eh))) < 1e-5
