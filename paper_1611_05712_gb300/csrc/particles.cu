@@ -1281,10 +1281,7 @@ __device__ __forceinline__ ChunkStats chunk_stats(const PartsF& p, const GeomF& 
 
 // Band of a chunk of cell-sorted particles whose first and last cells are iz_first, iz_last:
 // rows from iz_first - 1 to iz_last + 2 (moves of up to half a cell per half step, and the
-// +1 node), at most tz_max rows, of which a chunk that fills them all spares the first (it takes
-// only particles that move back into it, where the last row takes all of the last cells' +1 nodes:
-// a parameter scan's pushes at 3 and 2 modes 775 -> 745 and 531 -> 516 us, 2048 x 256 at 2 modes
-// 160 -> 158); r nodes from the chunk's lowest stencil node - jmargin to
+// +1 node), at most tz_max rows; r nodes from the chunk's lowest stencil node - jmargin to
 // its highest + 1 + jmargin (at least 2, at most jw_max); particles whose nodes are not all
 // inside deposit to the global grids.  bound (bound0) is an upper bound of |x| over the
 // chunk's J (rho) contributions.
@@ -1307,9 +1304,8 @@ __device__ __forceinline__ BandF make_band(int32_t* smem, int iz_first, int iz_l
   const int S0 = min(max(46 - lg_chunk - e, -126), 126);
   int RS = JW * nwp;
   RS += (40 - RS % 32) % 32;   // RS mod 32 = 8
-  const int lead = span + 3 <= 1 << lg ? 1 : 0;
-  const int iz_lo = iz_first < lead ? g.Nz - 1 : iz_first - lead;
-  return BandF{smem, iz_lo, 1 << lg, lg, j_lo, JW, RS, ldexpf(1.f, S), ldexpf(1.f, S0)};
+  return BandF{smem, iz_first == 0 ? g.Nz - 1 : iz_first - 1, 1 << lg, lg, j_lo, JW, RS, ldexpf(1.f, S),
+               ldexpf(1.f, S0)};
 }
 
 // Zero a band (all threads of the CTA; 16-byte stores).
