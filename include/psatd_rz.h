@@ -356,7 +356,7 @@ pic_status pic_window_state(pic_sim* sim, pic_window_info* out);
  *   dht_n_tile: rows of the Hankel matrix per tensor-core tile of the DHT (16..256, a
  *               multiple of 16, capped at 128 in the BF16 form; 0 = the built-in rule: Nr
  *               split into the fewest tiles of <= 256 (TF32) or <= 128 (BF16) rows);
- *   band_chunk: cell-sorted particles per CTA of the deposit kernels, at most (512, 1024 or 2048),
+ *   band_chunk: cell-sorted particles per CTA of the deposit kernels (512, 1024 or 2048),
  *               which also sets how many grid rows a CTA's shared-memory band covers.
  * Neither changes the arithmetic of a DHT output (same K order, bit-identical results);
  * band_chunk changes the order of the float additions to the global grid only.

@@ -2512,8 +2512,8 @@ GatherPushKernel gather_push_kernel(int nm, bool win, bool rho) {
   }
 }
 
-// Shared-memory bands for the deposits: chunks of cell-sorted particles per CTA (at most 1024,
-// or the tuned size: a power of two) and a
+// Shared-memory bands for the deposits: chunks of cell-sorted particles per CTA (1024, or
+// the tuned size: a power of two) and a
 // band of ncomp components (all modes, 16 bytes per complex node) within kBandBudget, so
 // that two CTAs fit on an SM: 8 or 4 full z-rows when they fit, else 4 rows of as many r
 // nodes as fit (at least 16).  jmargin: r nodes a particle can move before it deposits.
@@ -2524,18 +2524,9 @@ struct BandPlan {
 };
 BandPlan band_plan(const Sim* s, int ncomp, int jmargin) {
   const pic_config& c = s->cfg;
-  int64_t chunk = s->tune_chunk > 0 ? s->tune_chunk : 1024;
+  const int64_t chunk = s->tune_chunk > 0 ? s->tune_chunk : 1024;
   int lg = 0;
   while ((int64_t(1) << lg) < chunk) ++lg;
-  // Up to three waves of CTAs (two per SM): chunks shortened so that the last wave is full.  Pushes
-  // of the sets of a parameter scan at 0.17, 0.8, 1.3, 1.4, 2.3, 2.5, 2.6 waves took 16.8, 67, 62,
-  // 77, 129, 262, 69 us and take 10.9, 59, 58, 78, 129, 237, 66; at 4.3 waves (2048 x 256, 2 modes)
-  // the additional bands cost more than the last wave (160 -> 167 us).
-  const int64_t slots = 2 * 152, waves = (s->np + slots * chunk - 1) / (slots * chunk);
-  if (waves >= 1 && waves <= 3) {
-    const int64_t even = ((s->np + slots * waves - 1) / (slots * waves) + 31) & ~int64_t(31);
-    chunk = std::min(chunk, std::max<int64_t>(even, 128));
-  }
   BandPlan bp{BandArgs{chunk, 0, 0, jmargin, lg}, 0};
   if (ncomp <= 0) return bp;
   // one r node of one row: re hi, re lo for every mode, im hi, im lo for the modes m >= 1,
