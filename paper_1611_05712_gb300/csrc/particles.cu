@@ -205,14 +205,35 @@ struct Sf {
   unsigned s;      // sign in bit 31
 };
 
-__device__ __forceinline__ Sf sf_from(double x) {   // subnormal x count as zero
+// Exponents outside a float64's range say what a product is: they add up, and each kind outweighs
+// as many of the kinds before it as a product has factors.  A product of kind kSfInf whose mantissa is
+// zero has a zero among its factors: NaN.
+constexpr int kSfZero = -100000, kSfInf = 10000000, kSfNan = 1 << 28, kSfNone = -(1 << 30);
+
+__device__ __forceinline__ Sf sf_from(double x) {   // x zero or normal
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ffu);
   Sf r;
   r.h = e ? (((hi & 0xfffffu) | 0x100000u) << 10) | (lo >> 22) : 0u;
   r.l = e ? (lo << 9) & 0x7fffffffu : 0u;
-  r.e = e ? e : -100000;   // products with zero fall out of the exponent range (sf_far)
+  r.e = e ? e : kSfZero;   // products with zero fall out of the exponent range (sf_far)
   r.s = hi & 0x80000000u;
+  return r;
+}
+
+// Zero for numbers of the smallest and the largest exponent, those that sf_from may not hold (and zero).
+__device__ __forceinline__ unsigned sf_end(double x) { return ((unsigned)__double2hiint(x) + 0x100000u) & 0x7fe00000u; }
+
+__device__ __forceinline__ Sf sf_from_end(double x) {   // any x (rare)
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), e = (hi >> 20) & 0x7ffu;
+  const unsigned long long f = ((unsigned long long)(hi & 0xfffffu) << 32) | lo;
+  Sf r = sf_from(x);
+  if (e == 0x7ffu) r.e = f ? kSfNan : kSfInf;
+  if (e == 0u && f != 0ull) {
+    const int n = __clzll((long long)f);
+    const unsigned long long m = f << (n - 2);
+    r = Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, 12 - n, r.s};
+  }
   return r;
 }
 
@@ -228,12 +249,12 @@ __device__ __forceinline__ Sf operator*(const Sf& a, const Sf& b) {
   return Sf{(unsigned)(p >> 31), (unsigned)p & 0x7fffffffu, a.e + b.e - 1022, a.s ^ b.s};
 }
 
-// sf_double of zero and of results outside the normal range (NaN factors: e is large).  In line: a
-// call here would have the kernels keep their values in memory around it.
+// sf_double of zero and of results outside the normal range.  In line: a call here would have the
+// kernels keep their values in memory around it.
 __device__ __forceinline__ double sf_far(unsigned long long m, int e, unsigned s) {
   unsigned long long r;
   if (e > 12) {
-    r = m == 0ull ? 0ull : e > 3000 ? 0x7ff8000000000000ull : 0x7ff0000000000000ull;
+    r = e > kSfNan / 2 || (e > kSfInf / 2 && m == 0ull) ? 0x7ff8000000000000ull : m == 0ull ? 0ull : 0x7ff0000000000000ull;
   } else {   // m 2^(e - 10) units of the subnormal numbers
     const int sh = 10 - e;
     r = sh < 64 && sh > 0 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
@@ -256,7 +277,7 @@ __device__ __forceinline__ Sf sf_fraction(unsigned long long w) {
   if (w == kOne62) --w;
   const int n = __clzll((long long)w);
   const unsigned long long m = w << (n - 2 & 63);
-  return Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, w == 0ull ? -100000 : 1024 - n, 0u};
+  return Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, w == 0ull ? kSfZero : 1024 - n, 0u};
 }
 
 // a with its mantissa's leading bit at 2^61 again (a is zero or a product: at least 2^55).
@@ -727,8 +748,24 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
   const size_t RZ = (size_t)g.Nr * g.Nz;
   const int rot = threadIdx.x & 3;
   const bool ghost = st.j0 < 0;
-  const Sf qw = sf_from(a.q) * sf_from(w);
-  Sf rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (0 for the dropped node Nr)
+  Sf v[3], qw = sf_from(a.q) * sf_from(w);   // velocity; charge
+  // one test for all factors that may be no normal number: a conversion that handles every number took
+  // 1 to 2 % of the push, a call of float64 products up to 12 % of a deposit; this costs nothing
+  unsigned ends = min(sf_end(a.q), sf_end(w));
+  if (CUR) {
+    const double vr = c * vx + s * vy, vt = c * vy - s * vx;
+    v[0] = sf_from(vr);
+    v[1] = sf_from(vt);
+    v[2] = sf_from(vz);
+    ends = min(ends, min(min(sf_end(vr), sf_end(vt)), sf_end(vz)));
+    if (ends == 0u) {
+      v[0] = sf_from_end(vr);
+      v[1] = sf_from_end(vt);
+      v[2] = sf_from_end(vz);
+    }
+  }
+  if (ends == 0u) qw = sf_from_end(a.q) * sf_from_end(w);
+  Sf rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (kSfNone for the dropped node Nr)
   int jn[2];   // their grid rows (the ghost node j = -1 is row 0)
 #pragma unroll
   for (int dj = 0; dj < 2; ++dj) {
@@ -736,15 +773,10 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     const bool keep = j < g.Nr;
     jn[dj] = (j < 0 || !keep) ? 0 : j;
     rad[dj] = sf_normal(sf_fraction(keep ? (dj ? st.fr : kOne62 - st.fr) : 0ull) * (sf_from(invV[jn[dj]]) * qw));
+    if (!is_finite(r)) rad[dj].e = kSfNan;
+    if (!keep) rad[dj].e = kSfNone;
   }
-  Sf v[3], pr[MODES > 1 ? MODES - 1 : 1], pi[MODES > 1 ? MODES - 1 : 1];   // velocity; e^{+i m theta}, m = 1 ..
-  if (CUR) {
-    v[0] = sf_from(c * vx + s * vy);
-    v[1] = sf_from(c * vy - s * vx);
-    v[2] = sf_from(vz);
-  }
-  // a NaN or an infinity among the factors makes every product of the particle NaN
-  if (!is_finite(w) || !is_finite(a.q) || !is_finite(r) || (CUR && !(is_finite(vx) && is_finite(vy) && is_finite(vz)))) rad[0].e = rad[1].e = 1 << 20;
+  Sf pr[MODES > 1 ? MODES - 1 : 1], pi[MODES > 1 ? MODES - 1 : 1];   // e^{+i m theta}, m = 1 ..
   {
     double er = c, ei = s;
 #pragma unroll
@@ -762,7 +794,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
   for (int q = 0; q < 4; ++q) {
     const int node = (q + rot) & 3, dz = node >> 1, dj = node & 1;
     const Sf gq = (dj ? rad[1] : rad[0]) * (dz ? z1 : z0);
-    if ((gq.h | gq.l) == 0u) continue;
+    if ((gq.h | gq.l) == 0u && gq.e < kSfInf / 2) continue;
     const size_t o = (size_t)(dj ? jn[1] : jn[0]) * g.Nz + (dz ? st.i1 : st.i0);
     const unsigned fold = ghost && dj == 0 ? 0x80000000u : 0u;   // the ghost node: fold signs apply
     auto add = [&](double2* grid, size_t at, const Sf& f, unsigned flip) {   // mode 0
