@@ -267,7 +267,7 @@ __device__ __forceinline__ double sf_double(unsigned long long m, int e, unsigne
   const int lz = __clz((int)(unsigned)(m >> 32));
   const unsigned long long r = ((m << (lz - 1)) + 0x200u) >> 10;   // 53 bits, rounded (2^53 carries on)
   const int ex = e + 2 - lz;                                       // exponent field of the result
-  if ((unsigned)(ex - 1) >= 2044u) return sf_far(m, e, s);
+  if ((unsigned)(ex - 1) >= 2046u) return sf_far(m, e, s);   // 2046: rounding up gives infinity
   return __hiloint2double((int)((unsigned)(r >> 32) + ((unsigned)(ex - 1) << 20) | s), (int)(unsigned)r);
 }
 

@@ -105,3 +105,21 @@ def test_factors_out_of_range(weights, momenta, q, Nm):
         # a result below the normal range is off by one or two of its units
         tol = np.broadcast_to((1e-12 * np.where(np.isfinite(m), m, 0.0))[..., None], e.shape) + 1e-323
         assert (np.abs(g[ok] - e[ok]) <= tol[ok]).all()
+
+
+@pytest.mark.parametrize("top", [2.0 ** 1022, 1.7e308, 2.0 ** 1021])
+def test_largest_results(top):
+    """Charges a node holds up to the largest float64: finite where the product is."""
+    # z on a row of nodes and r halfway between two radial nodes: two contributions of half the charge
+    r = 6.0 * D
+    inv_v = 1.0 / O.Grid(Nz, Nr, 1, D, D, D / O.C_LIGHT).cell_volume()
+    w = top / max(0.5 * inv_v[5:7])
+    P = {"x": np.array([r]), "y": np.zeros(1), "z": np.array([8 * D]), "ux": np.zeros(1), "uy": np.zeros(1),
+         "uz": np.zeros(1), "w": np.array([w]), "id": np.zeros(1, np.int32)}
+    s = bd.Sim(bd.make_config(Nz, Nr, 1, D, D, D / O.C_LIGHT, 0, True, bd.PIC_FP64, 1, q=1.0))
+    s.write_particles(P)
+    s.deposit(bd.PIC_DEP_RHO)
+    rho = s.get("DEP")[0, 0].real
+    s.close()
+    # r, r/dr and the products: a few ulps, as above
+    assert np.isfinite(rho).all() and (np.abs(rho[5:7, 8] / (0.5 * w * inv_v[5:7]) - 1) < 1e-13).all()
