@@ -287,14 +287,15 @@ __device__ __forceinline__ Sf sf_normal(const Sf& a) {
   return Sf{(unsigned)(m >> 31), (unsigned)m & 0x7fffffffu, a.e - n, a.s};
 }
 
-// A weight (a product of two fractions) as a double word: 24 bits cut, the rest rounded.
+// A weight (a product of two fractions, zero or at least 2^-124) as a double word: 24 bits cut, the rest
+// rounded.
 __device__ __forceinline__ dw dw_weight(const Sf& a) {
   const Sf p = sf_normal(a);
-  if (p.h == 0u || p.e < 960) return dw(0.f, 0.f);   // weights below 2^-63 count as zero
+  if (p.h == 0u) return dw(0.f, 0.f);
   const unsigned long long m = sf_mantissa(p);
-  const float lo = __uint2float_rn((unsigned)(m >> 6)  /* bits 37 .. 6 */);
-  return dw(__uint_as_float(((unsigned)(p.e - 896) << 23) | ((unsigned)(m >> 38) & 0x7fffffu)),
-            __fmul_rn(lo, __uint_as_float((unsigned)(p.e - 951) << 23)));
+  const unsigned scale = (unsigned)(p.e - 896) << 23;   // the leading bit's value as a float
+  const float lo = __fmul_rn(__uint2float_rn((unsigned)(m >> 6)), 0x1p-55f);   // bits 37 .. 6
+  return dw(__uint_as_float(scale | ((unsigned)(m >> 38) & 0x7fffffu)), __fmul_rn(lo, __uint_as_float(scale)));
 }
 
 // u = x / d >= 0 as i + f 2^-62 from the bits, with d's reciprocal in 64 bits: off by less than u
