@@ -148,8 +148,8 @@ const char* pic_last_error(void);
 
 /* Copy n particles in (replacing all): soa[0..6] = x, y, z, ux, uy, uz, w (float64),
  * id (int32).  on_host != 0: the pointers are host memory (copied synchronously);
- * else device pointers (stream-ordered copy).  z must lie in [0, Nz dz) and
- * x^2 + y^2 < (Nr dr)^2.  Errors: PIC_ERR_ARG (n > capacity or negative). */
+ * else device pointers (stream-ordered copy).  Every array holds n elements.  z must lie in
+ * [0, Nz dz) and x^2 + y^2 < (Nr dr)^2.  Errors: PIC_ERR_ARG (n > capacity or negative). */
 pic_status pic_write_particles(pic_sim* sim, const double* const soa[7], const int32_t* id,
                                int64_t n, int32_t on_host);
 

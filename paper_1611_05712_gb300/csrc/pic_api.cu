@@ -1,16 +1,19 @@
 // C ABI of libpsatd_rz.so (declared in include/psatd_rz.h): configuration checks,
 // workspace layout, and the order of the stages of one quasi-cylindrical PSATD PIC cycle
 // (section "Finite order pseudo-spectral solvers" of arXiv:1611.05712).
+#include <cuda.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <string>
 #include <utility>
 #include <vector>
 
+#include "array_range.cuh"
 #include "pic_internal.cuh"
 
 namespace pic {
@@ -708,19 +711,44 @@ double* stage_array(const Sim* s, int k) {
                                       : s->at<double>(s->lay.part[s->cur][k]);
 }
 
+using AddressRangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+
+AddressRangeFn address_range_fn() {
+  static std::once_flag once;
+  static AddressRangeFn fn = nullptr;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<AddressRangeFn>(p);
+  });
+  return fn;
+}
+
 // Whether a kernel of this handle may work on the caller's device arrays themselves: every array
-// given lies on the workspace's own device, apart from the workspace, and is aligned to its
-// elements (a copy by the runtime needs none of this).
-bool readable_in_place(const Sim* s, const double* const* soa, const int32_t* id) {
+// given lies with all its n elements in one allocation on the workspace's own device, apart from the
+// workspace, and is aligned to its elements.  Any other array goes through a copy by the runtime,
+// which needs none of this and refuses what it cannot reach.
+bool in_place(const Sim* s, const double* const* soa, const int32_t* id, int64_t n) {
   cudaPointerAttributes own, a;
-  if (cudaPointerGetAttributes(&own, s->ws) != cudaSuccess) { cudaGetLastError(); return false; }
+  CUdeviceptr base = 0;
+  size_t bytes = 0;
+  const AddressRangeFn range = address_range_fn();
+  if (!range || cudaPointerGetAttributes(&own, s->ws) != cudaSuccess) { cudaGetLastError(); return false; }
   for (int k = 0; k < 8; ++k) {
     const void* p = k < 7 ? (soa ? static_cast<const void*>(soa[k]) : nullptr) : static_cast<const void*>(id);
     if (!p) continue;
-    const char* c = static_cast<const char*>(p);
-    if (reinterpret_cast<uintptr_t>(p) % (k < 7 ? 8 : 4) || (c >= s->ws && c < s->ws + s->ws_bytes)) return false;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    if (a.type != cudaMemoryTypeDevice || a.device != own.device) return false;
+    const size_t size = k < 7 ? 8 : 4;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    if (at % size) return false;
+    if (!array_inside(static_cast<uintptr_t>(base), bytes, at, n, size)) {   // not in the previous array's allocation
+      if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+      if (a.type != cudaMemoryTypeDevice || a.device != own.device) return false;
+      if (range(&base, &bytes, static_cast<CUdeviceptr>(at)) != CUDA_SUCCESS) return false;
+      if (!array_inside(static_cast<uintptr_t>(base), bytes, at, n, size)) return false;
+    }
+    if (!array_apart(at, n, size, reinterpret_cast<uintptr_t>(s->ws), s->ws_bytes)) return false;
   }
   return true;
 }
@@ -741,7 +769,7 @@ pic_status pic_write_particles(pic_sim* sim, const double* const soa[7], const i
   const bool mixed = s->cfg.precision != PIC_FP64;
   for (int k = 0; k < 7 && n > 0; ++k)
     if (!soa[k]) { set_error("particle array %d is NULL", k); return PIC_ERR_ARG; }
-  const bool direct = n > 0 && !on_host && readable_in_place(s, soa, id);
+  const bool direct = n > 0 && !on_host && in_place(s, soa, id, n);
   double* staged[7];
   for (int k = 0; k < 7; ++k) staged[k] = stage_array(s, k);
   int32_t* ids = mixed ? s->at<int32_t>(s->lay.perm_tmp) : s->at<int32_t>(s->lay.pid[s->cur]);
@@ -841,7 +869,7 @@ pic_status pic_read_particles(pic_sim* sim, double* const soa[7], int32_t* id, i
   if (n < 0 || n > s->np) { set_error("n=%lld exceeds the %lld particles held", (long long)n, (long long)s->np); return PIC_ERR_ARG; }
   const cudaMemcpyKind kind = on_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   const bool mixed = s->cfg.precision != PIC_FP64;
-  if (n > 0 && !on_host && readable_in_place(s, soa, id)) {
+  if (n > 0 && !on_host && in_place(s, soa, id, n)) {
     pic_status st = launch_particles_out(s, soa, id, n);
     return st != PIC_OK ? st : pic_sync(sim);
   }
