@@ -544,9 +544,12 @@ bool f64s_supported(const pic_config& c) { return c.precision == PIC_FP64 && c.N
 
 int f64s_digits(const pic_config& c) { return c.Nr <= kF64sMaxNr ? kF64sDigits : kF64sDigitsWide; }
 
-// Items whose panel planes the workspace holds at a time.  The wide form's planes are twice the
-// panels' bytes: a launch takes as many items as fit 1 GB (all 12 of a 2-mode run up to
-// 2048 x 1024), so that they stay a small part of the workspace at any size.
+// Items whose panel planes are held at a time.  The wide form's planes are twice the panels' bytes: a
+// launch takes as many items as fit 1 GB (all 12 of a 2-mode run up to 2048 x 1024).  The planes share
+// their memory with the spare particle buffer, so only handles of few particles a cell grow with them (by up
+// to a third, at 1800 x 400 x 2 without particles).  Fewer items a launch cost more than they save: field
+// cycles at 1800 x 400 x 2 and 4096 x 512 x 3 take 1.98 and 7.59 ms at 1 GB, 2.03 and 7.89 at 256 MB, 2.30
+// and 9.06 at 64 MB (last waves of tiles).
 int f64s_items(const pic_config& c) {
   const size_t item = (size_t)f64s_digits(c) * 2 * c.Nz * f64s_pitch(c.Nr) * 2;
   const int all = 6 * c.Nm;
@@ -615,8 +618,9 @@ pic_status f64s_make_maps(Sim* s) {
     set_error("cuTensorMapEncodeTiled failed (%d) for the sliced %s", (int)r, what);
     return PIC_ERR_CUDA;
   };
-  const pic_status st = make(0, s->lay.f64s_panel, Nc, f64s_items(s->cfg) * S, kF64sM, "panels");
-  return st != PIC_OK ? st : make(1, s->lay.f64s_mat, Nr, 6 * s->cfg.Nm * S, kF64sN, "matrices");
+  for (int b = 0; b < 2; ++b)
+    if (const pic_status st = make(b, s->lay.f64s_panel[b], Nc, f64s_items(s->cfg) * S, kF64sM, "panels")) return st;
+  return make(2, s->lay.f64s_mat, Nr, 6 * s->cfg.Nm * S, kF64sN, "matrices");
 }
 
 namespace {
@@ -626,11 +630,11 @@ pic_status launch_items(Sim* s, const DhtBatch& b, F64sParams P, int items) {
   const int Nr = P.Nr, Nc = P.Nc;
   int32_t* colexp = s->at<int32_t>(s->lay.f64s_colexp);
   k_f64s_panel<S><<<dim3(blocks_for(Nc, kPanelC), items), 256, 0, s->stream>>>(
-      b, P.b0, Nr, Nc, f64s_pitch(Nr), colexp, s->at<uint16_t>(s->lay.f64s_panel));
+      b, P.b0, Nr, Nc, f64s_pitch(Nr), colexp, s->at<uint16_t>(s->lay.f64s_panel[s->cur]));
   PIC_LAUNCHED(s);
   F64sMaps maps;
-  maps.panel = s->f64s_maps[0];
-  maps.mats = s->f64s_maps[1];
+  maps.panel = s->f64s_maps[s->cur];
+  maps.mats = s->f64s_maps[2];
   // narrower tiles while all of them still find an SM at once (256 x 64 x 2 modes, 32 and 48 tiles of
   // 64 rows: 17.3 -> 12.5 us a launch with 16 and 32 rows and the epilogue off the float64 unit)
   P.nw = kF64sN;

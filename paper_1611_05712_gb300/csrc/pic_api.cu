@@ -107,6 +107,11 @@ Layout make_layout(const pic_config& c) {
   L.svd_v = take((size_t)c.Nm * 3 * Nr2 * 8);
   L.svd_d = take((size_t)c.Nm * 3 * c.Nr * 8);
   L.pinv = take(pinv_scratch_bytes(c));
+  const size_t S = (size_t)f64s_digits(c), pitch16 = (size_t)split_pitch_b16(c.Nr), nmat = 6 * (size_t)c.Nm;
+  if (!mixed) {   // the matrices' digit planes take the place of the pseudo-inverses' scratch
+    L.f64s_mat = L.svd_w;
+    off = std::max(off, L.f64s_mat + ((nmat * S * c.Nr * pitch16 * 2 + 255) & ~(size_t)255));
+  }
   L.kzmod = take((size_t)c.Nz * 8);
   L.tz = take((size_t)c.Nz * 8);
   L.tr = take((size_t)c.Nm * c.Nr * 8);
@@ -124,14 +129,6 @@ Layout make_layout(const pic_config& c) {
       L.chirp_f = take((size_t)c.Nz * 8);
       L.bspec_f = take((size_t)M * 8);
     }
-  }
-  if (!mixed) {
-    const size_t pitch = (size_t)split_pitch_b16(c.Nr), Nc = 2 * (size_t)c.Nz, nmat = 6 * (size_t)c.Nm;
-    const size_t S = (size_t)f64s_digits(c), items = (size_t)f64s_items(c);
-    L.f64s_mat = take(nmat * S * c.Nr * pitch * 2);
-    L.f64s_rowexp = take(nmat * c.Nr * 4);
-    L.f64s_panel = take(items * S * Nc * pitch * 2);
-    L.f64s_colexp = take(items * Nc * 4);
   }
   if (mixed) {
     for (int b = 0; b < 2; ++b)
@@ -156,10 +153,21 @@ Layout make_layout(const pic_config& c) {
       L.binv_lo = take((size_t)c.Nm * 3 * c.Nr * split_pitch(c.Nr) * 4);
     }
   } else {
+    // the panels' digit planes live within one DHT, in the particle buffer that is not current (free
+    // outside the sort and the diagnostics) and, where that is too small, the gap between the two
+    const size_t Nc = 2 * (size_t)c.Nz, items = (size_t)f64s_items(c), planes = items * S * Nc * pitch16 * 2;
     for (int b = 0; b < 2; ++b) {
       for (int k = 0; k < 7; ++k) L.part[b][k] = take(cap * 8);
       L.pid[b] = take(cap * 4);
+      if (b == 0) {
+        L.f64s_panel[1] = L.part[0][0];
+        L.f64s_panel[0] = off;
+        const size_t spare = off - L.part[0][0];
+        if (planes > spare) take(planes - spare);
+      }
     }
+    L.f64s_rowexp = take(nmat * c.Nr * 4);
+    L.f64s_colexp = take(items * Nc * 4);
   }
   L.keys = take(cap * 4);
   L.perm = take(cap * 4);

@@ -55,8 +55,8 @@ struct Layout {
   // the chirp w_n (Nz), the chirp filter's spectrum (M), float copies
   size_t twm, twm_f, chirp, chirp_f, bspec, bspec_f;
   // FP64 form: the sliced tensor-core DHT (BF16 digit planes of the matrices and of the
-  // current panels, their row and column exponents)
-  size_t f64s_mat, f64s_rowexp, f64s_panel, f64s_colexp;
+  // current panels, by the current particle buffer, and their row and column exponents)
+  size_t f64s_mat, f64s_rowexp, f64s_panel[2], f64s_colexp;
   size_t total;
 };
 
@@ -129,7 +129,7 @@ struct Sim {
   struct alignas(64) TensorMapBytes {
     unsigned char b[128];
   } tmaps[2 * kMaxModes * 3][3];
-  TensorMapBytes f64s_maps[2];   // FP64 form: panel planes, matrix planes (sliced DHT)
+  TensorMapBytes f64s_maps[3];   // FP64 form: panel planes by current particle buffer, matrix planes
   WindowState win;
   double* diag_host = nullptr;   // pinned host copy of the diagnostics results (first use)
   // staged particle input (pic_stage_particles / pic_take_particles): a copy stream and
