@@ -615,7 +615,8 @@ def measure_scan(args, local, dist=None, rank=0, world=1):
         sims = list(ex.map(init, range(len(members))))
     init_s = time.perf_counter() - t0
     # tile sizes per member, one at a time so that the timings do not overlap
-    # each graph launch runs 2 cycles: sort on one of them (sort interval 2)
+    # each graph launch runs 2 cycles; with an interval of 2 they hold one sort and the graph ends with
+    # another, which brings the particle buffers back to where the next launch reads them
     for s in sims:
         s.set_sort_interval(min(args.sort_interval, 2))
     tunings = [s.autotune() for s in sims]

@@ -261,7 +261,8 @@ pic_status pic_step_timed(pic_sim* sim, int32_t n_steps, double* stage_ms);
  * into ONE CUDA graph: each simulation runs on its own stream (given at its pic_init; must
  * not be the default stream), forked from and joined back to origin_stream (a created
  * stream), so uneven simulations run concurrently.  cycles_per_launch must be even (the
- * particle double buffers return to their starting parity).  The handles must have been
+ * particle double buffers return to their starting parity; where a simulation's sort interval
+ * leaves an odd number of sorts in them, its part of the graph ends with one more).  The handles must have been
  * brought to their initial state (pic_init_fields) and must not be stepped through other
  * calls while the batch exists.  pic_batch_launch enqueues n graph launches on
  * origin_stream (asynchronous).  Errors: PIC_ERR_ARG, PIC_ERR_CUDA, PIC_ERR_OOM. */

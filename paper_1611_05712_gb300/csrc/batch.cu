@@ -5,9 +5,10 @@
 // The cycles of all simulations are captured once into a single CUDA graph: each
 // simulation keeps its own stream, forked from and joined back to the caller's origin
 // stream, so simulations of uneven size run concurrently and one graph launch advances
-// all of them with no per-kernel host work.  The particle double buffers flip once per
-// cycle, so a graph holds an even number of cycles and the buffers return to their
-// starting parity after every launch.
+// all of them with no per-kernel host work.  The particle double buffers flip with every
+// sort; a graph holds an even number of cycles, and where a sort interval leaves an odd number
+// of sorts in them the graph ends with one more, so that the buffers return to their starting
+// parity after every launch.
 #include <new>
 #include <vector>
 
@@ -76,7 +77,11 @@ extern "C" pic_status pic_batch_create(pic_sim* const* sims, int32_t n_sims, int
     if (ce != cudaSuccess) { batch_free(b); return cuda_status(ce, "cudaStreamSynchronize"); }
   }
   int64_t before = 0;
-  for (Sim* s : b->sims) before += s->launches;
+  std::vector<int32_t> cur;
+  for (Sim* s : b->sims) {
+    before += s->launches;
+    cur.push_back(s->cur);
+  }
   cudaError_t ce = cudaStreamBeginCapture(b->origin, cudaStreamCaptureModeThreadLocal);
   if (ce != cudaSuccess) { batch_free(b); return cuda_status(ce, "cudaStreamBeginCapture"); }
   pic_status st = PIC_OK;
@@ -86,6 +91,8 @@ extern "C" pic_status pic_batch_create(pic_sim* const* sims, int32_t n_sims, int
       st = cuda_status(ce, "cudaStreamWaitEvent");
   for (int k = 0; st == PIC_OK && k < b->cycles; ++k)
     for (size_t i = 0; st == PIC_OK && i < b->sims.size(); ++i) st = step_cycle(b->sims[i]);
+  for (size_t i = 0; st == PIC_OK && i < b->sims.size(); ++i)
+    if (b->sims[i]->cur != cur[i]) st = launch_sort(b->sims[i]);
   for (size_t i = 0; st == PIC_OK && i < b->sims.size(); ++i) {
     if ((ce = cudaEventRecord(b->events[i + 1], b->sims[i]->stream)) != cudaSuccess)
       st = cuda_status(ce, "cudaEventRecord");
@@ -95,6 +102,7 @@ extern "C" pic_status pic_batch_create(pic_sim* const* sims, int32_t n_sims, int
   cudaGraph_t g = nullptr;
   ce = cudaStreamEndCapture(b->origin, &g);
   b->graph = g;
+  for (size_t i = 0; i < b->sims.size(); ++i) b->sims[i]->cur = cur[i];   // also after a capture that failed
   if (st != PIC_OK) { batch_free(b); return st; }
   if (ce != cudaSuccess) { batch_free(b); return cuda_status(ce, "cudaStreamEndCapture"); }
   if ((ce = cudaGraphInstantiate(&b->exec, b->graph, 0)) != cudaSuccess) {
@@ -105,8 +113,6 @@ extern "C" pic_status pic_batch_create(pic_sim* const* sims, int32_t n_sims, int
   int64_t after = 0;
   for (Sim* s : b->sims) after += s->launches;
   b->kernels_per_launch = after - before;
-  // the capture ran the host side of every cycle: the particle buffers flipped an even
-  // number of times, so each handle's current buffer is unchanged
   *out = b;
   return PIC_OK;
 }
