@@ -34,8 +34,9 @@ __device__ __forceinline__ void warp_rank_cell(const int32_t* in, int32_t* out, 
 // Sorts the n distinct values in[0..n) ascending into out[0..n), using alt[0..n) as the
 // second buffer of the merge passes.  alt may be the same memory as in (in is fully read
 // before the first merge pass).  Called by every thread of the CTA, with sm holding
-// kCellChunk int32 of shared memory.  Ends with the CTA synchronised.
-__device__ __forceinline__ void cta_sort_cell(const int32_t* in, int32_t* out, int32_t* alt, int n,
+// kCellChunk int32 of shared memory.  Ends with the CTA synchronised; true if alt holds the sorted
+// values too.
+__device__ __forceinline__ bool cta_sort_cell(const int32_t* in, int32_t* out, int32_t* alt, int n,
                                               int32_t* sm) {
   const int tid = threadIdx.x, nt = blockDim.x;
   // phase 1: sorted runs of kCellChunk
@@ -60,7 +61,7 @@ __device__ __forceinline__ void cta_sort_cell(const int32_t* in, int32_t* out, i
     for (int i = tid; i < cnt; i += nt) out[b + i] = sm[i];
     __syncthreads();
   }
-  if (n <= kCellChunk) return;
+  if (n <= kCellChunk) return false;
   // phase 2: merge pairs of runs, ping-ponging between out and alt
   constexpr int E = 8;   // outputs per thread and step
   int32_t* src = out;
@@ -93,6 +94,7 @@ __device__ __forceinline__ void cta_sort_cell(const int32_t* in, int32_t* out, i
     for (int i = tid; i < n; i += nt) out[i] = src[i];
     __syncthreads();
   }
+  return src != out;
 }
 
 }  // namespace pic
