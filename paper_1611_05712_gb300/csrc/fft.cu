@@ -808,7 +808,7 @@ __device__ __forceinline__ void mixed_pass_r(int Rdx, const C2* src, C2* dst, co
 // COMP: room for the composite radices, which take more registers (64, four CTAs an SM); plans
 // without them are faster in the other instance.
 template <typename R, bool INV, bool COMP>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
+__global__ void __launch_bounds__(256, 4) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
                                                                 typename Vec2<R>::T* __restrict__ out,
                                                                 const typename Vec2<R>::T* __restrict__ twp,
                                                                 RowCombine rc, FftPlan plan, int rows_per_comp) {
