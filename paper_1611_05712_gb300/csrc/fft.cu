@@ -739,7 +739,7 @@ __device__ __forceinline__ void mixed_pass(const C2* __restrict__ src, C2* __res
                                            const C2* __restrict__ twp, const MixedIO<C2>& io, int N, int L) {
   const int NR = N / R;
   const float invL = 1.0f / (float)L;
-  const int step = COMP ? blockDim.x : 256;   // a constant keeps the plain radices in 48 registers
+  const int step = COMP ? blockDim.x : 256;   // plain plans run with 256 threads: a constant
   for (int t = threadIdx.x; t < NR; t += step) {
     // j = t / L, k = t mod L (t, L < 2^13: the float quotient is off by at most one)
     int j = (int)((float)t * invL);
@@ -805,8 +805,9 @@ __device__ __forceinline__ void mixed_pass_r(int Rdx, const C2* src, C2* dst, co
   }
 }
 
-// COMP: room for the composite radices, which take more registers (64, four CTAs an SM); plans
-// without them are faster in the other instance.
+// COMP: room for the composite radices, of which 14 to 16 spill up to 168 bytes at the 64 registers of four
+// CTAs an SM.  Plans without them take the other instance, which spills nothing: in this one their field
+// cycles take 0.98 to 1.15 (mean 1.04) times as long.
 template <typename R, bool INV, bool COMP>
 __global__ void __launch_bounds__(256, 4) k_fft_rows(const typename Vec2<R>::T* __restrict__ in,
                                                                 typename Vec2<R>::T* __restrict__ out,
@@ -909,11 +910,12 @@ struct RadixSearch {
 // many instructions for indices, twiddles and the exchange as for its butterflies), and among
 // those the smallest largest radix; the pass whose radix shares the smallest power of two with the
 // shared memory's 16 double banks comes first, since its stores step by the radix (odd radices meet no
-// bank conflicts).  A composite pass has fewer threads at work, which pays for short rows and where
-// the rows (4 Nm Nr in a forward transform) are twice as many as the SMs hold.  Field cycles of 70
-// lengths on 96 x 2 and 400 x 1 rows against radices up to 8 alone: 1.00 to 1.19 times as fast up to
-// 900 points, 0.98 to 1.08 (mean 1.03) beyond on the composite side of the line; on the other side
-// composites would take 0.90 to 1.17 (mean 0.98).
+// bank conflicts).  A composite pass has fewer threads at work, which pays where the rows (4 Nm Nr in a
+// forward transform) fill the SMs: up to 900 points from 600 rows on (four CTAs on 152 SMs are 608), beyond
+// where they are twice as many as the SMs hold.  Field cycles of 83 lengths, in time against radices up to 8
+// alone: up to 900 points 0.99 to 1.16 (mean 1.07) with up to 400 rows, 0.92 to 1.05 (0.99) with 600, 0.88
+// to 1.01 (0.95) with 768 and 800, 0.79 to 1.05 (0.89) with 1600 and 3600; beyond, 0.88 to 1.02 (0.95) with
+// 3600, 0.86 to 1.09 (0.98) with 768, 0.90 to 1.25 (1.05) with 48 to 400.
 bool plan_radix(int N, int precision, int64_t rows, int32_t* radix, int32_t* n_pass) {
   int n = N;
   for (int f : {2, 3, 5, 7})
@@ -922,7 +924,7 @@ bool plan_radix(int N, int precision, int64_t rows, int32_t* radix, int32_t* n_p
   int k = 0;
   n = N;
   const int64_t held = 152 * (int64_t)(227 * 1024 / (16 * N));   // rows on the SMs at once
-  const bool many = N <= 900 || rows >= 2 * held;
+  const bool many = N <= 900 ? rows >= 600 : rows >= 2 * held;
   if (precision == PIC_FP64 || (N & (N - 1)) == 0 || !many) {
     for (int f : {8, 4, 2, 3, 5, 7})
       while (n % f == 0) {
