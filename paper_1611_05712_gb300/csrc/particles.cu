@@ -832,8 +832,10 @@ __device__ __forceinline__ void deposit_one(const GridGeom& g, const DepArgs& a,
   deposit_at<MODES, RHO, CUR>(g, a, invV, r, c, s, z, w, vx, vy, vz);
 }
 
-template <int MODES, bool RHO, bool CUR>
-__global__ void __launch_bounds__(256, 3) k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a,
+// Bound by the L2's float64 atomics in large sets (200 to 240 G/s), by latency in small ones; CTAS on an
+// SM as chosen by deposit_kernel64.
+template <int MODES, bool RHO, bool CUR, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_deposit(const Parts p, int64_t np, GridGeom g, DepArgs a,
                                                     const double* invV, int32_t* err) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -2485,8 +2487,23 @@ __global__ void __launch_bounds__(kWinBlock) k_win_inject_f32(int32_t* flag, int
 bool is_mixed(const Sim* s) { return s->cfg.precision != PIC_FP64; }
 
 // Kernel instances of the FP64 form by the modes they have room for.
-template <int MODES> auto deposit_kernel64(const DepArgs& a) {
-  return !a.J ? k_deposit<MODES, true, false> : !a.rho ? k_deposit<MODES, false, true> : k_deposit<MODES, true, true>;
+// Deposits whose set one wave of three CTAs an SM (80 registers) does not hold: with three the few CTAs of the
+// second wave double the time.  Four (64 registers) beyond the point where they begin to win, 20 % above that
+// wave in 1 and 2 modes (J of 155 000 particles 43 -> 37 us), and 5 % above in 3 and 4, except that the
+// currents of those, which spill most, take two (128) as long as four would hold the set (J of
+// 130 000 in 3 modes 61 -> 53 us, 4 modes 81 -> 67) and rho and J in 4 modes two up to a second full wave (155 000: 107 ->
+// 95) and three beyond.
+template <int MODES, bool RHO, bool CUR> auto deposit_kernel64(int64_t np) {
+  constexpr int64_t wave = 152 * 3 * 256;
+  constexpr bool four = !(MODES == 4 && RHO && CUR);
+  if (MODES >= 3 ? 20 * np <= 21 * wave : 5 * np <= 6 * wave) return k_deposit<MODES, RHO, CUR, 3>;
+  if constexpr (MODES >= 3 && CUR)
+    if (four ? 3 * np <= 4 * wave : np <= 2 * wave) return k_deposit<MODES, RHO, CUR, 2>;
+  return k_deposit<MODES, RHO, CUR, four ? 4 : 3>;
+}
+template <int MODES> auto deposit_kernel64(const DepArgs& a, int64_t np) {
+  return !a.J ? deposit_kernel64<MODES, true, false>(np)
+              : !a.rho ? deposit_kernel64<MODES, false, true>(np) : deposit_kernel64<MODES, true, true>(np);
 }
 template <int MODES, int CTAS> auto push_kernel64(bool win, bool dwg) {
   return win ? (dwg ? k_gather_push<MODES, true, true, CTAS> : k_gather_push<MODES, true, false, CTAS>)
@@ -2665,7 +2682,8 @@ pic_status launch_deposit(Sim* s, int32_t what, int32_t id_lo, int32_t id_hi, vo
     if (a.J) PIC_CUDA(cudaMemsetAsync(a.J, 0, 3 * G * sizeof(double2), s->stream));
     if (s->np == 0) return PIC_OK;
     if (!a.rho && !a.J) return PIC_OK;
-    auto* kern = s->cfg.Nm <= 2 ? deposit_kernel64<2>(a) : s->cfg.Nm == 3 ? deposit_kernel64<3>(a) : deposit_kernel64<4>(a);
+    auto* kern = s->cfg.Nm <= 2 ? deposit_kernel64<2>(a, s->np)
+                                : s->cfg.Nm == 3 ? deposit_kernel64<3>(a, s->np) : deposit_kernel64<4>(a, s->np);
     kern<<<pgrid(s->np), 256, 0, s->stream>>>(parts_of(s, s->cur), s->np, geom_of(s), a, inv_volume(s), err);
   }
   PIC_LAUNCHED(s);
