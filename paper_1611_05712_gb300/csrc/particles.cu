@@ -878,11 +878,11 @@ __device__ __forceinline__ void win_mark(const WinArgs& wa, int32_t id, int64_t 
 // products are fused, and the stencils, the gather's weights and the deposits' products are formed
 // by the integer units (stencil62, Sf).  Momenta are read after the gather, requested into L2 before
 // it, and written before the deposits, and the gather goes node by node: the kernel needs more
-// registers than three CTAs per SM leave it (80; 236 to 408 bytes of its values go through local
-// memory), which still hides its latency better than two CTAs at 128.  1.35 M particles, two modes:
+// registers than three CTAs per SM leave it (80; it spills 184 to 464 bytes of stores and 252 to 696 of
+// loads, 228 and 288 in two modes), which still hides its latency better than two CTAs at 128.  1.35 M particles, two modes:
 // 846 us at first, 703 with the float64 unit's own work reduced, 593 with the integer products, 498
-// now (525 at 128 registers); 1.64 M particles, three modes: 959, 793, 746, 651 (664).  A set that
-// fits the SMs at once with 128 registers takes them (CTAS = 2): 36 000 particles 31.2 -> 28.1 us.
+// now (525 at 128 registers); 1.64 M particles, three modes: 959, 793, 746, 651 (664).  CTAS as
+// launch_gather_push chooses.
 template <int MODES, bool WIN, bool DWG, int CTAS>
 __global__ void __launch_bounds__(256, CTAS) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
                               const double2* __restrict__ B, const float4* __restrict__ EBdw, double k,
@@ -2755,7 +2755,12 @@ pic_status launch_gather_push(Sim* s, int32_t fuse_current, const WinArgs& wa, b
     const int threads = s->np < 152 * 1024 ? 128 : 256;
     const int grid = (int)((s->np + threads - 1) / threads);
     const bool win = wa.on != 0, dwg = ebdw != nullptr;
-    auto* kern = s->np <= 152 * 512 ? push_kernel64_nm<2>(c.Nm, win, dwg) : push_kernel64_nm<3>(c.Nm, win, dwg);
+    // two CTAs of 256 threads an SM at 128 registers where they take no more waves than three at 80: sets
+    // that one wave of two holds (36 000 particles 31.2 -> 28.1 us) and those that two of either take
+    // (140 000 in 2, 3 and 4 modes: 67.6 -> 64.9, 94.1 -> 90.5 and 134.8 -> 115.0 us)
+    const int64_t two = 152 * 512, three = 152 * 768;
+    auto* kern = (s->np + two - 1) / two <= (s->np + three - 1) / three ? push_kernel64_nm<2>(c.Nm, win, dwg)
+                                                                       : push_kernel64_nm<3>(c.Nm, win, dwg);
     kern<<<grid, threads, 0, s->stream>>>(p, s->np, g, E, B, ebdw, kq, c.dt, a, inv_volume(s), fuse_current, err, wa);
   }
   PIC_LAUNCHED(s);
