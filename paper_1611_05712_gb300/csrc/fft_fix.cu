@@ -14,13 +14,14 @@
 //     row's exponent counts it.  Sums are exact; a product is off by at most 2 units;
 //   * the last pass converts to float64 with one rounding.
 // The error stays near 2^-57 of the row's largest value, below the rounding of the twiddles
-// (float64 values) and of the results: measured against extended precision it is smaller than
-// that of the IEEE float64 passes at every length and shape of row in the tests.
+// (float64 values) and of the results: against extended precision the tests hold it, at every length
+// and shape of row, below 1.25 times that of the IEEE float64 passes or one rounding of the row's norm.
 // A 64-bit addition is two instructions and a complex product about 22 (12 wide multiply-adds of
 // 31-bit halves), against 11 and 54 for pairs of floats and, for float64, the time of 64 and 256.
 // Rows with an infinity or a NaN become NaN.
 // Bound by instruction issue (about half of the issue slots; the integer unit's 64 lanes a clock
-// are its busiest part).  Measured, forward + inverse rows of one cycle: 2048 points x 256 x 2
+// are its busiest part).  The power-of-two kernel spills 504 bytes of stores and 816 of loads a thread
+// at its 64 registers forward (two sources' eight values and their sums), 108 and 500 inverse.  Measured, forward + inverse rows of one cycle: 2048 points x 256 x 2
 // modes 126 + 204 us with float pairs -> 95 + 163 us; 1800 points x 400 x 2 modes 558 + 859 us in
 // IEEE float64 -> 200 + 300 us.
 //
@@ -518,12 +519,8 @@ __global__ void __launch_bounds__(T, 1024 / T) k_fft_fix_rows(const __grid_const
   row_max<false>(&top, m);
   __syncthreads();
   set_scale(io, top);
-  const int np = A.n_pass;
+  const int np = A.n_pass;   // two at least (the shortest length is 9 = 3 x 3)
   int R = (int)(A.radix & 15);
-  if (np == 1) {
-    mixed_pass_r<INV, true, true>(R, A, io, src, dst, 1, 0, out_of<INV>(A, io));
-    return;
-  }
   unsigned b = mixed_pass_r<INV, true, false>(R, A, io, src, src, 1, 0, OutScale{});
   int L = R;
   for (int p = 1;; ++p) {
