@@ -7,7 +7,9 @@ Workload (default): the 2048 x 256 grid, 2 azimuthal modes, stencil order 32, FP
 configuration.  A step is one full cycle: gather + push + current deposit, cell sort,
 charge deposit, z-FFT + DHT, PSATD update, inverse DHT + z-FFT.
 
-Prints ONE JSON line (rank 0).  Under torchrun each rank runs its own independent
+Prints ONE JSON line (rank 0) with the headline figures, a few kB at most; everything measured (the other
+forms in full, the large run, every member of the scan) goes to stderr before it and, with --record, to a
+file.  Under torchrun each rank runs its own independent
 simulation (weak scaling; no collective on the data path), and the time is the max
 over ranks.  ``--impl reference`` times the FP64 CPU oracle on the host cores instead.
 """
@@ -101,6 +103,7 @@ def parse():
     ap.add_argument("--sweep-steps", type=int, default=2000, help="cycles per order in the order sweep")
     ap.add_argument("--window-cycles", type=int, default=8192,
                     help="cycles of the moving-window propagation after the timed cycles")
+    ap.add_argument("--record", metavar="FILE", help="write everything measured to FILE as JSON")
     ap.add_argument("--profile-range", action="store_true",
                     help="bracket each timed region with cudaProfilerStart/Stop (for "
                          "ncu --profile-from-start off); no work is skipped")
@@ -122,6 +125,52 @@ def config_of(w, n, precision="fp64", sort_interval=None):
     if sort_interval is not None:
         c["sort_interval"] = sort_interval
     return c
+
+
+# ------------------------------------------------------------------------- output
+HEAD_KEYS = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "particle_updates_per_s", "stage_ms_per_step", "roofline", "e2e",
+             "gpu_launches", "graph_launches", "clocks", "cpu_baseline", "chosen_form")
+PART_KEYS = ("value", "unit", "ms_per_step", "dtype", "speedup_vs_fp64")
+LINE_BYTES = 4000   # a reader that keeps the last few kB of the output still has the whole line
+
+
+def rounded(x, digits=6):
+    """x with its floats rounded to that many significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}")
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    return [rounded(v, digits) for v in x] if isinstance(x, list) else x
+
+
+def short_line(record):
+    """The record's headline as one line of JSON below LINE_BYTES: the keys of the contract (the figures of
+    it as measured, the rest rounded), lists of more than 8 values by their length and range, and the
+    other runs by their throughput."""
+    line = {k: record[k] for k in HEAD_KEYS if k in record}
+    if isinstance(line.get("config"), dict):
+        line["config"] = {k: ({"n": len(v), "min": min(v), "max": max(v)} if isinstance(v, list) and len(v) > 8 else v)
+                          for k, v in line["config"].items()}
+    for k in ("mixed_form", "mixed_form_bf16", "large", "scan"):
+        if k in record:
+            line[k] = {q: record[k][q] for q in PART_KEYS if q in record[k]}
+            if "e2e" in record[k]:
+                line[k]["e2e"] = record[k]["e2e"]["value"]
+    line = {k: v if k in ("value", "ms_per_step", "e2e", "config", "cpu_baseline") else rounded(v) for k, v in line.items()}
+    for k in ("stage_ms_per_step", "chosen_form", "scan", "large", "mixed_form_bf16", "mixed_form"):
+        if len(json.dumps(line)) > LINE_BYTES:   # what is left out is in the record
+            line.pop(k, None)
+    return json.dumps(line)
+
+
+def emit(record, args):
+    full = json.dumps(record)
+    if getattr(args, "record", None):
+        with open(args.record, "w") as f:
+            f.write(full + "\n")
+    print("record: " + full, file=sys.stderr, flush=True)
+    print(short_line(record), flush=True)
 
 
 # ------------------------------------------------------------------------- clocks
@@ -263,7 +312,7 @@ def run_reference(args):
                          "sample": f"{args.steps} full cycles of the workload (numpy FP64 oracle)"},
         "e2e": {"value": v, "unit": "steps/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
     }
-    print(json.dumps(line), flush=True)
+    emit(line, args)
     return 0
 
 
@@ -582,7 +631,7 @@ def run_ours(args):
         if "scan" in line:
             line["scan"]["cpu_baseline"] = oracle_scan_baseline()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
@@ -682,7 +731,7 @@ def run_scan(args):
     torch.cuda.set_device(local)
     line = measure_scan(args, local, dist, rank, world)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
@@ -795,7 +844,7 @@ def run_large(args):
     torch.cuda.set_device(local)
     line = measure_large(args, local, dist, world, args.large_accuracy_cycles, crop=args.workload == "crop")
     if int(os.environ.get("RANK", "0")) == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, args)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
@@ -971,7 +1020,7 @@ def run_window(args):
                 "propagation_cycles": args.window_cycles,
                 "propagation_um": args.window_cycles * w.dz * 1e6})
     steps_win = args.steps / (ms_win * 1e-3)
-    print(json.dumps({
+    emit({
         "metric": "pic_steps_per_s_moving_window", "value": steps_win, "unit": "steps/s", "n_gpus": 1,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_win / args.steps,
         "ms_per_step_without_window": ms_plain / args.steps,
@@ -984,7 +1033,7 @@ def run_window(args):
                         "plasma_active_start": npl, "plasma_active_end": plasma_active,
                         "plasma_active_samples": {"columns": ["cycles", "active_plasma", "dropped"],
                                                   "rows": samples},
-                        "beams": beams_out}}), flush=True)
+                        "beams": beams_out}}, args)
     s.close()
     return 0
 
