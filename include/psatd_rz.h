@@ -385,15 +385,17 @@ pic_status pic_get_tuning(pic_sim* sim, pic_tuning* out);
  * Fourier transforms are the operations, this chooses how their float64 results are
  * computed).  The DHT path:
  *   PIC_DHT_AUTO        digit products on the tensor cores at every Nr (the default): six
- *                       digits up to Nr = 256 (as SLICED), eight beyond, whose results are the
- *                       exact sums rounded once, as accurate as the FP64 GEMM's;
+ *                       digits up to Nr = 256 (as SLICED), eight beyond, whose sums miss at
+ *                       most 2^-59 of (row max x column max x Nr) before one rounding: as
+ *                       accurate as the FP64 GEMM's;
  *   PIC_DHT_F64_GEMM    FP64 SIMT GEMM on the FP64 units, and the z-FFT rows in IEEE float64
  *                       too (the reference arithmetic for studies of rounding floors);
  *   PIC_DHT_F64_SLICED  every row of the matrix and column of the panel scaled by a power
  *                       of two and cut into six balanced base-256 digits (exact BF16
  *                       numbers); the digit products accumulate exactly in FP32 on the tensor
- *                       cores and are combined in FP64: agrees with the FP64 product to about
- *                       2^-49 of (row max x column max x Nr).  Needs Nr <= 256.
+ *                       cores and are combined in FP64: within 2^-46 of (row max x column max
+ *                       x Nr) of the product at worst, about 2^-50 of (row max x column max x
+ *                       sqrt Nr) where the digits' signs average.  Needs Nr <= 256.
  * With AUTO and SLICED the 7-smooth z-FFT rows run in 64-bit block fixed point (64-bit
  * integers with one exponent per row; rows stay float64 in memory and keep float64's range;
  * no further off than IEEE float64 rows, both measured against extended precision).  With

@@ -23,14 +23,18 @@
 // Two forms (F64sForm below):
 //   Nr <= 256: S = 6, T = 8, B = 48, 21 products.  The first digit reaches 256, so groups 2
 //     and 3 are split over two accumulators each to stay exact; groups 4 and 5 add at most an
-//     FP32 rounding at weight <= 2^-48.  Error about 2^-50 of max|A_n| max|X_c| sqrt(K) (on the
-//     Hankel matrices with random, beam-like, decaying and smooth panels 2 to 6 times smaller
-//     than the seven sign-magnitude 7-bit slices, 28 products, that stood here before);
+//     FP32 rounding at weight <= 2^-48.  At worst, with every digit left out of one sign, 2^-46 of
+//     max|A_n| max|X_c| K is missing (a term's five products of group 6 are up to 5 2^14 2^-64 =
+//     2^-47.7, its operands' rounding 2^-48); the signs average, and the error found is about
+//     2^-50 of max|A_n| max|X_c| sqrt(K) (on the Hankel matrices with random, beam-like, decaying and
+//     smooth panels 2 to 6 times smaller than the seven sign-magnitude 7-bit slices, 28 products,
+//     that stood here before);
 //   Nr > 256: S = 8, T = 6, B = 62, 36 products, the accumulators drained into integers every
-//     256 K: groups 0..3 exact, the rest exact unless sums align adversarially (then an FP32
-//     rounding at weight <= 2^-44).  All 53 bits of entries down to 2^-9 of the largest take
-//     part: the result is the exact sum rounded once to within 2^-62 of max|A_n| max|X_c| K, no
-//     further off than the float64 product's own accumulated roundings.
+//     256 K: groups 0..3 exact, the rest exact unless sums align adversarially (more than 2^24 units
+//     of one sign: then FP32 roundings at weight <= 2^-44).  All 53 bits of entries down to 2^-9 of the
+//     largest take part.  At worst 2^-59 of max|A_n| max|X_c| K is missing (a term's seven products of
+//     group 8, up to 7 2^14 2^-76 = 2^-59.2, and its operands' rounding, 2^-62), and the rest is
+//     rounded once: no further off than the float64 product's own accumulated roundings.
 // Measured, one cycle's 20 DHTs with their panels' digits: 2048 x 256 x 2 modes 0.45 -> 0.32 ms
 // against the seven-slice form; 1800 x 400 x 2 modes 21.1 ms on the FP64 SIMT GEMM -> 1.04 ms.
 //
@@ -320,9 +324,9 @@ __device__ __forceinline__ double scale_pow2(double t, int k) {
 
 // A tile's accumulators are drained in two steps: the group sums of a thread's 16 outputs are
 // combined into 64-bit integers and TMEM is released at once, so that the next tile's products
-// run while these warps convert to float64 (one instruction per output on the scarce float64
-// unit; three for S = 8) and store.  With the conversions before the release the products stood
-// still for 14 k of a tile's 35 k cycles.
+// run while these warps convert to float64 (on the integer units; S = 8 adds its two sums in one
+// float64 operation an output) and store.  With the conversions before the release the products
+// stood still for 14 k of a tile's 35 k cycles.
 template <int S>
 __global__ void __launch_bounds__(kF64sThreads, 1) k_dht_f64s(DhtBatch bt, F64sParams P,
                                                                const __grid_constant__ F64sMaps maps,

@@ -5,9 +5,10 @@
 // The FP64 form's 7-smooth rows run in block fixed point (fft_fix.cu) unless PIC_DHT_F64_GEMM
 // asks for IEEE float64.  Here: power-of-two lengths use radix-8 passes with the values in
 // registers (k_fft_pow2 for IEEE double rows; k_fft_pow2_tma for float rows, persistent and fed
-// by bulk copies); other 7-smooth lengths a mixed-radix (8, 4, 2, 3, 5, 7) self-sorting Stockham
-// sequence of passes between two shared row buffers (k_fft_rows).  All read per-pass twiddle
-// tables.  Any other length goes through Bluestein's chirp-z algorithm on power-of-two rows.
+// by bulk copies); other 7-smooth lengths a mixed-radix (8, 4, 2, 3, 5, 7, for float rows also
+// composite radices up to 16: plan_radix) self-sorting Stockham sequence of passes between two
+// shared row buffers (k_fft_rows).  All read per-pass twiddle tables.  Any other length goes
+// through Bluestein's chirp-z algorithm on power-of-two rows.
 // The component combination of the quasi-cylindrical scheme is fused into the row load:
 // out = ca * inA + cb * inB, which forms J_+- = (J_r -+ i J_theta)/2 before the forward
 // transform and E_r = E_+ + E_-, E_theta = i (E_+ - E_-) before the inverse one.

@@ -21,9 +21,9 @@
 // Rows with an infinity or a NaN become NaN.
 // Bound by instruction issue (about half of the issue slots; the integer unit's 64 lanes a clock
 // are its busiest part).  The power-of-two kernel spills 504 bytes of stores and 816 of loads a thread
-// at its 64 registers forward (two sources' eight values and their sums), 108 and 500 inverse.  Measured, forward + inverse rows of one cycle: 2048 points x 256 x 2
-// modes 126 + 204 us with float pairs -> 95 + 163 us; 1800 points x 400 x 2 modes 558 + 859 us in
-// IEEE float64 -> 200 + 300 us.
+// at its 64 registers forward (two sources' eight values and their sums), 108 and 500 inverse.
+// Measured, forward + inverse rows of one cycle: 2048 points x 256 x 2 modes 126 + 204 us with float
+// pairs -> 95 + 163 us; 1800 points x 400 x 2 modes 558 + 859 us in IEEE float64 -> 200 + 300 us.
 //
 // Radix-8 (4, 2, 3, 5, 7) self-sorting Stockham passes, butterflies in registers, the first
 // pass from global memory with the component combination (J_+- = (J_r -+ i J_theta)/2 before

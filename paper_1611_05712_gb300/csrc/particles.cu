@@ -2777,8 +2777,7 @@ pic_status launch_diag(Sim* s, int32_t lo, int32_t hi, pic_diag* out, double* sl
   return run_diag(s, a, lo, hi, out, slice_sigma, max_slices);
 }
 
-// Mixed form: float64 SoA (the staging area, or src with its stride) -> FP32 particles of
-// the current buffer.
+// A particle set's arrays as a kernel argument (null arrays are left out).
 static Soa64 soa_of(const double* const v[7], const int32_t* id) {
   Soa64 o;
   for (int k = 0; k < 7; ++k) o.v[k] = v ? const_cast<double*>(v[k]) : nullptr;
