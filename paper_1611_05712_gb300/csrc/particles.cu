@@ -759,6 +759,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     }
   }
   if (ends == 0u) qw = sf_from_end(a.q) * sf_from_end(w);
+  const bool special = ends == 0u || !is_finite(r);
   Sf rad[2];   // q w w_r / V_j of the radial nodes j0, j0 + 1 (kSfNone for the dropped node Nr)
   int jn[2];   // their grid rows (the ghost node j = -1 is row 0)
 #pragma unroll
@@ -767,8 +768,8 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
     const bool keep = j < g.Nr;
     jn[dj] = (j < 0 || !keep) ? 0 : j;
     rad[dj] = sf_normal(sf_fraction(keep ? (dj ? st.fr : kOne62 - st.fr) : 0ull) * (sf_from(invV[jn[dj]]) * qw));
-    if (!is_finite(r)) rad[dj].e = kSfNan;
-    if (!keep) rad[dj].e = kSfNone;
+    if (special && !is_finite(r)) rad[dj].e = kSfNan;
+    if (special && !keep) rad[dj].e = kSfNone;
   }
   Sf pr[MODES > 1 ? MODES - 1 : 1], pi[MODES > 1 ? MODES - 1 : 1];   // e^{+i m theta}, m = 1 ..
   {
@@ -788,7 +789,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
   for (int q = 0; q < 4; ++q) {
     const int node = (q + rot) & 3, dz = node >> 1, dj = node & 1;
     const Sf gq = (dj ? rad[1] : rad[0]) * (dz ? z1 : z0);
-    if ((gq.h | gq.l) == 0u && gq.e < kSfInf / 2) continue;
+    if ((gq.h | gq.l) == 0u && !(special && gq.e >= kSfInf / 2)) continue;
     const size_t o = (size_t)(dj ? jn[1] : jn[0]) * g.Nz + (dz ? st.i1 : st.i0);
     const unsigned fold = ghost && dj == 0 ? 0x80000000u : 0u;   // the ghost node: fold signs apply
     auto add = [&](double2* grid, size_t at, const Sf& f, unsigned flip) {   // mode 0
