@@ -744,7 +744,7 @@ __device__ void deposit_at(const GridGeom& g, const DepArgs& a, const double* in
   const bool ghost = st.j0 < 0;
   Sf v[3], qw = sf_from(a.q) * sf_from(w);   // velocity; charge
   // one test for all factors that may be no normal number: a conversion that handles every number took
-  // 1 to 2 % of the push, a call of float64 products up to 12 % of a deposit; this costs nothing
+  // 1 to 2 % of the push, a call of float64 products up to 12 % of a deposit; this takes up to 1 %
   unsigned ends = min(sf_end(a.q), sf_end(w));
   if (CUR) {
     const double vr = c * vx + s * vy, vt = c * vy - s * vx;
@@ -2488,16 +2488,18 @@ __global__ void __launch_bounds__(kWinBlock) k_win_inject_f32(int32_t* flag, int
 bool is_mixed(const Sim* s) { return s->cfg.precision != PIC_FP64; }
 
 // Kernel instances of the FP64 form by the modes they have room for.
-// Deposits whose set one wave of three CTAs an SM (80 registers) does not hold: with three the few CTAs of the
-// second wave double the time.  Four (64 registers) beyond the point where they begin to win, 20 % above that
-// wave in 1 and 2 modes (J of 155 000 particles 43 -> 37 us), and 5 % above in 3 and 4, except that the
-// currents of those, which spill most, take two (128) as long as four would hold the set (J of
-// 130 000 in 3 modes 61 -> 53 us, 4 modes 81 -> 67) and rho and J in 4 modes two up to a second full wave (155 000: 107 ->
-// 95) and three beyond.
+// Deposits take three CTAs an SM (80 registers) up to the sets that one wave of those holds and a little
+// beyond: then the few CTAs of a second wave double the time, and four (64) win, from 20 % above the wave in 1 and
+// 2 modes (J of 155 000 particles 43 -> 37 us), from 5 % above in 3 and 4.  Except: the currents of 3 and 4 modes, which spill
+// most, take two (128) as long as four would hold the set (J of 130 000 in 3 modes 61 -> 53 us, in 4
+// 81 -> 67), rho and J in 4 modes two up to a second full wave (155 000: 107 -> 95) and three beyond; and three beyond 2^21
+// particles, whose grids outgrow L2 (J of 25 M in 2 and 3 modes 3.36 and 5.48 ms, with four 3.47 and 5.67),
+// but for rho in 1 and 2 modes (0.90 ms, with four 0.79).
 template <int MODES, bool RHO, bool CUR> auto deposit_kernel64(int64_t np) {
   constexpr int64_t wave = 152 * 3 * 256;
   constexpr bool four = !(MODES == 4 && RHO && CUR);
   if (MODES >= 3 ? 20 * np <= 21 * wave : 5 * np <= 6 * wave) return k_deposit<MODES, RHO, CUR, 3>;
+  if (np > (1 << 21) && (CUR || MODES >= 3)) return k_deposit<MODES, RHO, CUR, 3>;
   if constexpr (MODES >= 3 && CUR)
     if (four ? 3 * np <= 4 * wave : np <= 2 * wave) return k_deposit<MODES, RHO, CUR, 2>;
   return k_deposit<MODES, RHO, CUR, four ? 4 : 3>;
