@@ -254,7 +254,9 @@ __device__ __forceinline__ Sf operator*(const Sf& a, const Sf& b) {
 __device__ __forceinline__ double sf_far(unsigned long long m, int e, unsigned s) {
   unsigned long long r;
   if (e > 12) {
-    r = e > kSfNan / 2 || (e > kSfInf / 2 && m == 0ull) ? 0x7ff8000000000000ull : m == 0ull ? 0ull : 0x7ff0000000000000ull;
+    r = e > kSfNan / 2 || (e > kSfInf / 2 && m == 0ull) ? 0x7ff8000000000000ull
+        : m == 0ull                                      ? 0ull
+                                                         : 0x7ff0000000000000ull;
   } else {   // m 2^(e - 10) units of the subnormal numbers
     const int sh = 10 - e;
     r = sh < 64 && sh > 0 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
@@ -930,11 +932,11 @@ __device__ __forceinline__ void win_mark(const WinArgs& wa, int32_t id, int64_t 
 // products are fused, and the stencils, the gather's weights and the deposits' products are formed
 // by the integer units (stencil62, Sf).  Momenta are read after the gather, requested into L2 before
 // it, and written before the deposits, and the gather goes node by node: the kernel needs more
-// registers than three CTAs per SM leave it (80; it spills 184 to 464 bytes of stores and 252 to 696 of
-// loads, 228 and 288 in two modes), which still hides its latency better than two CTAs at 128.  1.35 M particles, two modes:
-// 846 us at first, 703 with the float64 unit's own work reduced, 593 with the integer products, 498
-// now (525 at 128 registers); 1.64 M particles, three modes: 959, 793, 746, 651 (664).  CTAS as
-// launch_gather_push chooses.
+// registers than three CTAs per SM leave it (80; it spills 160 to 456 bytes of stores and 228 to 692
+// of loads, 204 and 268 in two modes), which still hides its latency better than two CTAs at 128.
+// 1.35 M particles, two modes: 846 us at first, 703 with the float64 unit's own work reduced, 593 with
+// the integer products, 498 now (525 at 128 registers); 1.64 M particles, three modes: 959, 793, 746, 642
+// (664).  CTAS as launch_gather_push chooses.
 template <int MODES, bool WIN, bool DWG, int CTAS>
 __global__ void __launch_bounds__(256, CTAS) k_gather_push(Parts p, int64_t np, GridGeom g, const double2* __restrict__ E,
                               const double2* __restrict__ B, const float4* __restrict__ EBdw, double k,
@@ -1588,7 +1590,8 @@ __global__ void k_keys_f32(const PartsF p, int64_t np, GeomF g, int32_t* keys, i
 // dst[at] = src[e] in the sorted order (sorted_place) for the 13 arrays.
 template <bool WIN>
 __global__ void k_permute_f32(const PartsF src, PartsF dst, const Sorted so, int64_t np, int32_t* slot) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; (i & ~31ll) < np; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; (i & ~31ll) < np;
+       i += (int64_t)gridDim.x * blockDim.x) {
     const bool ok = i < np;
     const int32_t k = so.tmp[ok ? i : np - 1];
     // in flight while the place is found
@@ -2542,13 +2545,14 @@ __global__ void __launch_bounds__(kWinBlock) k_win_inject_f32(int32_t* flag, int
 bool is_mixed(const Sim* s) { return s->cfg.precision != PIC_FP64; }
 
 // Kernel instances of the FP64 form by the modes they have room for.
-// Deposits take three CTAs an SM (80 registers) up to the sets that one wave of those holds and a little
-// beyond: then the few CTAs of a second wave double the time, and four (64) win, from 20 % above the wave in 1 and
-// 2 modes (J of 155 000 particles 43 -> 37 us), from 5 % above in 3 and 4.  Except: the currents of 3 and 4 modes, which spill
-// most, take two (128) as long as four would hold the set (J of 130 000 in 3 modes 61 -> 53 us, in 4
-// 81 -> 67), rho and J in 4 modes two up to a second full wave (155 000: 107 -> 95) and three beyond; and three beyond 2^21
-// particles, whose grids outgrow L2 (J of 25 M in 2 and 3 modes 3.36 and 5.48 ms, with four 3.47 and 5.67),
-// but for rho in 1 and 2 modes (0.90 ms, with four 0.79).
+// Deposits take three CTAs an SM (80 registers) up to the sets that one wave of those holds and a
+// little beyond.  From 20 % above that wave in 1 and 2 modes (J of 155 000 particles 43 -> 37 us), and 5 %
+// above it in 3 and 4, the few CTAs of a second wave would double the time, and four (64 registers) win.
+// Exceptions: the currents of 3 and 4 modes, which spill most, take two (128) as long as four would hold
+// the set (J of 130 000 in 3 modes 61 -> 53 us, in 4 81 -> 67); rho and J in 4 modes two up to a second
+// full wave (155 000: 107 -> 95) and three beyond; sets of more than 2^21, whose grids outgrow L2, three (J
+// of 25 M in 2 and 3 modes 3.36 and 5.48 ms, with four 3.47 and 5.67), but for rho in 1 and 2 modes (0.90
+// ms, with four 0.79).
 template <int MODES, bool RHO, bool CUR> auto deposit_kernel64(int64_t np) {
   constexpr int64_t wave = 152 * 3 * 256;
   constexpr bool four = !(MODES == 4 && RHO && CUR);
@@ -2676,8 +2680,8 @@ pic_status launch_sort(Sim* s) {
   const int nblk = (nbin + kScanBlock - 1) / kScanBlock;
   k_scan_local<<<nblk, kScanThreads, 0, s->stream>>>(count, start, blk, nbin, big_count);
   PIC_LAUNCHED(s);
-  k_scan_add<<<(nbin + kScanBlock / 4 - 1) / (kScanBlock / 4), 256, 0, s->stream>>>(count, start, blk, nbin, ncell, big_list,
-                                                                                   big_count, cell_of);
+  k_scan_add<<<(nbin + kScanBlock / 4 - 1) / (kScanBlock / 4), 256, 0, s->stream>>>(count, start, blk, nbin, ncell,
+                                                                                     big_list, big_count, cell_of);
   PIC_LAUNCHED(s);
   k_scatter<<<pgrid(np), 256, 0, s->stream>>>(keys, perm, start, np, tmp);
   PIC_LAUNCHED(s);
