@@ -1587,8 +1587,8 @@ __global__ void k_keys_f32(const PartsF p, int64_t np, GeomF g, int32_t* keys, i
   }
 }
 
-// dst[at] = src[e] in the sorted order (sorted_place) for the 13 arrays.
-template <bool WIN>
+// dst[at] = src[e] in the sorted order (SEARCH: sorted_place_warp, else sorted_place) for the 13 arrays.
+template <bool WIN, bool SEARCH>
 __global__ void k_permute_f32(const PartsF src, PartsF dst, const Sorted so, int64_t np, int32_t* slot) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; (i & ~31ll) < np;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -1599,7 +1599,8 @@ __global__ void k_permute_f32(const PartsF src, PartsF dst, const Sorted so, int
     const float fz = src.fz[k], fx = src.fx[k], fy = src.fy[k], ux = src.ux[k], uy = src.uy[k], uz = src.uz[k],
                 uxl = src.uxl[k], uyl = src.uyl[k], uzl = src.uzl[k], w = src.w[k];
     asm volatile("" ::: "memory");   // the loads are issued before the search, not after it
-    const int32_t at = sorted_place_warp(so, (int32_t)i, k, ok);
+    if (!SEARCH && !ok) return;
+    const int32_t at = SEARCH ? sorted_place_warp(so, (int32_t)i, k, ok) : sorted_place(so, (int32_t)i, k);
     if (!ok) return;
     dst.iz[at] = iz; dst.fz[at] = fz; dst.ixy[at] = ixy; dst.fx[at] = fx; dst.fy[at] = fy;
     dst.ux[at] = ux; dst.uy[at] = uy; dst.uz[at] = uz;
@@ -2662,8 +2663,9 @@ pic_status launch_sort(Sim* s) {
   if (np == 0) return PIC_OK;
   const bool win = slot != nullptr;
   // perm holds the particles' places within their keys until the scatter has read them; the staging area
-  // (mixed forms) is free between calls
-  int32_t* cell_of = is_mixed(s) ? s->at<int32_t>(s->lay.stage64) : nullptr;
+  // (mixed forms) is free between calls.  Below 1.5 M particles the keys come from L2 and the search for the
+  // cells costs 1 us more than it saves in sets that are nearly in order (1.35 M: 24 and 25 us)
+  int32_t* cell_of = is_mixed(s) && np >= 3 << 19 ? s->at<int32_t>(s->lay.stage64) : nullptr;
   if (is_mixed(s)) {
     if (win)
       k_keys_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), np, geomf_of(s), keys, count, perm, err);
@@ -2688,14 +2690,11 @@ pic_status launch_sort(Sim* s) {
   k_cell_sort_big<<<152 * 4, 256, 0, s->stream>>>(start, tmp, perm, big_list, big_count, cell_of);
   PIC_LAUNCHED(s);
   const Sorted so{keys, start, tmp, perm, ncell, cell_of};
-  if (is_mixed(s))
-    if (win)
-      k_permute_f32<true><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), so, np,
-                                                            slot);
-    else
-      k_permute_f32<false><<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), so, np,
-                                                             slot);
-  else if (win)
+  if (is_mixed(s)) {
+    auto* k = cell_of ? (win ? k_permute_f32<true, true> : k_permute_f32<false, true>)
+                      : (win ? k_permute_f32<true, false> : k_permute_f32<false, false>);
+    k<<<pgrid(np), 256, 0, s->stream>>>(partsf_of(s, s->cur), partsf_of(s, 1 - s->cur), so, np, slot);
+  } else if (win)
     k_permute<true><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), so, np, slot);
   else
     k_permute<false><<<pgrid(np), 256, 0, s->stream>>>(parts_of(s, s->cur), parts_of(s, 1 - s->cur), so, np, slot);

@@ -1,6 +1,7 @@
-"""The mixed form's sort finds the cells of 32 places at a time from the cells' ends: particles a fixed number of cells
-apart (one to beyond the 128 cells that are searched), cells that end with the 32 places and around them, few
-particles, and inactive ones behind them (moving window), bit for bit."""
+"""The mixed form's sort, whose permutation finds the cells of 32 places at a time from the cells' ends in sets of 1.5 M
+particles and more: particles a fixed number of cells apart (one to beyond the 128 cells that are searched), cells
+that end with the 32 places and around them, and inactive particles behind them (moving window), bit for bit; the
+same in small sets, which go by the keys."""
 import numpy as np
 import pytest
 
@@ -56,3 +57,21 @@ def test_gaps(gap, n):
 def test_cells_around_the_places(counts, window):
     key = np.repeat(np.arange(len(counts)) * 3, counts)
     _check(16, 16, key, window)
+
+
+@pytest.mark.parametrize("n", [(3 << 19) - 1, 3 << 19, (3 << 19) + 1, (3 << 19) + 77777])
+@pytest.mark.parametrize("window", [False, True])
+def test_sets_that_are_searched(n, window):
+    Nz, Nr = 2048, 512   # 1 M cells
+    parts, at = [], 7
+    for counts in ((32, 32, 32), (31, 1, 32, 33), (64, 0, 0, 63, 1), (128, 129, 127), (1, 2000, 31, 96), (5, 130, 0, 27, 3, 95)):
+        parts.append(np.repeat(at + np.arange(len(counts)), counts))
+        at += len(counts) + 300
+    for gap in (2, 3, 16, 31, 32, 33, 63, 127, 128, 129, 500):
+        parts.append(at + gap * np.arange(400))
+        at += gap * 400
+    left = n - sum(len(p) for p in parts)
+    cells = Nz * Nr - at - 100000   # the rest at 3 a cell, the last 100000 cells empty but for two
+    parts.append(at + np.arange(left - 2) % cells)
+    parts.append(np.array([Nz * Nr - 50000, Nz * Nr - 1]))
+    _check(Nz, Nr, np.concatenate(parts), window)
